@@ -70,7 +70,10 @@ typedef struct {
                              from there); execution only, it does not change the
                              result                                                */
     uint32_t warps_per_cta; /* 1..8; 0 = 4 for 128-row tiles from L = 65536, else 8;
-                             execution only                                        */
+                             execution only. With run and warps_per_cta both 0,
+                             lattices of 128 x 128 tiles and 4 x 4 cells up to
+                             L = 4096 (tile sets: L = 8192) run all sweeps of a
+                             kpz_run call in one launch instead of one each      */
     void* stream;         /* cudaStream_t to queue work on (NULL = default stream)  */
     void* dev_buf;        /* optional caller-owned device memory for the lattice and
                              its scratch; at least kpz_device_bytes(L) bytes,
@@ -147,7 +150,8 @@ kpz_status kpz_init(kpz_ctx** out, uint32_t L, double p, double q, uint64_t seed
 kpz_status kpz_reset(kpz_ctx* ctx);
 
 /* Queue n_mcs sweeps (n_mcs * L*L attempts) on the context's stream and
- * return; errors of the queued work surface at the next synchronising call. */
+ * return; errors of the queued work surface at the next synchronising call
+ * (KPZ_ETIMEOUT if a device-side barrier of a one-launch run gave up).      */
 kpz_status kpz_run(kpz_ctx* ctx, uint64_t n_mcs);
 
 /* Exact height sums and W^2 at the current time (eq. Wdef, Sec. 2.1).

@@ -11,6 +11,7 @@
 
 #include "kpz.h"
 #include "kpz_internal.h"
+#include "kpz_resident.h"
 #include "kpz_rsu.h"
 
 using namespace kpz;
@@ -42,6 +43,9 @@ struct kpz_ctx {
   unsigned long long* acc = nullptr;   // S1, S2 lo, S2 hi
   uint32_t* hcar = nullptr;            // import: height of (0, j0) modulo 4
   uint32_t* queue = nullptr;           // sweep work queue (zero between launches)
+  ResidentSync* sync = nullptr;        // resident kernels: grid barrier and error flag
+  uint32_t resident = 0;               // kpz_run's resident kernel (resident_kind), 0: one launch per sweep
+  bool unchecked = false;              // resident launches since the error flag was read
   int32_t* col0 = nullptr;             // h(0,j)
   void* io = nullptr;                  // staging band for host transfers
   size_t io_bytes = 0;
@@ -78,7 +82,7 @@ Layout layout(uint32_t L) {
   Layout y{};
   const size_t lat_bytes = (size_t)L * L / 8;   // 1 bit per site
   y.lat = 0;
-  y.small = align_up(lat_bytes);                 // t, h00, acc[3], hcar, queue
+  y.small = align_up(lat_bytes);                 // t, h00, acc[3], hcar, queue; at +128 ResidentSync
   y.col0 = y.small + kAlign;
   y.io = y.col0 + align_up((size_t)L * 4);
   const size_t io_bytes = std::min(kIoMax, (size_t)L * L / 4);
@@ -141,6 +145,17 @@ cudaError_t io_prepare(kpz_ctx* c) {
 uint32_t io_band_rows(const kpz_ctx* c, size_t row_bytes, size_t* half) {
   *half = (c->io_bytes / 2) / kAlign * kAlign;
   return (uint32_t)std::min<size_t>(c->g.L, *half / row_bytes) & ~3u;
+}
+
+// Reads the resident kernels' error flag if launches are outstanding; for
+// calls that synchronise and do not read the block of small values anyway.
+kpz_status settle(kpz_ctx* ctx) {
+  if (!ctx->unchecked) return KPZ_OK;
+  uint32_t err = 0;
+  KPZ_CUDA(cudaMemcpyAsync(&err, &ctx->sync->err, sizeof(err), cudaMemcpyDeviceToHost, ctx->stream));
+  KPZ_CUDA(cudaStreamSynchronize(ctx->stream));
+  ctx->unchecked = false;
+  return err ? fail(ctx, KPZ_ETIMEOUT, "a grid barrier of kpz_run timed out") : KPZ_OK;
 }
 
 SweepParams sweep_params(const kpz_ctx* c) {
@@ -276,9 +291,15 @@ kpz_status kpz_init(kpz_ctx** out, uint32_t L, double p, double q, uint64_t seed
   ctx->acc = (unsigned long long*)(base + y.small + 16);
   ctx->hcar = (uint32_t*)(base + y.small + 40);
   ctx->queue = (uint32_t*)(base + y.small + 48);
+  ctx->sync = (ResidentSync*)(base + y.small + 128);
   ctx->col0 = (int32_t*)(base + y.col0);
   ctx->io = base + y.io;
   ctx->io_bytes = y.total - y.io;
+
+  // Execution knobs select the work-queue sweep; without them lattices that
+  // would leave most of the GPU idle sweep with the resident kernels.
+  if (o.run == 0 && o.warps_per_cta == 0 && ctx->decomposition <= 1u)
+    ctx->resident = resident_kind(sweep_params(ctx), ctx->decomposition == 1u);
 
   kpz_status st = KPZ_OK;
   cudaError_t e = cudaMemsetAsync(base + y.small, 0, kAlign, ctx->stream);
@@ -304,7 +325,15 @@ kpz_status kpz_run(kpz_ctx* ctx, uint64_t n_mcs) {
   if (st) return st;
   SweepParams P = sweep_params(ctx);
   while (n_mcs > 0) {
-    const uint32_t chunk = (uint32_t)std::min<uint64_t>(n_mcs, 1u << 20);
+    // A resident launch takes 65536 sweeps at most (0.15 to 1.4 s).
+    const uint32_t chunk = (uint32_t)std::min<uint64_t>(n_mcs, ctx->resident ? 1u << 16 : 1u << 20);
+    if (ctx->resident) {
+      ctx->unchecked = true;
+      KPZ_CUDA(launch_resident(P, ctx->decomposition == 1u, ctx->resident, chunk, (uint32_t*)ctx->io, ctx->sync, ctx->stream));
+      ctx->t_host += chunk;
+      n_mcs -= chunk;
+      continue;
+    }
     for (uint32_t i = 0; i < chunk; ++i) {
       P.s_add = i;
       if (ctx->decomposition == 1u)      KPZ_CUDA(launch_sweep_tilesets(P, ctx->stream));
@@ -325,12 +354,17 @@ kpz_status kpz_roughness(kpz_ctx* ctx, kpz_rough* out) {
   if (st) return st;
   if (!out) return fail(ctx, KPZ_EINVAL, "null output");
   KPZ_CUDA(launch_roughness(ctx->lat, ctx->g, ctx->col0, ctx->acc, ctx->stream));
-  unsigned long long host[4];
-  KPZ_CUDA(cudaMemcpyAsync(host, ctx->acc, 3 * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
-                           ctx->stream));
-  KPZ_CUDA(cudaMemcpyAsync(host + 3, ctx->h00, sizeof(unsigned long long), cudaMemcpyDeviceToHost,
-                           ctx->stream));
+  // One copy of the block of small values: h00, S1, S2 lo, S2 hi, error flag.
+  unsigned char small[kAlign];
+  KPZ_CUDA(cudaMemcpyAsync(small, ctx->t_dev, sizeof(small), cudaMemcpyDeviceToHost, ctx->stream));
   KPZ_CUDA(cudaStreamSynchronize(ctx->stream));
+  unsigned long long host[4];
+  memcpy(host, small + 16, 3 * sizeof(host[0]));
+  memcpy(host + 3, small + 8, sizeof(host[0]));
+  ResidentSync rs;
+  memcpy(&rs, small + 128, sizeof(rs));
+  ctx->unchecked = false;
+  if (rs.err) return fail(ctx, KPZ_ETIMEOUT, "a grid barrier of kpz_run timed out");
   const uint64_t N = (uint64_t)ctx->g.L * ctx->g.L;
   out->t_mcs = ctx->t_host;
   out->n_sites = N;
@@ -360,7 +394,7 @@ kpz_status kpz_heights(kpz_ctx* ctx, int64_t* host_out, int absolute) {
                              cudaMemcpyDeviceToHost, ctx->stream));
     KPZ_CUDA(cudaStreamSynchronize(ctx->stream));
   }
-  return KPZ_OK;
+  return settle(ctx);
 }
 
 kpz_status kpz_slopes(kpz_ctx* ctx, uint32_t* host_out) {
@@ -385,7 +419,7 @@ kpz_status kpz_slopes(kpz_ctx* ctx, uint32_t* host_out) {
     KPZ_CUDA(cudaEventRecord(ctx->io_ev[2 + k], ctx->io_stream));
   }
   KPZ_CUDA(cudaStreamSynchronize(ctx->io_stream));
-  return KPZ_OK;
+  return settle(ctx);
 }
 
 kpz_status kpz_set_slopes(kpz_ctx* ctx, const uint32_t* host_in, int64_t h00, uint64_t t_mcs) {
@@ -418,7 +452,7 @@ kpz_status kpz_set_slopes(kpz_ctx* ctx, const uint32_t* host_in, int64_t h00, ui
   KPZ_CUDA(cudaMemcpyAsync(ctx->t_dev, small, sizeof(small), cudaMemcpyHostToDevice, ctx->stream));
   KPZ_CUDA(cudaStreamSynchronize(ctx->stream));
   ctx->t_host = t_mcs;
-  return KPZ_OK;
+  return settle(ctx);
 }
 
 namespace {
@@ -459,6 +493,7 @@ kpz_status kpz_ckpt_save(kpz_ctx* ctx, const char* path) {
   kpz_status st = enter(ctx);
   if (st) return st;
   if (!path) return fail(ctx, KPZ_EINVAL, "null path");
+  if ((st = settle(ctx)) != KPZ_OK) return st;
   const uint32_t L = ctx->g.L;
   CkptHeader hd{};
   memcpy(hd.magic, kCkptMagic, 8);

@@ -1,0 +1,787 @@
+// kpz_resident.cu -- many sweeps of one small or medium lattice in one launch
+// (arXiv:1204.5072, Sec. 3 and 3.1; same dynamics and random streams as
+// kpz_sweep.cu and kpz_tileset.cu, bit for bit).
+//
+// What bounds these sizes is latency, not work: at L = 4096 a sweep has 1024
+// tiles for 608 warp schedulers, at L = 256 four. So every tile of a step has
+// a warp of its own, and the chain a sweep cannot avoid -- window in, 16
+// dependent rounds, changes out, everybody done -- is stripped of everything
+// else:
+//   - one launch runs all sweeps of a kpz_run call; a barrier of the cluster
+//     (L <= 1024, lattice in distributed shared memory) or of the grid
+//     separates them instead of a launch;
+//   - the random numbers do not depend on the surface, so the Philox blocks of
+//     the next step are drawn into shared memory by warps of their own or
+//     while the barrier is pending, and a round only reads them;
+//   - between sweeps the lattice is held in the frame of the last sweep's
+//     origin: word (K, p, R) of the layout in kpz_common.cuh then belongs to
+//     tile (K, R / 32) alone, so a tile goes back with 16 plain stores (with a
+//     fixed frame every word is shared by two tiles and goes back as a
+//     read-modify-write; red.xor took 45 cycles each, 1400 to 2400 a tile).
+//     Two scratch lattices take turns; the last step writes the fixed frame.
+// Microseconds per sweep, p = 1 / p = 0.95, against one launch per sweep with
+// runs of 8 tiles (and of one tile, the fastest there): L = 256 2.1 / 3.3
+// against 12.4 / 22.8 (10.2 / 15.9), L = 1024 2.7 / 4.6 against 25 / 63 (10.2 /
+// 17.7), L = 4096 3.8 / 7.9 against 29 / 80 (14.1 / 25.8); tile sets at
+// L = 2048 13.8 / 19.3 against 44 at p = 1. At L = 512 (one tile a block, one
+// tile warp a scheduler) the 16 rounds take 2000 / 4300 cycles of a sweep's
+// 4400 / 7000; the rest is the window's trip and the barrier. At L = 4096 and
+// general rates the eight tiles of an SM bind it (logic and Philox pipes).
+#include <algorithm>
+
+#include "kpz_resident.h"
+#include "kpz_rounds.cuh"
+#include "kpz_tilemem.cuh"
+
+namespace kpz {
+namespace {
+
+using rounds::TileCtx;
+using tilemem::QuadTab;
+using tilemem::TileMem;
+
+// Random numbers of one tile and sweep, lane = cell row: position blocks of
+// the eight round pairs and, at general rates, the acceptance block of each
+// round and the outcome of its four deep numbers against both thresholds: bit
+// 7 - r % 8 of byte k of deep[r / 8].x (.y) is set when the k-th tie of the row
+// in round r is accepted as a minimum (maximum) (streams as in
+// kpz_rounds.cuh). setw[0]: the quadrant sets, [1], [2]: the sweep's origin.
+template <bool kGeneral>
+struct TileRand {
+  uint4 pos[kRounds / 2][32];
+  uint4 acc[kGeneral ? kRounds : 1][kGeneral ? 32 : 1];
+  uint2 deep[kGeneral ? 2 : 1][kGeneral ? 32 : 1];
+  uint32_t setw[4];
+};
+
+// Four Philox blocks (counter words c0[i], c1, c2, c3) at once: ten rounds of
+// one block are a serial chain, four chains keep the multiplier busy.
+__device__ __forceinline__ void philox4(const uint32_t (&ctr)[4], uint32_t c1, uint32_t c2, uint32_t c3, uint32_t k0,
+                                        uint32_t k1, uint4 (&out)[4]) {
+  uint32_t x[4], y[4], z[4], w[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) { x[i] = ctr[i]; y[i] = c1; z[i] = c2; w[i] = c3; }
+#pragma unroll
+  for (int r = 0; r < kPhiloxRounds; ++r) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t hiA = __umulhi(kPhiloxMulA, x[i]), loA = kPhiloxMulA * x[i];
+      const uint32_t hiB = __umulhi(kPhiloxMulB, z[i]), loB = kPhiloxMulB * z[i];
+      x[i] = hiB ^ y[i] ^ k0;
+      z[i] = hiA ^ w[i] ^ k1;
+      y[i] = loB;
+      w[i] = loA;
+    }
+    k0 += kPhiloxWeylA;
+    k1 += kPhiloxWeylB;
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) out[i] = make_uint4(x[i], y[i], z[i], w[i]);
+}
+
+// Four 12-bit numbers (the 16-bit halves of lo, hi) against a threshold t:
+// t + 0x7FFF - h has its top bit set exactly when h < t.
+__device__ __forceinline__ uint32_t deep_below(uint32_t lo, uint32_t hi, uint32_t t) {
+  const uint32_t c = ((t & 0xFFFu) + 0x7FFFu) * 0x10001u;
+  return __byte_perm(c - (lo & 0x0FFF0FFFu), c - (hi & 0x0FFF0FFFu), 0x7531) & 0x80808080u;
+}
+
+// Draws part `part` of `parts` (1 or 2) of a tile's blocks.
+template <bool kGeneral>
+__device__ __forceinline__ void draw_tile(const SweepParams& P, TileRand<kGeneral>& B, uint32_t tid, uint32_t s,
+                                          uint32_t lane, uint32_t part, uint32_t parts) {
+  if (part == 0u) {
+    const uint32_t w = philox(kTagSet << 28, tid, s, P.sample, P.k0, P.k1).x;
+    const uint4 o = philox(kTagOrigin << 28, 0u, s, P.sample, P.k0, P.k1);
+    if (lane == 0u) { B.setw[0] = w; B.setw[1] = o.x & (P.g.L - 1u); B.setw[2] = o.y & (P.g.L - 1u); }
+  }
+  uint4 o[4];
+  if constexpr (kGeneral) {
+    const uint32_t n = (kRounds / 2) / parts;
+    uint32_t dp = 0u, dq = 0u;   // outcomes of four round pairs
+#pragma unroll 1
+    for (uint32_t rp = part * n; rp < part * n + n; ++rp) {
+      const uint32_t c[4] = {(kTagPos << 28) | (lane << 3) | rp, (kTagAcc << 28) | (lane << 4) | (2u * rp),
+                             (kTagAcc << 28) | (lane << 4) | (2u * rp + 1u), (kTagDeep << 28) | (lane << 8) | (rp << 4)};
+      philox4(c, tid, s, P.sample, P.k0, P.k1, o);
+      B.pos[rp][lane] = o[0];
+      B.acc[2u * rp][lane] = o[1];
+      B.acc[2u * rp + 1u][lane] = o[2];
+      const uint32_t j = 2u * (rp & 3u);
+      dp |= (deep_below(o[3].x, o[3].y, P.Tp) >> j) | (deep_below(o[3].z, o[3].w, P.Tp) >> (j + 1u));
+      dq |= (deep_below(o[3].x, o[3].y, P.Tq) >> j) | (deep_below(o[3].z, o[3].w, P.Tq) >> (j + 1u));
+      if ((rp & 3u) == 3u) {
+        B.deep[rp >> 2][lane] = make_uint2(dp, dq);
+        dp = dq = 0u;
+      }
+    }
+  } else {
+    const uint32_t n = (kRounds / 2) / parts;
+#pragma unroll 1
+    for (uint32_t rp = part * n; rp < part * n + n; rp += 4u) {
+      const uint32_t c0 = (kTagPos << 28) | (lane << 3) | rp;
+      const uint32_t c[4] = {c0, c0 + 1u, c0 + 2u, c0 + 3u};
+      philox4(c, tid, s, P.sample, P.k0, P.k1, o);
+#pragma unroll
+      for (uint32_t i = 0; i < 4u; ++i) B.pos[rp + i][lane] = o[i];
+    }
+  }
+}
+
+// Acceptance of a general-rate round from the drawn blocks (the rule of
+// rounds::one_round): the candidates' top four bits against their threshold
+// (Tp's bits for a minimum, Tq's for a maximum) by a majority chain, ties by
+// the low twelve bits. No votes: the numbers are there already.
+struct Rates {
+  uint32_t dpm, dqm, pall, qall, bp[4], bq[4];
+  __device__ __forceinline__ explicit Rates(const SweepParams& P) {
+    dpm = (P.Tp != 0u && P.Tp < 65536u) ? ~0u : 0u;
+    dqm = (P.Tq != 0u && P.Tq < 65536u) ? ~0u : 0u;
+    pall = (P.Tp >> 16) ? ~0u : 0u;
+    qall = (P.Tq >> 16) ? ~0u : 0u;
+#pragma unroll
+    for (uint32_t n = 0; n < 4u; ++n) {
+      bp[n] = 0u - ((P.Tp >> (15u - n)) & 1u);
+      bq[n] = 0u - ((P.Tq >> (15u - n)) & 1u);
+    }
+  }
+};
+// All ones where the top bit of byte k of w is set.
+template <int k>
+__device__ __forceinline__ uint32_t byte_mask(uint32_t w) {
+  uint32_t r;
+  asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r) : "r"(w), "n"(0x8888 + 0x1111 * k));
+  return r;
+}
+__device__ __forceinline__ uint32_t accept_cells(const SweepParams& P, const Rates& R, const TileCtx& tc, const uint4& A,
+                                                 const uint2& W, uint32_t lane, uint32_t r, uint32_t up, uint32_t uq) {
+  const uint32_t dm = (up & R.dpm) | (uq & R.dqm);   // candidates that need random bits
+  const uint32_t w[4] = {A.x, A.y, A.z, A.w};
+  uint32_t b[4];
+#pragma unroll
+  for (uint32_t n = 0; n < 4u; ++n) b[n] = (up & R.bp[n]) | (~up & R.bq[n]);
+  uint32_t lt = 0u;
+#pragma unroll
+  for (int n = 3; n >= 0; --n) lt = (~w[n] & lt) | (~w[n] & b[n]) | (lt & b[n]);
+  const uint32_t tie = (dm & ~(w[0] ^ b[0]) & ~(w[1] ^ b[1])) & (~(w[2] ^ b[2]) & ~(w[3] ^ b[3]));
+  uint32_t acc = (up & R.pall) | (uq & R.qall) | (lt & dm);
+  // The k-th tie from below takes the k-th outcome.
+  const uint32_t g0 = (up & byte_mask<0>(W.x)) | (~up & byte_mask<0>(W.y));
+  const uint32_t g1 = (up & byte_mask<1>(W.x)) | (~up & byte_mask<1>(W.y));
+  const uint32_t g2 = (up & byte_mask<2>(W.x)) | (~up & byte_mask<2>(W.y));
+  const uint32_t g3 = (up & byte_mask<3>(W.x)) | (~up & byte_mask<3>(W.y));
+  const uint32_t m1 = tie & (tie - 1u), m2 = m1 & (m1 - 1u), m3 = m2 & (m2 - 1u), m4 = m3 & (m3 - 1u);
+  acc |= (tie & ~m1 & g0) | (m1 & ~m2 & g1) | (m2 & ~m3 & g2) | (m3 & ~m4 & g3);
+  if (m4 != 0u) {   // more than four ties in a row: the overflow blocks of the round
+    uint4 X = make_uint4(0u, 0u, 0u, 0u);
+    uint32_t m = m4;
+    for (uint32_t k = 0u; m != 0u; ++k) {
+      const uint32_t bit = m & (0u - m);
+      m ^= bit;
+      if ((k & 7u) == 0u)
+        X = philox((kTagDeep << 28) | (lane << 8) | (r << 3) | (1u + (k >> 3)), tc.tid, tc.s, P.sample, P.k0, P.k1);
+      const uint32_t x = (k & 4u) ? ((k & 2u) ? X.w : X.z) : ((k & 2u) ? X.y : X.x);
+      const uint32_t h = ((k & 1u) ? (x >> 16) : x) & 0xFFFu;
+      acc |= (h < (((bit & up) ? P.Tp : P.Tq) & 0xFFFu)) ? bit : 0u;
+    }
+  }
+  return acc;
+}
+
+// The 16 single-hit rounds of the tile in m from its drawn numbers. The
+// offsets and numbers of a round are loaded one round ahead, so its chain is
+// quadrant in, logic, quadrant out.
+template <bool kGeneral, int kPar, bool kTrack>
+__device__ __forceinline__ int rounds_from(TileMem& m, const QuadTab& tab, uint32_t ghost, const SweepParams& P,
+                                           const TileCtx& tc, const tilemem::Origin& og, const TileRand<kGeneral>& B,
+                                           uint32_t lane) {
+  char* base = reinterpret_cast<char*>(&m) + lane * 8u;
+  int dh = 0;
+  const Rates R(P);
+  auto one = [&](const uint4& at, const uint4& sh, uint32_t X, uint32_t Y, uint32_t r, const uint4& A, const uint2& W) {
+    if constexpr (kGeneral)
+      tilemem::round_general<kPar, kTrack>(base, at, sh, ghost, X, Y, og, dh, [&](uint32_t up, uint32_t uq) {
+        return accept_cells(P, R, tc, A, W, lane, r, up, uq);
+      });
+    else
+      tilemem::round_p1<kPar, kTrack>(base, at, sh, ghost, X, Y, og, dh);
+  };
+  uint32_t setw = tc.setw;
+  uint4 at0 = tab.at[setw & 3u], sh0 = tab.sh[setw & 3u], pos = B.pos[0][lane];
+  uint4 A0 = B.acc[0][kGeneral ? lane : 0u];
+  uint2 W = B.deep[0][kGeneral ? lane : 0u];   // outcomes of the next eight rounds, shifted round by round
+#pragma unroll 1
+  for (uint32_t rp = 0; rp < kRounds / 2; ++rp) {
+    const uint32_t k1 = (setw >> 2) & 3u, k2 = (setw >> 4) & 3u, nx = (rp + 1u) & 7u;
+    setw >>= 4;
+    const uint4 at1 = tab.at[k1], sh1 = tab.sh[k1];
+    uint4 A1 = A0;
+    if constexpr (kGeneral) {
+      A1 = B.acc[2u * rp + 1u][lane];
+      if (rp == 4u) W = B.deep[1][lane];
+    }
+    one(at0, sh0, pos.x, pos.y, 2u * rp, A0, W);
+    at0 = tab.at[k2];
+    sh0 = tab.sh[k2];
+    const uint4 pn = B.pos[nx][lane];
+    if constexpr (kGeneral) A0 = B.acc[2u * nx][lane];
+    one(at1, sh1, pos.z, pos.w, 2u * rp + 1u, A1, make_uint2(W.x << 1, W.y << 1));
+    pos = pn;
+    W.x <<= 2;
+    W.y <<= 2;
+  }
+  return dh;
+}
+
+// Lattice words in HBM / L2: other SMs change them between steps, so reads
+// bypass L1.
+struct GlobalLat {
+  uint32_t* p;
+  __device__ __forceinline__ uint32_t ld(uint32_t i) const { return __ldcg(p + i); }
+  __device__ __forceinline__ void st(uint32_t i, uint32_t v) const { __stcg(p + i, v); }
+};
+// A tile's words and the sites around it.
+struct Window {
+  uint32_t T[4][4], hx[4], hy[4], left[4], up[4];
+};
+
+// The window whose site (0,0) is site (X0, Y0) of the frame the lattice is
+// held in (geometry as in run::sweep_run, kpz_run.cuh). kHalo: 0 the tile
+// alone, 1 with the column right of it (hx) and the row below it (hy), 2 also
+// the column left of it and the row above.
+template <int kHalo>
+__device__ __forceinline__ void load_window(const Geometry& g, const GlobalLat lat, uint32_t lane, uint32_t X0,
+                                            uint32_t Y0, Window& w) {
+  const uint32_t NR = g.NR, NB = g.NB;
+  const uint32_t by = Y0 & 3u, Rb = Y0 >> 2, bx = X0 & 3u, a = X0 >> 2;
+  uint32_t offY[4], sh[4], w0[4], w1[4], wm3 = 0u;
+#pragma unroll
+  for (uint32_t yq = 0; yq < 4; ++yq)
+    offY[yq] = ((by + yq) & 3u) * 4u * NR + ((Rb + lane + ((by + yq) >> 2)) & (NR - 1u));
+  const uint32_t offH = by * 4u * NR + ((Rb + 32u) & (NR - 1u));                                   // row below
+  const uint32_t offU = ((by + 3u) & 3u) * 4u * NR + ((Rb - 1u + ((by + 3u) >> 2)) & (NR - 1u));   // row above
+#pragma unroll
+  for (uint32_t xq = 0; xq < 4; ++xq) {
+    const uint32_t st = (a + ((bx + xq) >> 2)) & (g.L / 4u - 1u);
+    const uint32_t kx = st >> 5, offX = ((bx + xq) & 3u) * NR;
+    sh[xq] = st & 31u;
+    w0[xq] = kx * kPlanes * NR + offX;
+    w1[xq] = ((kx + 1u) & (NB - 1u)) * kPlanes * NR + offX;
+    if (xq == 3) wm3 = ((kx + NB - 1u) & (NB - 1u)) * kPlanes * NR + offX;
+  }
+  uint32_t C[4][4], N[4][4], H[4][2], U[4][2], B3[4];
+#pragma unroll
+  for (uint32_t xq = 0; xq < 4; ++xq) {
+#pragma unroll
+    for (uint32_t yq = 0; yq < 4; ++yq) {
+      C[yq][xq] = lat.ld(w0[xq] + offY[yq]);
+      N[yq][xq] = lat.ld(w1[xq] + offY[yq]);
+      if (kHalo == 2 && xq == 3) B3[yq] = lat.ld(wm3 + offY[yq]);
+    }
+    if (kHalo >= 1) { H[xq][0] = lat.ld(w0[xq] + offH); H[xq][1] = lat.ld(w1[xq] + offH); }   // lane 31 needs it
+    if (kHalo == 2) { U[xq][0] = lat.ld(w0[xq] + offU); U[xq][1] = lat.ld(w1[xq] + offU); }   // lane 0 needs it
+  }
+#pragma unroll
+  for (uint32_t xq = 0; xq < 4; ++xq) {
+#pragma unroll
+    for (uint32_t yq = 0; yq < 4; ++yq) {
+      w.T[yq][xq] = __funnelshift_r(C[yq][xq], N[yq][xq], sh[xq]);
+      if (kHalo >= 1 && xq == 0) w.hx[yq] = (N[yq][0] >> sh[0]) & 1u;
+      if (kHalo == 2 && xq == 3) w.left[yq] = ((sh[3] ? C[yq][3] : B3[yq]) >> ((sh[3] + 31u) & 31u)) & 1u;
+    }
+    if (kHalo >= 1) w.hy[xq] = __funnelshift_r(H[xq][0], H[xq][1], sh[xq]);
+    if (kHalo == 2) w.up[xq] = __funnelshift_r(U[xq][0], U[xq][1], sh[xq]);
+  }
+}
+
+// Tile (tx, ty) of the frame the lattice is held in, with all sites around it.
+__device__ __forceinline__ void load_tile(const Geometry& g, const GlobalLat lat, uint32_t lane, uint32_t tx, uint32_t ty,
+                                          Window& w) {
+  const uint32_t NR = g.NR, NB = g.NB, R = ty * 32u + lane;
+  const uint32_t Ru = (ty * 32u + NR - 1u) & (NR - 1u), Rd = (ty * 32u + 32u) & (NR - 1u);
+  const uint32_t o = tx * kPlanes * NR, ol = ((tx + NB - 1u) & (NB - 1u)) * kPlanes * NR,
+                 orr = ((tx + 1u) & (NB - 1u)) * kPlanes * NR;
+#pragma unroll
+  for (uint32_t y = 0; y < 4; ++y) {
+#pragma unroll
+    for (uint32_t x = 0; x < 4; ++x) w.T[y][x] = lat.ld(o + plane(y, x) * NR + R);
+    w.left[y] = lat.ld(ol + plane(y, 3) * NR + R) >> 31;
+    w.hx[y] = lat.ld(orr + plane(y, 0) * NR + R) & 1u;
+  }
+#pragma unroll
+  for (uint32_t x = 0; x < 4; ++x) {
+    w.hy[x] = lat.ld(o + plane(0, x) * NR + Rd);
+    w.up[x] = lat.ld(o + plane(3, x) * NR + Ru);
+  }
+}
+
+__device__ __forceinline__ void store_tile(const Geometry& g, const GlobalLat lat, uint32_t lane, uint32_t tx, uint32_t ty,
+                                           const uint32_t (&T)[4][4]) {
+  const uint32_t o = tx * kPlanes * g.NR + ty * 32u + lane;
+#pragma unroll
+  for (uint32_t y = 0; y < 4; ++y)
+#pragma unroll
+    for (uint32_t x = 0; x < 4; ++x) lat.st(o + plane(y, x) * g.NR, T[y][x]);
+}
+
+// The rounds of tile (tx, ty) of the sweep with origin (ox, oy); w.T holds the
+// tile before and after. kLive: every site of the tile is live, its neighbours
+// are idle (kpz_tileset.cu); otherwise its low row and column are dead.
+template <bool kGeneral, bool kLive>
+__device__ __forceinline__ void tile_rounds(const SweepParams& P, Window& w, TileMem& m, const QuadTab& tab,
+                                            const TileRand<kGeneral>& B, uint32_t lane, uint32_t s, uint32_t ox,
+                                            uint32_t oy, uint32_t tx, uint32_t ty) {
+  const uint32_t L = P.g.L;
+  const uint32_t Y0 = (oy + ty * kTile) & (L - 1u), X0 = (ox + tx * kTile) & (L - 1u);
+  TileCtx tc;   // what the overflow draws need
+  tc.tid = ty * P.ntx + tx;
+  tc.s = s;
+  tc.setw = B.setw[0];
+  const uint32_t uo = (0u - X0) & (L - 1u), vo = (0u - Y0) & (L - 1u);
+  const bool track = (uo < kTile) && (vo < kTile), odd = (X0 + Y0 + P.g.par) & 1u;
+  const tilemem::Origin og(lane, uo, vo);
+  const uint32_t ghost = tilemem::put_tile<kLive>(m, lane, w.T, w.hx, w.hy, w.left, w.up);
+  int dh;
+  if (track) dh = odd ? rounds_from<kGeneral, 1, true>(m, tab, ghost, P, tc, og, B, lane)
+                      : rounds_from<kGeneral, 0, true>(m, tab, ghost, P, tc, og, B, lane);
+  else       dh = odd ? rounds_from<kGeneral, 1, false>(m, tab, ghost, P, tc, og, B, lane)
+                      : rounds_from<kGeneral, 0, false>(m, tab, ghost, P, tc, og, B, lane);
+  if (track && dh != 0) atomicAdd(P.h00, (unsigned long long)(long long)dh);
+#pragma unroll
+  for (uint32_t y = 0; y < 4; ++y)
+#pragma unroll
+    for (uint32_t px = 0; px < 2; ++px) {
+      const uint2 v = m.w[y][px][1u + lane];
+      w.T[y][2 * px] = v.x;
+      w.T[y][2 * px + 1] = v.y;
+    }
+}
+
+// Set swept in phase `phase` of sweep s (the shuffle of kpz_tileset.cu).
+__device__ __forceinline__ uint32_t phase_set(const SweepParams& P, uint32_t s, uint32_t phase) {
+  const uint4 w = philox(kTagPhase << 28, 0u, s, P.sample, P.k0, P.k1);
+  uint32_t perm[4] = {0u, 1u, 2u, 3u};
+  const uint32_t r[3] = {w.x, w.y, w.z};
+#pragma unroll
+  for (uint32_t i = 3; i >= 1; --i) {
+    const uint32_t j = r[3 - i] % (i + 1u);
+    const uint32_t t = perm[i];
+    perm[i] = j == 0u ? perm[0] : j == 1u ? perm[1] : j == 2u ? perm[2] : t;
+    if (j == 0u) perm[0] = t; else if (j == 1u) perm[1] = t; else if (j == 2u) perm[2] = t;
+  }
+  return phase == 0u ? perm[0] : phase == 1u ? perm[1] : phase == 2u ? perm[2] : perm[3];
+}
+
+__device__ __forceinline__ uint64_t now_ns() {
+  uint64_t t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+__device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint32_t add_release(uint32_t* p, uint32_t v) {
+  uint32_t old;
+  asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+  return old;
+}
+__device__ __forceinline__ void red_release(uint32_t* p) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
+}
+__device__ __forceinline__ void bar_sync(uint32_t id, uint32_t n) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(uint32_t id, uint32_t n) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+constexpr uint64_t kWaitNs = 10000000000ull;   // bound of every grid wait
+
+// Grid version. A step is a sweep, or one tile set of a sweep (kSets); every
+// tile of a step has a tile warp of its own. Warps of a block: wpc tile warps,
+// makers * wpc drawing warps (they draw the next step's numbers into the other
+// of two buffers while this step runs; with makers = 0 the tile warps draw
+// their own numbers while the barrier is pending) and one barrier warp, which
+// collects the block (named barrier 1), reports the step to the grid, waits
+// for all blocks (bounded in time) and releases the block (named barrier 2).
+// A last step brings the lattice back to the fixed frame.
+template <bool kGeneral, bool kSets>
+__global__ void __launch_bounds__(320, 1) resident_grid_kernel(const SweepParams P, uint32_t n, uint32_t tiles,
+                                                               uint32_t wpc, uint32_t makers, uint32_t* scratch,
+                                                               ResidentSync* sync) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  TileRand<kGeneral>* rnd = reinterpret_cast<TileRand<kGeneral>*>(smem_raw);   // [1 or 2][wpc]
+  TileMem* mem = reinterpret_cast<TileMem*>(rnd + (makers ? 2u : 1u) * wpc);   // [wpc]
+  __shared__ QuadTab tab;
+  __shared__ uint32_t stop;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const uint32_t nsteps = n * (kSets ? 4u : 1u);   // without the last one
+  if (threadIdx.x == 0) stop = 0u;
+  if (threadIdx.x < 4u) tilemem::fill_quad_tab(tab, threadIdx.x);
+  __syncthreads();
+  if (warp == nwarps - 1u) {   // barrier warp
+    for (uint32_t k = 1; k <= nsteps; ++k) {
+      bar_sync(1, blockDim.x);
+      if (lane == 0) {
+        red_release(&sync->arrived);
+        const uint32_t want = k * gridDim.x;
+        if (ld_acquire(&sync->arrived) < want) {
+          const uint64_t t0 = now_ns();
+          for (uint32_t it = 1; ld_acquire(&sync->arrived) < want; ++it) {
+            if ((it & 63u) == 0u && (now_ns() - t0 > kWaitNs || *(volatile uint32_t*)&sync->err)) {
+              atomicExch(&sync->err, 1u);
+              stop = 1u;
+              break;
+            }
+          }
+        }
+      }
+      __syncwarp();
+      bar_sync(2, blockDim.x);
+      if (*(volatile uint32_t*)&stop) return;
+    }
+    bar_sync(1, blockDim.x);
+    // The last block out resets the counters and advances the sweep count.
+    if (lane == 0) {
+      __threadfence();
+      if (add_release(&sync->finished, 1u) == gridDim.x - 1u) {
+        sync->arrived = 0u;
+        sync->finished = 0u;
+        *const_cast<uint64_t*>(P.t_dev) += n;
+      }
+    }
+    return;
+  }
+  const uint32_t t0 = (uint32_t)(*(const volatile uint64_t*)P.t_dev) + P.s_add;
+  const bool maker = warp >= wpc;
+  const uint32_t slot = maker ? (warp - wpc) % wpc : warp, part = maker ? (warp - wpc) / wpc : 0u;
+  const uint32_t c = blockIdx.x * wpc + slot;    // this warp's tile of every step
+  const uint32_t across = kSets ? P.ntx / 2u : P.ntx, cy = c / across, cx = c - cy * across;
+  const bool live = c < tiles;
+  // Sweep and tile of step k.
+  auto place = [&](uint32_t k, uint32_t& s, uint32_t& tx, uint32_t& ty) {
+    s = t0 + (kSets ? k >> 2 : k);
+    const uint32_t set = kSets ? phase_set(P, s, k & 3u) : 0u;
+    tx = kSets ? 2u * cx + (set & 1u) : cx;
+    ty = kSets ? 2u * cy + (set >> 1) : cy;
+  };
+  const uint32_t L = P.g.L, words = L * L / 32u;
+  uint32_t s, tx, ty, ox = 0u, oy = 0u, px = 0u, py = 0u;
+  if (maker) {
+    place(0u, s, tx, ty);
+    if (live) draw_tile<kGeneral>(P, rnd[slot], ty * P.ntx + tx, s, lane, part, makers);
+  }
+  if (makers) bar_sync(3, blockDim.x - 32u);
+  for (uint32_t k = 0; k <= nsteps; ++k) {
+    if (k != 0u && makers) {
+      bar_sync(2, blockDim.x);
+      if (*(volatile uint32_t*)&stop) return;
+    }
+    if (maker) {
+      if (k + 1u < nsteps && live) {
+        place(k + 1u, s, tx, ty);
+        draw_tile<kGeneral>(P, rnd[((k + 1u) & 1u) * wpc + slot], ty * P.ntx + tx, s, lane, part, makers);
+      }
+    } else {
+      const uint32_t sw = kSets ? k >> 2 : k;    // sweeps before this step
+      const bool back = k == nsteps;             // the fixed frame again
+      TileRand<kGeneral>& B = rnd[(makers ? (k & 1u) * wpc : 0u) + slot];
+      place(k, s, tx, ty);
+      if (!kSets || (k & 3u) == 0u) {
+        px = ox;
+        py = oy;
+      }
+      if (!makers) {
+        if (live && !back) draw_tile<kGeneral>(P, B, ty * P.ntx + tx, s, lane, 0u, 1u);
+        __syncwarp();
+        if (k != 0u) {
+          bar_sync(2, blockDim.x);
+          if (*(volatile uint32_t*)&stop) return;
+        }
+      }
+      if (!kSets || (k & 3u) == 0u) {
+        ox = back ? 0u : B.setw[1];
+        oy = back ? 0u : B.setw[2];
+      }
+      const GlobalLat from{sw == 0u ? P.lat : scratch + ((sw - 1u) & 1u) * words};
+      const GlobalLat to{back ? P.lat : scratch + (sw & 1u) * words};
+      if (live) {
+        Window w;
+        const uint32_t rx = ox - px, ry = oy - py;   // new frame in the old one
+        if (kSets && (back || (k & 3u) == 0u)) {     // the four tiles of this warp change frames
+#pragma unroll 1
+          for (uint32_t q = 0; q < 4u; ++q) {
+            const uint32_t qx = 2u * cx + (q & 1u), qy = 2u * cy + (q >> 1);
+            if (!back && qx == tx && qy == ty) continue;
+            load_window<0>(P.g, from, lane, (rx + qx * kTile) & (L - 1u), (ry + qy * kTile) & (L - 1u), w);
+            store_tile(P.g, to, lane, qx, qy, w.T);
+          }
+        }
+        if (kSets) {
+          if (!back) {
+            if ((k & 3u) == 0u)
+              load_window<2>(P.g, from, lane, (rx + tx * kTile) & (L - 1u), (ry + ty * kTile) & (L - 1u), w);
+            else
+              load_tile(P.g, to, lane, tx, ty, w);
+            tile_rounds<kGeneral, true>(P, w, mem[slot], tab, B, lane, s, ox, oy, tx, ty);
+            store_tile(P.g, to, lane, tx, ty, w.T);
+          }
+        } else {
+          load_window<1>(P.g, from, lane, (rx + tx * kTile) & (L - 1u), (ry + ty * kTile) & (L - 1u), w);
+          if (!back) tile_rounds<kGeneral, false>(P, w, mem[slot], tab, B, lane, s, ox, oy, tx, ty);
+          store_tile(P.g, to, lane, tx, ty, w.T);
+        }
+      }
+    }
+    bar_arrive(1, blockDim.x);
+  }
+}
+
+// Cluster version (L <= 1024): one cluster of 1 to 16 blocks holds the whole
+// lattice in its shared memory, two frames of it by turns, a block the words
+// of its `tpc` tiles; windows are read over distributed shared memory and the
+// hardware's cluster barrier ends a sweep. Warps of a block: tpc tile warps,
+// makers * tpc drawing warps.
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint32_t map_to(uint32_t addr, uint32_t cta) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(cta));
+  return r;
+}
+__device__ __forceinline__ uint32_t ld_cluster(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// load_window over the cluster: `lat` = shared address of the frame in every
+// block ([tpc][16 planes][32 lanes] words), tpc = 1 << lg tiles per block.
+template <int kHalo>
+__device__ __forceinline__ void load_window_cluster(const SweepParams& P, uint32_t lat, uint32_t lg, uint32_t lane,
+                                                    uint32_t X0, uint32_t Y0, Window& w) {
+  const uint32_t NR = P.g.NR, NB = P.g.NB;
+  const uint32_t by = Y0 & 3u, Rb = Y0 >> 2, bx = X0 & 3u, a = X0 >> 2, K = a >> 5;
+  // Address of plane 0 of block columns K, K + 1, K + 2 at cell rows Rb + lane,
+  // Rb + lane + 1 and Rb + 32.
+  uint32_t at[3][3];
+#pragma unroll
+  for (uint32_t i = 0; i < (kHalo ? 3u : 2u); ++i) {
+    const uint32_t R = (Rb + (i == 2u ? 32u : lane + i)) & (NR - 1u);
+#pragma unroll
+    for (uint32_t j = 0; j < 3u; ++j) {
+      const uint32_t t = (R >> 5) * P.ntx + ((K + j) & (NB - 1u));
+      at[i][j] = map_to(lat + (t & ((1u << lg) - 1u)) * (kPlanes * 128u) + (R & 31u) * 4u, t >> lg);
+    }
+  }
+  uint32_t C[4][4], N[4][4], H[4][2], sh[4];
+#pragma unroll
+  for (uint32_t xq = 0; xq < 4; ++xq) {
+    const uint32_t st = a + ((bx + xq) >> 2), x4 = (bx + xq) & 3u;
+    sh[xq] = st & 31u;
+    const bool next = (st >> 5) != K;   // carried into the next block column
+#pragma unroll
+    for (uint32_t yq = 0; yq < 4; ++yq) {
+      const uint32_t y4 = (by + yq) & 3u, p = plane(y4, x4) * 128u;
+      const bool wrap = by + yq >= 4u;
+      const uint32_t a0 = wrap ? at[1][0] : at[0][0], a1 = wrap ? at[1][1] : at[0][1], a2 = wrap ? at[1][2] : at[0][2];
+      C[yq][xq] = ld_cluster((next ? a1 : a0) + p);
+      N[yq][xq] = ld_cluster((next ? a2 : a1) + p);
+    }
+    if (kHalo) {
+      const uint32_t p = plane(by, x4) * 128u;
+      H[xq][0] = ld_cluster((next ? at[2][1] : at[2][0]) + p);
+      H[xq][1] = ld_cluster((next ? at[2][2] : at[2][1]) + p);
+    }
+  }
+#pragma unroll
+  for (uint32_t xq = 0; xq < 4; ++xq) {
+#pragma unroll
+    for (uint32_t yq = 0; yq < 4; ++yq) {
+      w.T[yq][xq] = __funnelshift_r(C[yq][xq], N[yq][xq], sh[xq]);
+      if (kHalo && xq == 0) w.hx[yq] = (N[yq][0] >> sh[0]) & 1u;
+    }
+    if (kHalo) w.hy[xq] = __funnelshift_r(H[xq][0], H[xq][1], sh[xq]);
+  }
+}
+
+template <bool kGeneral>
+__global__ void __launch_bounds__(384, 1) resident_cluster_kernel(const SweepParams P, uint32_t n, uint32_t lg,
+                                                                  uint32_t makers) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const uint32_t tpc = 1u << lg;
+  TileRand<kGeneral>* rnd = reinterpret_cast<TileRand<kGeneral>*>(smem_raw);   // [2][tpc]
+  TileMem* mem = reinterpret_cast<TileMem*>(rnd + 2u * tpc);                   // [tpc]
+  uint32_t* frame = reinterpret_cast<uint32_t*>(mem + tpc);                    // [2][tpc][16][32]
+  __shared__ QuadTab tab;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const uint32_t t0 = (uint32_t)(*(const volatile uint64_t*)P.t_dev) + P.s_add;
+  const uint32_t L = P.g.L;
+  if (threadIdx.x < 4u) tilemem::fill_quad_tab(tab, threadIdx.x);
+  const bool maker = warp >= tpc;
+  const uint32_t slot = maker ? (warp - tpc) & (tpc - 1u) : warp, part = maker ? (warp - tpc) >> lg : 0u;
+  const uint32_t tile = blockIdx.x * tpc + slot, ty = tile / P.ntx, tx = tile - ty * P.ntx;
+  uint32_t* own = frame + slot * (kPlanes * 32u) + lane;   // this lane's words, 32 apart; + the frame's offset
+  const uint32_t half = tpc * kPlanes * 32u;               // words of one frame in this block
+  Window w;
+  if (maker) {
+    draw_tile<kGeneral>(P, rnd[slot], tile, t0, lane, part, makers);
+  } else {
+    const uint32_t o = tx * kPlanes * P.g.NR + ty * 32u + lane;
+#pragma unroll
+    for (uint32_t p = 0; p < kPlanes; ++p) own[p * 32u] = __ldcg(P.lat + o + p * P.g.NR);
+  }
+  uint32_t px = 0u, py = 0u;
+  cluster_sync();
+  for (uint32_t k = 0; k < n; ++k) {
+    const uint32_t s = t0 + k, buf = k & 1u;
+    if (maker) {
+      if (k + 1u < n) draw_tile<kGeneral>(P, rnd[(buf ^ 1u) * tpc + slot], tile, s + 1u, lane, part, makers);
+    } else {
+      const TileRand<kGeneral>& B = rnd[buf * tpc + slot];
+      const uint32_t ox = B.setw[1], oy = B.setw[2];
+      load_window_cluster<1>(P, smem_u32(frame + buf * half), lg, lane, (ox - px + tx * kTile) & (L - 1u),
+                             (oy - py + ty * kTile) & (L - 1u), w);
+      tile_rounds<kGeneral, false>(P, w, mem[slot], tab, B, lane, s, ox, oy, tx, ty);
+      uint32_t* to = own + (buf ^ 1u) * half;
+#pragma unroll
+      for (uint32_t p = 0; p < kPlanes; ++p) to[p * 32u] = w.T[p >> 2][p & 3u];
+      px = ox;
+      py = oy;
+    }
+    cluster_sync();
+  }
+  if (!maker) {
+    load_window_cluster<0>(P, smem_u32(frame + (n & 1u) * half), lg, lane, (tx * kTile - px) & (L - 1u),
+                           (ty * kTile - py) & (L - 1u), w);
+    store_tile(P.g, GlobalLat{P.lat}, lane, tx, ty, w.T);
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) *const_cast<uint64_t*>(P.t_dev) += n;
+  cluster_sync();   // no block leaves while its shared memory is read
+}
+
+struct Shape {
+  bool cluster;             // cluster version
+  uint32_t wpc, grid;       // tile warps per block, blocks
+  uint32_t tiles, makers;   // tiles per step, drawing warps per tile
+  size_t smem;
+};
+
+// How a lattice is laid over the chip (wpc = 0: not served). p = 1 draws 8
+// blocks a tile and sweep, general rates 32; one warp draws a block in about
+// 120 cycles, an SM's quarter in 80 (the wide multiplies), so drawing warps
+// pay while an SM has at most two tiles; with eight they take the issue slots
+// the tile warps need (L = 4096 at p = 0.95: 9.0 us a sweep with them, 7.9
+// without). The cluster serves up to 64 tiles, four a block: there it takes
+// 2.7 / 4.6 us a sweep against 3.3 / 5.4 on a grid of 64 blocks, at 16 tiles
+// 2.1 / 3.4 against 3.2 / 5.4. Beyond 1024 tiles an SM would have more than
+// two tiles a scheduler, and work, not latency, is the bound.
+Shape shape_of(const SweepParams& P, bool tilesets, bool general, bool cluster) {
+  Shape h{};
+  const size_t rnd = general ? sizeof(TileRand<true>) : sizeof(TileRand<false>);
+  const uint32_t all = P.ntx * P.nty;
+  if (cluster) {
+    if (tilesets || all > 64u) return h;
+    h.cluster = true;
+    h.tiles = all;
+    h.grid = std::min(all, 16u);
+    h.wpc = all / h.grid;
+    h.makers = general ? 2u : 1u;
+    h.smem = h.wpc * (2u * rnd + sizeof(TileMem) + 2u * kPlanes * 32u * sizeof(uint32_t));
+    return h;
+  }
+  h.tiles = tilesets ? all / 4u : all;
+  if (h.tiles > 1024u) return h;
+  h.wpc = std::max(1u, h.tiles / 128u);      // up to 128 blocks of 1 to 8 tile warps
+  h.grid = (h.tiles + h.wpc - 1u) / h.wpc;
+  h.makers = h.wpc > 2u ? 0u : (general ? 2u : 1u);
+  h.smem = h.wpc * ((h.makers ? 2u : 1u) * rnd + sizeof(TileMem));
+  return h;
+}
+
+const void* kernel_of(const Shape& h, bool tilesets, bool general) {
+  if (h.cluster)
+    return general ? (const void*)resident_cluster_kernel<true> : (const void*)resident_cluster_kernel<false>;
+  if (tilesets)
+    return general ? (const void*)resident_grid_kernel<true, true> : (const void*)resident_grid_kernel<false, true>;
+  return general ? (const void*)resident_grid_kernel<true, false> : (const void*)resident_grid_kernel<false, false>;
+}
+
+uint32_t threads_of(const Shape& h) { return 32u * (h.wpc * (1u + h.makers) + (h.cluster ? 0u : 1u)); }
+
+cudaLaunchConfig_t config_of(const Shape& h, cudaLaunchAttribute* attr, cudaStream_t st) {
+  if (h.cluster) {
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = h.grid;
+    attr->val.clusterDim.y = attr->val.clusterDim.z = 1u;
+  } else {
+    attr->id = cudaLaunchAttributeCooperative;
+    attr->val.cooperative = 1;
+  }
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(h.grid);
+  c.blockDim = dim3(threads_of(h));
+  c.dynamicSmemBytes = h.smem;
+  c.stream = st;
+  c.attrs = attr;
+  c.numAttrs = 1;
+  return c;
+}
+
+// Whether the current device holds all blocks of the kernel at once.
+bool fits(const Shape& h, bool tilesets, bool general) {
+  if (h.wpc == 0u) return false;
+  int dev = 0, per_sm = 0, sms = 0, coop = 0;
+  const void* f = kernel_of(h, tilesets, general);
+  bool ok = cudaGetDevice(&dev) == cudaSuccess &&
+            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h.smem) == cudaSuccess;
+  if (ok && h.cluster) {
+    if (h.grid > 8u) ok = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t c = config_of(h, &attr, nullptr);
+    int clusters = 0;
+    ok = ok && cudaOccupancyMaxActiveClusters(&clusters, f, &c) == cudaSuccess && clusters > 0;
+  } else if (ok) {
+    ok = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
+         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, (int)threads_of(h), h.smem) == cudaSuccess &&
+         (uint32_t)(per_sm * sms) >= h.grid;
+  }
+  if (!ok) cudaGetLastError();
+  return ok;
+}
+
+bool is_general(const SweepParams& P) { return !(P.Tp == 65536u && P.Tq == 0u); }
+
+}  // namespace
+
+uint32_t resident_kind(const SweepParams& P, bool tilesets) {
+  if (P.cell == 2u || P.nty * kTile != P.g.L) return 0u;
+  const bool general = is_general(P);
+  if (fits(shape_of(P, tilesets, general, true), tilesets, general)) return 2u;
+  return fits(shape_of(P, tilesets, general, false), tilesets, general) ? 1u : 0u;
+}
+
+cudaError_t launch_resident(const SweepParams& P, bool tilesets, uint32_t kind, uint32_t n, uint32_t* scratch,
+                            ResidentSync* sync, cudaStream_t st) {
+  const bool general = is_general(P);
+  const Shape h = shape_of(P, tilesets, general, kind == 2u);
+  if (h.wpc == 0u) return cudaErrorInvalidValue;
+  SweepParams Q = P;
+  uint32_t nn = n, makers = h.makers, tiles = h.tiles, wpc = h.wpc, lg = 0u;
+  while ((1u << lg) < h.wpc) ++lg;
+  void* cluster_args[] = {&Q, &nn, &lg, &makers};
+  void* grid_args[] = {&Q, &nn, &tiles, &wpc, &makers, &scratch, &sync};
+  cudaLaunchAttribute attr;
+  const cudaLaunchConfig_t c = config_of(h, &attr, st);
+  const cudaError_t e =
+      cudaLaunchKernelExC(&c, kernel_of(h, tilesets, general), h.cluster ? cluster_args : grid_args);
+  if (e != cudaSuccess) return e;
+  count_launch();
+  return cudaGetLastError();
+}
+
+}  // namespace kpz
