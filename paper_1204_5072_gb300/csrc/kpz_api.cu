@@ -8,9 +8,11 @@
 #include <atomic>
 #include <new>
 #include <string>
+#include <thread>
 
 #include "kpz.h"
 #include "kpz_internal.h"
+#include "kpz_observe.h"
 #include "kpz_resident.h"
 #include "kpz_rsu.h"
 
@@ -40,13 +42,15 @@ struct kpz_ctx {
   uint32_t* lat = nullptr;             // L*L/32 words (one bit per site)
   uint64_t* t_dev = nullptr;           // sweep counter
   unsigned long long* h00 = nullptr;   // absolute height of site (0,0)
-  unsigned long long* acc = nullptr;   // S1, S2 lo, S2 hi
+  uint32_t* ticket = nullptr;          // roughness: blocks that have finished (zero between launches)
+  long long* sums = nullptr;           // pinned host memory: results of the roughness kernel
   uint32_t* hcar = nullptr;            // import: height of (0, j0) modulo 4
   uint32_t* queue = nullptr;           // sweep work queue (zero between launches)
   ResidentSync* sync = nullptr;        // resident kernels: grid barrier and error flag
   uint32_t resident = 0;               // kpz_run's resident kernel (resident_kind), 0: one launch per sweep
+  bool direct_host = false;            // the GPU reads and writes pageable host memory itself
   bool unchecked = false;              // resident launches since the error flag was read
-  int32_t* col0 = nullptr;             // h(0,j)
+  int32_t* col0 = nullptr;             // h(0,j); roughness: the bands' partial sums
   void* io = nullptr;                  // staging band for host transfers
   size_t io_bytes = 0;
   // Slope import/export: copies on io_stream overlap the conversion kernels
@@ -82,7 +86,7 @@ Layout layout(uint32_t L) {
   Layout y{};
   const size_t lat_bytes = (size_t)L * L / 8;   // 1 bit per site
   y.lat = 0;
-  y.small = align_up(lat_bytes);                 // t, h00, acc[3], hcar, queue; at +128 ResidentSync
+  y.small = align_up(lat_bytes);                 // t, h00, hcar, queue, ticket; at +128 ResidentSync
   y.col0 = y.small + kAlign;
   y.io = y.col0 + align_up((size_t)L * 4);
   const size_t io_bytes = std::min(kIoMax, (size_t)L * L / 4);
@@ -139,6 +143,35 @@ cudaError_t io_prepare(kpz_ctx* c) {
   e = cudaEventRecord(c->io_ev[4], c->stream);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(c->io_stream, c->io_ev[4], 0);
   return e;
+}
+
+// Writes to every page of a caller's buffer that the call is about to fill.
+// Pages of a fresh allocation exist only once touched, and a GPU that is the
+// first to touch one waits some 55 us for each 64 KiB (heights at L = 2048 took
+// 28 ms into a fresh array, 1.2 ms into a touched one); the CPU takes 3.5 us a
+// page, and large buffers are split over a few threads.
+void touch_pages(void* p, size_t bytes) {
+  constexpr size_t kPage = 4096, kPart = size_t(4) << 20, kThreads = 8;
+  auto touch = [](char* a, char* b) {
+    for (; a < b; a += kPage) *(volatile char*)a = 0;
+  };
+  char* base = (char*)p;
+  const size_t parts = std::min(kThreads, bytes / kPart);
+  size_t done = 0;
+  std::thread th[kThreads];
+  size_t n = 0;
+  try {
+    for (; n + 1 < parts; ++n) {
+      const size_t end = done + bytes / parts / kPage * kPage;
+      th[n] = std::thread(touch, base + done, base + end);
+      done = end;
+    }
+  } catch (...) {   // no thread to be had: the rest is touched here
+  }
+  touch(base + done, base + bytes);
+  for (std::thread& t : th)
+    if (t.joinable()) t.join();
+  if (bytes) *(volatile char*)(base + bytes - 1) = 0;
 }
 
 // Rows per band when the staging band is used as two halves.
@@ -275,20 +308,31 @@ kpz_status kpz_init(kpz_ctx** out, uint32_t L, double p, double q, uint64_t seed
     ctx->own_buf = true;
     ctx->buf_bytes = y.total;
   }
+  if (cudaHostAlloc((void**)&ctx->sums, 8 * sizeof(long long), cudaHostAllocMapped | cudaHostAllocPortable) !=
+      cudaSuccess) {
+    cudaGetLastError();
+    if (ctx->own_buf) cudaFree(ctx->buf);
+    delete ctx;
+    return KPZ_ENOMEM;
+  }
   if (ctx->decomposition == 4u) {   // per-sweep attempt buckets of the exact random-sequential sweep
     cudaError_t e = cudaMalloc(&ctx->rsu_scratch, rsu_scratch_bytes(L));
     if (e != cudaSuccess) {
       cudaGetLastError();
+      cudaFreeHost(ctx->sums);
       if (ctx->own_buf) cudaFree(ctx->buf);
       delete ctx;
       return KPZ_ENOMEM;
     }
   }
+  int pageable = 0;
+  cudaDeviceGetAttribute(&pageable, cudaDevAttrPageableMemoryAccess, ctx->device);
+  ctx->direct_host = pageable != 0;
   char* base = (char*)ctx->buf;
   ctx->lat = (uint32_t*)(base + y.lat);
   ctx->t_dev = (uint64_t*)(base + y.small);
   ctx->h00 = (unsigned long long*)(base + y.small + 8);
-  ctx->acc = (unsigned long long*)(base + y.small + 16);
+  ctx->ticket = (uint32_t*)(base + y.small + 56);
   ctx->hcar = (uint32_t*)(base + y.small + 40);
   ctx->queue = (uint32_t*)(base + y.small + 48);
   ctx->sync = (ResidentSync*)(base + y.small + 128);
@@ -353,18 +397,15 @@ kpz_status kpz_roughness(kpz_ctx* ctx, kpz_rough* out) {
   kpz_status st = enter(ctx);
   if (st) return st;
   if (!out) return fail(ctx, KPZ_EINVAL, "null output");
-  KPZ_CUDA(launch_roughness(ctx->lat, ctx->g, ctx->col0, ctx->acc, ctx->stream));
-  // One copy of the block of small values: h00, S1, S2 lo, S2 hi, error flag.
-  unsigned char small[kAlign];
-  KPZ_CUDA(cudaMemcpyAsync(small, ctx->t_dev, sizeof(small), cudaMemcpyDeviceToHost, ctx->stream));
+  // The kernel leaves its results in pinned host memory: no copy to queue.
+  KPZ_CUDA(launch_roughness(ctx->lat, ctx->g, ctx->col0, RoughOut{ctx->ticket, ctx->sums, ctx->h00, &ctx->sync->err},
+                            ctx->stream));
   KPZ_CUDA(cudaStreamSynchronize(ctx->stream));
-  unsigned long long host[4];
-  memcpy(host, small + 16, 3 * sizeof(host[0]));
-  memcpy(host + 3, small + 8, sizeof(host[0]));
-  ResidentSync rs;
-  memcpy(&rs, small + 128, sizeof(rs));
+  const volatile long long* res = ctx->sums;
+  const unsigned long long host[4] = {(unsigned long long)res[0], (unsigned long long)res[1],
+                                      (unsigned long long)res[2], (unsigned long long)res[3]};
   ctx->unchecked = false;
-  if (rs.err) return fail(ctx, KPZ_ETIMEOUT, "a grid barrier of kpz_run timed out");
+  if (res[4]) return fail(ctx, KPZ_ETIMEOUT, "a grid barrier of kpz_run timed out");
   const uint64_t N = (uint64_t)ctx->g.L * ctx->g.L;
   out->t_mcs = ctx->t_host;
   out->n_sites = N;
@@ -385,15 +426,31 @@ kpz_status kpz_heights(kpz_ctx* ctx, int64_t* host_out, int absolute) {
   if (!host_out) return fail(ctx, KPZ_EINVAL, "null output");
   const uint32_t L = ctx->g.L;
   KPZ_CUDA(launch_col0(ctx->lat, ctx->g, ctx->col0, ctx->stream));
-  const uint32_t band = (uint32_t)std::max<size_t>(1, std::min<size_t>(L, ctx->io_bytes / ((size_t)L * 8)));
-  for (uint32_t j0 = 0; j0 < L; j0 += band) {
-    const uint32_t nr = std::min(band, L - j0);
-    KPZ_CUDA(launch_heights(ctx->lat, ctx->g, ctx->col0, j0, nr, absolute ? ctx->h00 : nullptr,
-                            (int64_t*)ctx->io, ctx->stream));
-    KPZ_CUDA(cudaMemcpyAsync(host_out + (size_t)j0 * L, ctx->io, (size_t)nr * L * 8,
-                             cudaMemcpyDeviceToHost, ctx->stream));
+  touch_pages(host_out, (size_t)L * L * 8);
+  if (ctx->direct_host) {   // the kernel stores to the caller's buffer itself
+    KPZ_CUDA(launch_heights(ctx->lat, ctx->g, ctx->col0, 0, L, absolute ? ctx->h00 : nullptr, host_out, ctx->stream));
     KPZ_CUDA(cudaStreamSynchronize(ctx->stream));
+    return settle(ctx);
   }
+  // Bands through the two halves of the staging band, as in kpz_slopes.
+  const size_t row_bytes = (size_t)L * 8;
+  const size_t half = (ctx->io_bytes / 2) / kAlign * kAlign;   // at least two rows
+  const uint32_t band = (uint32_t)std::min<size_t>(L, half / row_bytes);
+  char* buf[2] = {(char*)ctx->io, (char*)ctx->io + half};
+  KPZ_CUDA(io_prepare(ctx));
+  uint32_t b = 0;
+  for (uint32_t j0 = 0; j0 < L; j0 += band, ++b) {
+    const uint32_t nr = std::min(band, L - j0), k = b & 1u;
+    if (b >= 2) KPZ_CUDA(cudaStreamWaitEvent(ctx->stream, ctx->io_ev[2 + k], 0));   // half k read out
+    KPZ_CUDA(launch_heights(ctx->lat, ctx->g, ctx->col0, j0, nr, absolute ? ctx->h00 : nullptr, (int64_t*)buf[k],
+                            ctx->stream));
+    KPZ_CUDA(cudaEventRecord(ctx->io_ev[k], ctx->stream));
+    KPZ_CUDA(cudaStreamWaitEvent(ctx->io_stream, ctx->io_ev[k], 0));
+    KPZ_CUDA(cudaMemcpyAsync((char*)host_out + (size_t)j0 * row_bytes, buf[k], nr * row_bytes, cudaMemcpyDeviceToHost,
+                             ctx->io_stream));
+    KPZ_CUDA(cudaEventRecord(ctx->io_ev[2 + k], ctx->io_stream));
+  }
+  KPZ_CUDA(cudaStreamSynchronize(ctx->io_stream));
   return settle(ctx);
 }
 
@@ -406,6 +463,7 @@ kpz_status kpz_slopes(kpz_ctx* ctx, uint32_t* host_out) {
   size_t half = 0;
   const uint32_t band = io_band_rows(ctx, row_bytes, &half);
   char* buf[2] = {(char*)ctx->io, (char*)ctx->io + half};
+  touch_pages(host_out, (size_t)L * row_bytes);
   KPZ_CUDA(io_prepare(ctx));
   uint32_t b = 0;
   for (uint32_t j0 = 0; j0 < L; j0 += band, ++b) {
@@ -620,6 +678,10 @@ void kpz_free(kpz_ctx* ctx) {
   if (ctx->rsu_scratch) {
     cudaStreamSynchronize(ctx->stream);
     cudaFree(ctx->rsu_scratch);
+  }
+  if (ctx->sums) {
+    cudaStreamSynchronize(ctx->stream);
+    cudaFreeHost(ctx->sums);
   }
   delete ctx;
 }

@@ -6,12 +6,12 @@
 // after start-up.
 // kpz_roughness_static gives them the reduction of kpz_roughness on a lattice
 // they already hold (the pointer kpz_device_lattice returns), with its scratch
-// (column-0 heights and three 64-bit accumulators) in the file-scope array
+// (the bands' partial sums, a ticket and the results) in the file-scope array
 // below instead of memory the library would allocate.
 #include <mutex>
 
 #include "kpz.h"
-#include "kpz_internal.h"
+#include "kpz_observe.h"
 
 using namespace kpz;
 
@@ -19,8 +19,9 @@ namespace {
 
 constexpr uint32_t kMaxL = 131072;  // largest lattice the static scratch serves
 constexpr size_t kAccOffset = (size_t)kMaxL * sizeof(int32_t);  // 256-byte aligned
-// Column-0 heights (kMaxL int32) followed by the three accumulators:
-// 512 KiB + 256 B, held by every GPU that loads the library until exit.
+// Partial sums (at most 24 kMaxL / 32 bytes of the 4 kMaxL) followed by the
+// results and the ticket: 512 KiB + 256 B, held by every GPU that loads the
+// library until exit.
 static __device__ __align__(256) int32_t g_scratch[kMaxL + 64];
 
 constexpr int kMaxDevices = 64;
@@ -50,19 +51,19 @@ extern "C" kpz_status kpz_roughness_static(const void* lattice_dev, uint32_t L, 
     }
     base = g_scratch_addr[dev];
   }
-  int32_t* col0 = static_cast<int32_t*>(base);
-  unsigned long long* acc = reinterpret_cast<unsigned long long*>(static_cast<char*>(base) + kAccOffset);
+  long long* sums = reinterpret_cast<long long*>(static_cast<char*>(base) + kAccOffset);
+  const RoughOut ro{reinterpret_cast<uint32_t*>(sums + 8), sums, nullptr, nullptr};
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   Geometry g{};
   g.L = L;
   g.NR = L / 4;
   g.NB = L / 128;
   g.par = parity & 1u;
-  // launch_roughness zeroes the accumulators before it adds into them.
-  if (launch_roughness(static_cast<const uint32_t*>(lattice_dev), g, col0, acc, st) != cudaSuccess)
+  if (cudaMemsetAsync(ro.ticket, 0, sizeof(*ro.ticket), st) != cudaSuccess ||
+      launch_roughness(static_cast<const uint32_t*>(lattice_dev), g, base, ro, st) != cudaSuccess)
     return KPZ_ECUDA;
   unsigned long long host[3];
-  if (cudaMemcpyAsync(host, acc, sizeof(host), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+  if (cudaMemcpyAsync(host, sums, sizeof(host), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess)
     return KPZ_ECUDA;
   const uint64_t N = (uint64_t)L * L;

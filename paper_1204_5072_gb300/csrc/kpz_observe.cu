@@ -9,8 +9,9 @@
 // then along each row, h(i,j) = h(0,j) + sum_{l<i} sigma_x(l,j); on a valid
 // (curl-free) surface this equals any other path sum.
 #include <algorithm>
+#include <mutex>
 
-#include "kpz_internal.h"
+#include "kpz_observe.h"
 #include "kpz_w2.cuh"
 
 namespace kpz {
@@ -241,98 +242,222 @@ __global__ void __launch_bounds__(kCol0Threads) col0_kernel(const uint32_t* __re
   }
 }
 
-// Work split: warp -> (y4, 8 consecutive storage rows R); lane -> row R + (lane & 7)
-// and segment q = lane >> 3 of kSegs block columns each; a segment's start
-// height is col0 plus the height changes of the segments before it (a scan
-// over the 4 lanes of the row).
-constexpr uint32_t kRowsPerWarp = 8, kSegs = 4;
+// Exact W^2. A band is 32 rows (8 cell rows); a block takes bands by turns and
+// leaves of each the column-0 height change D over it and the sums S1, S2 of
+// its heights relative to its first site; the last block to finish chains the
+// bands (band k starts at the sum of the D above it). One launch: no memset,
+// no column-0 kernel, no atomics on the sums.
+//
+// Warp w of a block takes the rows y4 = w & 3 of the band's cell rows (lane &
+// 7) and the segments 4 (w >> 2) + (lane >> 3) of 8 (a lane reads 8
+// consecutive cell rows' words with its neighbours: full 32-byte sectors).
+// Along a segment a run of 8 sites (kpz_w2.cuh) that starts at height h has
+// the height sum m = 8h + A1 and the square sum (m^2 + V) / 8 with V = 8 A2 -
+// A1^2, so a run costs one table entry {8D << 16 | V, A1}, whose first word is
+// also the running height: m from one shift-add, m and m^2 accumulated.
+// The per-run unpacking of D, A1, A2 and the three-term update it replaces
+// took 2.57 instructions a site.
+constexpr uint32_t kBandRows = 32, kBandCells = kBandRows / 4u, kBandThreads = 256, kSegs = 8;
+constexpr size_t kRunTab2Bytes = 256u * 32u * sizeof(uint2);   // one copy per lane
 
-__global__ void __launch_bounds__(256) roughness_kernel(const uint32_t* __restrict__ lat, Geometry g,
-                                                        const int32_t* __restrict__ col0,
-                                                        unsigned long long* __restrict__ acc) {
-  __shared__ uint32_t tab[w2::kRunTableWords];
-  w2::fill_run_table(tab);
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t* tl = tab + lane;
-  const uint32_t gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const uint32_t y4 = gw & 3u, R = (gw >> 2) * kRowsPerWarp + (lane & (kRowsPerWarp - 1u));
-  const uint32_t q = lane / kRowsPerWarp;
-  const uint32_t seg = (g.NB + kSegs - 1u) / kSegs;               // block columns per segment
-  const uint32_t K0 = q * seg, K1 = min(g.NB, K0 + seg);
-  const bool active = R < g.NR && K0 < K1;
-  long long s1 = 0, s2 = 0, dH = 0;   // relative to the segment's first site
-  if (active) {
-    uint32_t P[4], Pn[4];
-#pragma unroll
-    for (uint32_t x4 = 0; x4 < 4; ++x4) {
-      P[x4] = __ldcg(lat + g.word(K0, plane(y4, x4), R));
-      Pn[x4] = __ldcg(lat + g.word((K0 + 1u) & (g.NB - 1u), plane(y4, x4), R));
-    }
-    const uint32_t j = 4u * R + y4;
-    for (uint32_t K = K0; K < K1; ++K) {
-      uint32_t Pnn[4];   // two blocks ahead
-      const uint32_t K2 = (K + 2u) & (g.NB - 1u);
-#pragma unroll
-      for (uint32_t x4 = 0; x4 < 4; ++x4) Pnn[x4] = __ldcg(lat + g.word(K2, plane(y4, x4), R));
-      uint32_t S[4];
-      w2::sigma_x_planes(P, Pn[0] & 1u, j, g.par, S);
-      int32_t h, a1, a2;
-      w2::block_sums(tl, S, h, a1, a2);
-      s1 += 128 * dH + a1;
-      s2 += 128 * dH * dH + 2 * dH * (long long)a1 + (long long)a2;
-      dH += h;
-#pragma unroll
-      for (uint32_t x4 = 0; x4 < 4; ++x4) { P[x4] = Pn[x4]; Pn[x4] = Pnn[x4]; }
-    }
+// Table entry of run byte b (kpz_w2.cuh): {8 D << 16 | V, A1}.
+__device__ __forceinline__ uint2 run_entry2(uint32_t b) {
+  const uint32_t e = w2::run_entry(b);
+  const int32_t A2 = (int32_t)(e & 0xFFu), A1 = (int32_t)((e >> 8) & 0xFFu) - 28, D = (int32_t)(e >> 16) - 8;
+  return make_uint2((uint32_t)(8 * D * 65536 + 8 * A2 - A1 * A1), (uint32_t)A1);
+}
+
+__global__ void __launch_bounds__(kBandThreads, 3) roughness_kernel(const uint32_t* __restrict__ lat, Geometry g,
+                                                                    long long* __restrict__ part, RoughOut out) {
+  extern __shared__ __align__(16) uint2 tab2[];   // [256][32]
+  __shared__ long long seg_s1[kBandRows][kSegs], seg_s2[kBandRows][kSegs];
+  __shared__ int seg_dh[kBandRows][kSegs];
+  __shared__ bool last;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  {
+    const uint2 e = run_entry2(threadIdx.x);   // kBandThreads = 256 entries; a warp writes its 32 side by side
+#pragma unroll 8
+    for (uint32_t i = 0; i < 32u; ++i)
+      tab2[(warp * 32u + i) * 32u + lane] =
+          make_uint2(__shfl_sync(0xffffffffu, e.x, i), __shfl_sync(0xffffffffu, e.y, i));
   }
-  // Start height of this segment: col0[j] + height changes of the row's earlier segments.
-  long long pre = dH;
+  __syncthreads();
+  const char* tl = reinterpret_cast<const char*>(tab2);
+  const uint32_t lane8 = lane * 8u;
+  const uint32_t y4 = warp & 3u, rr = lane & 7u, q = (warp >> 2) * 4u + (lane >> 3);
+  const uint32_t seg = (g.NB + kSegs - 1u) / kSegs, K0 = min(g.NB, q * seg), K1 = min(g.NB, K0 + seg);
+  const uint32_t nb = g.L / kBandRows;
+  for (uint32_t band = blockIdx.x; band < nb; band += gridDim.x) {
+    const uint32_t R = band * kBandCells + rr, j = 4u * R + y4;
+    long long s1 = 0, s2 = 0;   // relative to the segment's first site
+    int dH = 0;
+    if (K0 < K1) {
+      uint32_t Pl[4], Pn[4];
 #pragma unroll
-  for (uint32_t d = kRowsPerWarp; d < 32u; d <<= 1) {
-    const long long v = __shfl_up_sync(0xffffffffu, pre, d);
-    if (lane >= d) pre += v;
+      for (uint32_t x4 = 0; x4 < 4; ++x4) {
+        Pl[x4] = __ldcg(lat + g.word(K0, plane(y4, x4), R));
+        Pn[x4] = __ldcg(lat + g.word((K0 + 1u) & (g.NB - 1u), plane(y4, x4), R));
+      }
+      for (uint32_t K = K0; K < K1; ++K) {
+        uint32_t Pnn[4];   // two blocks ahead
+        const uint32_t K2 = (K + 2u) & (g.NB - 1u);
+#pragma unroll
+        for (uint32_t x4 = 0; x4 < 4; ++x4) Pnn[x4] = __ldcg(lat + g.word(K2, plane(y4, x4), R));
+        uint32_t S[4], u[4];
+        w2::sigma_x_planes(Pl, Pn[0] & 1u, j, g.par, S);
+        w2::run_bytes(S, u);
+        int32_t run = 0, sm = 0, sq = 0;
+#pragma unroll
+        for (uint32_t m = 0; m < 4; ++m)
+#pragma unroll
+          for (uint32_t k = 0; k < 4; ++k) {
+            const uint32_t v = m == 0u ? u[k] << 8 : u[k] >> (8u * m - 8u);
+            const uint2 e = *reinterpret_cast<const uint2*>(tl + ((v & 0xFF00u) | lane8));
+            const int32_t mm = (run >> 16) + (int32_t)e.y;
+            sm += mm;
+            sq += mm * mm;
+            run += (int32_t)e.x;
+          }
+        const int32_t a2 = (sq + (run & 0xFFFF)) >> 3;
+        s1 += 128ll * dH + sm;
+        s2 += (long long)dH * (128ll * dH + 2ll * sm) + a2;
+        dH += run >> 19;
+#pragma unroll
+        for (uint32_t x4 = 0; x4 < 4; ++x4) { Pl[x4] = Pn[x4]; Pn[x4] = Pnn[x4]; }
+      }
+    }
+    seg_s1[4u * rr + y4][q] = s1;
+    seg_s2[4u * rr + y4][q] = s2;
+    seg_dh[4u * rr + y4][q] = dH;
+    __syncthreads();
+    if (warp == 0u) {   // lane = row of the band
+      const uint32_t jr = band * kBandRows + lane;
+      const uint32_t b0 = site_bit(lat, g, 0u, jr), b1 = site_bit(lat, g, 0u, (jr + 1u) & (g.L - 1u));
+      const uint32_t upm = __ballot_sync(0xffffffffu, (b0 ^ b1) == ((jr + g.par) & 1u));   // sigma_y(0, jr) = +1
+      long long H = 2 * (int)__popc(upm & ((1u << lane) - 1u)) - (int)lane, t1 = 0, t2 = 0;
+      for (uint32_t k = 0; k < kSegs; ++k) {
+        const long long n = 128ll * (min(g.NB, (k + 1u) * seg) - min(g.NB, k * seg));
+        const long long a = seg_s1[lane][k];
+        t1 += n * H + a;
+        t2 += H * (n * H + 2 * a) + seg_s2[lane][k];
+        H += seg_dh[lane][k];
+      }
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) {
+        t1 += __shfl_xor_sync(0xffffffffu, t1, off);
+        t2 += __shfl_xor_sync(0xffffffffu, t2, off);
+      }
+      if (lane == 0u) {
+        part[3u * band] = 2 * (int)__popc(upm) - 32;
+        part[3u * band + 1u] = t1;
+        part[3u * band + 2u] = t2;
+      }
+    }
+    __syncthreads();
   }
-  long long t1 = 0;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(out.ticket, 1u) == gridDim.x - 1u;
+  }
+  __syncthreads();
+  if (!last) return;
+  // Chain the bands: thread t takes bands [t per, (t + 1) per), at most 32; a
+  // band's sum of squares is below 2^57, so a thread's fits 64 bits, and the
+  // block adds the threads' 32-bit halves.
+  __threadfence();
+  __shared__ long long scan[kBandThreads];
+  const uint32_t per = (nb + kBandThreads - 1u) / kBandThreads, k0 = min(nb, threadIdx.x * per), k1 = min(nb, k0 + per);
+  long long d = 0;
+  for (uint32_t k = k0; k < k1; ++k) d += __ldcg(part + 3u * k);
+  scan[threadIdx.x] = d;
+  __syncthreads();
+  for (uint32_t off = 1; off < kBandThreads; off <<= 1) {   // inclusive scan
+    const long long v = threadIdx.x >= off ? scan[threadIdx.x - off] : 0;
+    __syncthreads();
+    scan[threadIdx.x] += v;
+    __syncthreads();
+  }
+  long long H = scan[threadIdx.x] - d, t1 = 0;
   unsigned long long t2 = 0;
-  if (active) {
-    const long long H0 = (long long)col0[4u * R + y4] + (pre - dH);
-    const long long n = 128ll * (K1 - K0);
-    t1 = n * H0 + s1;
-    t2 = (unsigned long long)(n * H0 * H0 + 2 * H0 * s1 + s2);
+  const long long n = (long long)kBandRows * g.L;
+  for (uint32_t k = k0; k < k1; ++k) {
+    const long long a = __ldcg(part + 3u * k + 1u);
+    t1 += n * H + a;
+    t2 += (unsigned long long)(H * (n * H + 2 * a) + __ldcg(part + 3u * k + 2u));
+    H += __ldcg(part + 3u * k);
   }
+  unsigned long long lo = t2 & 0xffffffffull, hi = t2 >> 32;
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
     t1 += __shfl_xor_sync(0xffffffffu, t1, off);
-    t2 += __shfl_xor_sync(0xffffffffu, t2, off);
+    lo += __shfl_xor_sync(0xffffffffu, lo, off);
+    hi += __shfl_xor_sync(0xffffffffu, hi, off);
   }
-  if (lane == 0 && (t1 != 0 || t2 != 0)) {
-    atomicAdd(&acc[0], (unsigned long long)t1);
-    const unsigned long long old = atomicAdd(&acc[1], t2);
-    if (old + t2 < old) atomicAdd(&acc[2], 1ull);
+  __syncthreads();
+  if (lane == 0u) { scan[warp] = t1; scan[8u + warp] = (long long)lo; scan[16u + warp] = (long long)hi; }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    long long a = 0;
+    unsigned long long l = 0, h = 0;
+    for (uint32_t k = 0; k < kBandThreads / 32u; ++k) {
+      a += scan[k];
+      l += (unsigned long long)scan[8u + k];
+      h += (unsigned long long)scan[16u + k];
+    }
+    const unsigned long long s2lo = (h << 32) + l, s2hi = (h >> 32) + (s2lo < l ? 1ull : 0ull);
+    *out.ticket = 0u;
+    out.sums[0] = a;
+    out.sums[1] = (long long)s2lo;
+    out.sums[2] = (long long)s2hi;
+    if (out.h00) out.sums[3] = *(volatile const long long*)out.h00;
+    if (out.err) out.sums[4] = *(volatile const uint32_t*)out.err;
+    __threadfence_system();
   }
 }
 
-__global__ void heights_kernel(const uint32_t* __restrict__ lat, Geometry g,
-                               const int32_t* __restrict__ col0, uint32_t j0, uint32_t nrows,
-                               const unsigned long long* __restrict__ h00, int64_t* __restrict__ out) {
-  const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
+// Heights of the rows of a band, one warp per row and segment of kHeightSeg
+// block columns: the segment's start height is col0 plus the height changes of
+// the block columns before it (a lane each), then lane c writes the four
+// sites of cell c, 32 bytes beside its neighbours'. One thread per row with
+// 8-byte stores a row apart took 0.3 ms for a 64-row band at L = 2048.
+constexpr uint32_t kHeightSeg = 4;
+
+__global__ void __launch_bounds__(256) heights_kernel(const uint32_t* __restrict__ lat, Geometry g,
+                                                      const int32_t* __restrict__ col0, uint32_t j0, uint32_t nrows,
+                                                      const unsigned long long* __restrict__ h00,
+                                                      int64_t* __restrict__ out) {
+  const uint32_t lane = threadIdx.x & 31u, gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const uint32_t nseg = (g.NB + kHeightSeg - 1u) / kHeightSeg, r = gw / nseg, q = gw - r * nseg;
   if (r >= nrows) return;
-  const uint32_t j = j0 + r, R = j >> 2, y4 = j & 3u;
-  int64_t h = col0[j] + (h00 ? (int64_t)*h00 : 0);
-  int64_t* o = out + (size_t)r * g.L;
-  for (uint32_t K = 0; K < g.NB; ++K) {
+  const uint32_t j = j0 + r, R = j >> 2, y4 = j & 3u, K0 = q * kHeightSeg, K1 = min(g.NB, K0 + kHeightSeg);
+  auto steps = [&](uint32_t K, uint32_t (&S)[4]) {
     uint32_t P[4];
 #pragma unroll
-    for (uint32_t x4 = 0; x4 < 4; ++x4) P[x4] = lat[g.word(K, plane(y4, x4), R)];
-    const uint32_t nxt = site_bit(lat, g, (128u * K + 128u) & (g.L - 1u), j);
+    for (uint32_t x4 = 0; x4 < 4; ++x4) P[x4] = __ldg(lat + g.word(K, plane(y4, x4), R));
+    w2::sigma_x_planes(P, __ldg(lat + g.word((K + 1u) & (g.NB - 1u), plane(y4, 0), R)) & 1u, j, g.par, S);
+  };
+  int before = 0;
+  for (uint32_t K = lane; K < K0; K += 32u) {
     uint32_t S[4];
-    w2::sigma_x_planes(P, nxt, j, g.par, S);
-    for (uint32_t c = 0; c < 32; ++c)
+    steps(K, S);
+    before += 2 * (__popc(S[0]) + __popc(S[1]) + __popc(S[2]) + __popc(S[3])) - 128;
+  }
+  before = __reduce_add_sync(0xffffffffu, before);
+  int64_t H = (int64_t)col0[j] + (h00 ? (int64_t)*h00 : 0) + before;
+  int64_t* o = out + (size_t)r * g.L + 4u * lane;
+  const uint32_t below = (1u << lane) - 1u;
+  for (uint32_t K = K0; K < K1; ++K) {
+    uint32_t S[4];
+    steps(K, S);
+    const int up = __popc(S[0] & below) + __popc(S[1] & below) + __popc(S[2] & below) + __popc(S[3] & below);
+    int64_t h[4];
+    h[0] = H + 2 * up - 4 * (int)lane;
 #pragma unroll
-      for (uint32_t x4 = 0; x4 < 4; ++x4) {
-        o[128u * K + 4u * c + x4] = h;
-        h += 2 * (int64_t)((S[x4] >> c) & 1u) - 1;
-      }
+    for (int x = 0; x < 3; ++x) h[x + 1] = h[x] + 2 * (int)((S[x] >> lane) & 1u) - 1;
+    longlong2* v = reinterpret_cast<longlong2*>(o + 128u * K);
+    v[0] = make_longlong2(h[0], h[1]);
+    v[1] = make_longlong2(h[2], h[3]);
+    H += 2 * (__popc(S[0]) + __popc(S[1]) + __popc(S[2]) + __popc(S[3])) - 128;
   }
 }
 
@@ -376,15 +501,30 @@ cudaError_t launch_col0(const uint32_t* lat, Geometry g, int32_t* col0, cudaStre
   return cudaGetLastError();
 }
 
-cudaError_t launch_roughness(const uint32_t* lat, Geometry g, int32_t* col0,
-                             unsigned long long* acc, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(acc, 0, 3 * sizeof(unsigned long long), st);
+cudaError_t launch_roughness(const uint32_t* lat, Geometry g, void* scratch, const RoughOut& out, cudaStream_t st) {
+  constexpr int kMaxDev = 64;
+  static std::mutex mu;
+  static uint32_t blocks[kMaxDev] = {};   // resident blocks of the device
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  col0_kernel<<<1, std::min(kCol0Threads, g.L / 32u), 0, st>>>(lat, g, col0);
-  count_launch();
-  const uint32_t warps = 4u * ((g.NR + kRowsPerWarp - 1u) / kRowsPerWarp);
-  const uint32_t wpc = 8;
-  roughness_kernel<<<(warps + wpc - 1) / wpc, wpc * 32, 0, st>>>(lat, g, col0, acc);
+  uint32_t room = 0;
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    if (dev < kMaxDev) room = blocks[dev];
+    if (!room) {
+      int per_sm = 0, sms = 0;
+      e = cudaFuncSetAttribute(roughness_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRunTab2Bytes);
+      if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, roughness_kernel, (int)kBandThreads, kRunTab2Bytes);
+      if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+      if (e != cudaSuccess) return e;
+      room = (uint32_t)std::max(per_sm, 1) * (uint32_t)std::max(sms, 1);
+      if (dev < kMaxDev) blocks[dev] = room;
+    }
+  }
+  roughness_kernel<<<std::min(room, g.L / kBandRows), kBandThreads, kRunTab2Bytes, st>>>(
+      lat, g, static_cast<long long*>(scratch), out);
   count_launch();
   return cudaGetLastError();
 }
@@ -392,7 +532,8 @@ cudaError_t launch_roughness(const uint32_t* lat, Geometry g, int32_t* col0,
 cudaError_t launch_heights(const uint32_t* lat, Geometry g, const int32_t* col0, uint32_t j0,
                            uint32_t nrows, const unsigned long long* h00, int64_t* out,
                            cudaStream_t st) {
-  heights_kernel<<<(nrows + 127) / 128, 128, 0, st>>>(lat, g, col0, j0, nrows, h00, out);
+  const uint32_t warps = nrows * ((g.NB + kHeightSeg - 1u) / kHeightSeg);
+  heights_kernel<<<(warps + 7u) / 8u, 256, 0, st>>>(lat, g, col0, j0, nrows, h00, out);
   count_launch();
   return cudaGetLastError();
 }
