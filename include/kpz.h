@@ -66,9 +66,9 @@ typedef struct {
                              trajectories; 128 x 256 needs L >= 256               */
     uint32_t run;         /* tiles per work item: the resident warps take runs of
                              `run` tiles of one tile row from a queue (power of two
-                             <= L/128; 0 = min(8, L/128) below L = 65536, L/4096
-                             from there); execution only, it does not change the
-                             result                                                */
+                             <= L/128; 0 = as many as leave 8192 runs, at least 1,
+                             at most L/4096); execution only, it does not change
+                             the result                                            */
     uint32_t warps_per_cta; /* 1..8; 0 = 4 for 128-row tiles from L = 65536, else 8;
                              execution only. With run and warps_per_cta both 0,
                              lattices of 128 x 128 tiles and 4 x 4 cells up to

@@ -284,15 +284,20 @@ kpz_status kpz_init(kpz_ctx** out, uint32_t L, double p, double q, uint64_t seed
   ctx->decomposition = o.decomposition;
   ctx->cell = o.cell ? o.cell : 4u;
   ctx->colour_m = o.colour_sparsity ? o.colour_sparsity : 3u;
-  // Default schedule, measured on GB300 at p = 1 (results do not depend on
-  // it): runs of 8 tiles and 8-warp CTAs up to 256 tiles per row; from 512
-  // tiles per row runs of ntx/32 tiles, which halve the per-run cost (window
-  // prologue, start copy, edge write-backs) while about 4.5 (L = 2^16) or 9
-  // (L = 2^17) runs per resident warp keep the last wave short, with 4-warp
-  // CTAs for 128-row tiles. L = 2^16: 0.4765 ms per sweep against 0.4954 ms;
-  // L = 2^17: 1.827 ms against 1.920 ms.
+  // Default schedule of the work-queue sweep, measured on GB300 (results do not
+  // depend on it): about 8192 runs, two to three for each resident warp, but
+  // none longer than 1/32 of a tile row, which keeps the last wave short. A
+  // longer run saves window prologues, start copies and edge write-backs, a
+  // shorter one fills the GPU: us per sweep at p = 1 / 0.95 with runs of 1, 2,
+  // 4, 8 tiles, L = 8192: 24 / 37, 25 / 50, 30 / -, 37 / 128; L = 16384: 55 / 107,
+  // 47 / 102, 63 / 115, 62 / 200; L = 32768: 178 / -, 155 / -, 142 / 349, 138 /
+  // 340; L = 65536: runs of 8 482 / 1270, 16 465 / 1270. From L = 65536 4-warp
+  // CTAs for 128-row tiles (465 against 485 at p = 1), below it 8-warp ones.
   const bool wide = ntx >= 512u;
-  ctx->run = o.run ? o.run : (wide ? ntx / 32u : std::min(8u, ntx));   // tiles per work-queue chunk
+  const uint32_t tiles = ntx * (L / ctx->tile_y);
+  uint32_t auto_run = 1u;
+  while (2u * auto_run <= std::min(tiles / 8192u, ntx / 32u)) auto_run *= 2u;
+  ctx->run = o.run ? o.run : auto_run;   // tiles per work-queue chunk
   ctx->wpc = o.warps_per_cta ? o.warps_per_cta : (wide && ctx->tile_y == kTile ? 4u : 8u);
   ctx->stream = (cudaStream_t)o.stream;
   if (o.dev_buf) {

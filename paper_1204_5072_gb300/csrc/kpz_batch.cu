@@ -19,6 +19,7 @@
 #include <cmath>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "kpz.h"
@@ -41,7 +42,7 @@ struct Real {                   // one realisation, sorted by run length, longes
   SweepParams P;                // lattice, geometry, rates, key, tiles per run
   uint32_t n_items;             // tile runs per sweep
   uint32_t nb;                  // W^2 bands per sample (L/128 rows of 128)
-  uint32_t general;             // rates other than p = 1, q = 0
+  uint32_t mode;                // run::Mode of the rates
 };
 
 struct Plan {
@@ -165,7 +166,7 @@ __device__ void band_sums(const SweepParams& P, const uint32_t* tl, uint32_t k, 
 // cp.async writes, so every warp's slot must start on a 16-byte boundary.
 template <int CR>
 struct alignas(16) WarpSlot {
-  run::WarpStage<CR> stage;
+  std::conditional_t<CR == 1, run::WarpStageMem<CR>, run::WarpStage<CR>> stage;
   SweepParams P;
   uint4 rk[kPhiloxRounds / 2];   // Philox round keys of the item's realisation
 };
@@ -178,6 +179,8 @@ __global__ void __launch_bounds__(256, 2) batch_kernel(const __grid_constant__ P
   extern __shared__ __align__(16) unsigned char smem_raw[];
   WarpSlot<CR>& ws = reinterpret_cast<WarpSlot<CR>*>(smem_raw)[threadIdx.x >> 5];
   __shared__ uint32_t tab[w2::kRunTableWords];   // W^2 run table (kpz_w2.cuh)
+  __shared__ tilemem::QuadTab qtab;
+  if (threadIdx.x < 4u) tilemem::fill_quad_tab(qtab, threadIdx.x);
   w2::fill_run_table(tab);
   const uint32_t lane = threadIdx.x & 31u;
   for (;;) {
@@ -226,7 +229,7 @@ __global__ void __launch_bounds__(256, 2) batch_kernel(const __grid_constant__ P
       uint32_t* dst = reinterpret_cast<uint32_t*>(&ws.P);
       for (uint32_t w = lane; w < sizeof(SweepParams) / 4; w += 32u) dst[w] = src[w];
     }
-    const uint32_t general = re->general;
+    const uint32_t mode = re->mode;
     __syncwarp();
     // Its Philox round keys, read by the tile code from shared memory.
     if (lane < kPhiloxRounds / 2) {
@@ -257,8 +260,13 @@ __global__ void __launch_bounds__(256, 2) batch_kernel(const __grid_constant__ P
       // Device layer: this sweep's random tile origin (Sec. 3).
       const uint4 o = philox(kTagOrigin << 28, 0u, g, ws.P.sample, ws.P.k0, ws.P.k1);
       const uint32_t L = ws.P.g.L, ox = o.x & (L - 1u), oy = o.y & (L - 1u);
-      if (general) run::sweep_run<true, CR, true, true>(ws.P, ws.stage, ws.rk, lane, g, ox, oy, ty, tx0, ws.P.run);
-      else         run::sweep_run<false, CR, true, true>(ws.P, ws.stage, ws.rk, lane, g, ox, oy, ty, tx0, ws.P.run);
+      auto sweep = [&](auto m) {
+        run::sweep_run<decltype(m)::value, CR, true, true>(ws.P, ws.stage, ws.rk, qtab, lane, g, ox, oy, ty, tx0, ws.P.run);
+      };
+      using std::integral_constant;
+      if (CR == 1 && mode == run::kInner) sweep(integral_constant<int, run::kInner>{});
+      else if (mode != run::kGrowth)      sweep(integral_constant<int, run::kEdgeRate>{});
+      else                                sweep(integral_constant<int, run::kGrowth>{});
     }
     __threadfence();
     __syncwarp();
@@ -467,7 +475,7 @@ kpz_status prepare(kpz_batch* b, const std::vector<uint64_t>* cap_T) {
     set_philox_key(r.P, s.seed);
     r.P.sample = s.sample;
     r.P.h00 = m.h00 + i;
-    r.general = !(r.P.Tp == 65536u && r.P.Tq == 0u);
+    r.mode = (uint32_t)run::mode_of(r.P);
   }
   // A probe replaces the run lengths by shorter ones (capped copies of the specs).
   std::vector<kpz_spec> saved;

@@ -73,10 +73,6 @@ cudaError_t launch_import_packed(uint32_t* lat, Geometry g, uint32_t j0, uint32_
                                  const uint32_t* packed, uint32_t* hcar, int32_t* hcol,
                                  cudaStream_t st);
 
-// Exact height sums, eq. Wdef: col0[L] (int32) and acc[3] (S1, S2 lo, S2 hi)
-// are scratch that the caller provides.
-cudaError_t launch_roughness(const uint32_t* lat, Geometry g, int32_t* col0,
-                             unsigned long long* acc, cudaStream_t st);
 // Heights of rows [j0, j0 + nrows) into out[(j - j0) * L + i], gauge h(0,0) = 0
 // plus *h00 when h00 is not null; needs col0 filled by launch_col0.
 cudaError_t launch_col0(const uint32_t* lat, Geometry g, int32_t* col0, cudaStream_t st);

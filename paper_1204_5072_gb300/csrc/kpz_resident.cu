@@ -30,13 +30,11 @@
 #include <algorithm>
 
 #include "kpz_resident.h"
-#include "kpz_rounds.cuh"
 #include "kpz_tilemem.cuh"
 
 namespace kpz {
 namespace {
 
-using rounds::TileCtx;
 using tilemem::QuadTab;
 using tilemem::TileMem;
 
@@ -45,13 +43,15 @@ using tilemem::TileMem;
 // round and the outcome of its four deep numbers against both thresholds: bit
 // 7 - r % 8 of byte k of deep[r / 8].x (.y) is set when the k-th tie of the row
 // in round r is accepted as a minimum (maximum) (streams as in
-// kpz_rounds.cuh). setw[0]: the quadrant sets, [1], [2]: the sweep's origin.
+// kpz_rounds.cuh), the rounds' quadrant offsets (tilemem::QuadTab) and the
+// sweep's origin.
 template <bool kGeneral>
 struct TileRand {
   uint4 pos[kRounds / 2][32];
   uint4 acc[kGeneral ? kRounds : 1][kGeneral ? 32 : 1];
   uint2 deep[kGeneral ? 2 : 1][kGeneral ? 32 : 1];
-  uint32_t setw[4];
+  uint4 at[kRounds], sh[kRounds];
+  uint32_t origin[4];
 };
 
 // Four Philox blocks (counter words c0[i], c1, c2, c3) at once: ten rounds of
@@ -79,26 +79,25 @@ __device__ __forceinline__ void philox4(const uint32_t (&ctr)[4], uint32_t c1, u
   for (int i = 0; i < 4; ++i) out[i] = make_uint4(x[i], y[i], z[i], w[i]);
 }
 
-// Four 12-bit numbers (the 16-bit halves of lo, hi) against a threshold t:
-// t + 0x7FFF - h has its top bit set exactly when h < t.
-__device__ __forceinline__ uint32_t deep_below(uint32_t lo, uint32_t hi, uint32_t t) {
-  const uint32_t c = ((t & 0xFFFu) + 0x7FFFu) * 0x10001u;
-  return __byte_perm(c - (lo & 0x0FFF0FFFu), c - (hi & 0x0FFF0FFFu), 0x7531) & 0x80808080u;
-}
-
 // Draws part `part` of `parts` (1 or 2) of a tile's blocks.
 template <bool kGeneral>
-__device__ __forceinline__ void draw_tile(const SweepParams& P, TileRand<kGeneral>& B, uint32_t tid, uint32_t s,
-                                          uint32_t lane, uint32_t part, uint32_t parts) {
+__device__ __forceinline__ void draw_tile(const SweepParams& P, const QuadTab& tab, TileRand<kGeneral>& B,
+                                          uint32_t tid, uint32_t s, uint32_t lane, uint32_t part, uint32_t parts) {
   if (part == 0u) {
     const uint32_t w = philox(kTagSet << 28, tid, s, P.sample, P.k0, P.k1).x;
     const uint4 o = philox(kTagOrigin << 28, 0u, s, P.sample, P.k0, P.k1);
-    if (lane == 0u) { B.setw[0] = w; B.setw[1] = o.x & (P.g.L - 1u); B.setw[2] = o.y & (P.g.L - 1u); }
+    if (lane < kRounds) {
+      B.at[lane] = tab.at[(w >> (2u * lane)) & 3u];
+      B.sh[lane] = tab.sh[(w >> (2u * lane)) & 3u];
+    }
+    if (lane == 0u) { B.origin[0] = o.x & (P.g.L - 1u); B.origin[1] = o.y & (P.g.L - 1u); }
   }
   uint4 o[4];
   if constexpr (kGeneral) {
     const uint32_t n = (kRounds / 2) / parts;
     uint32_t dp = 0u, dq = 0u;   // outcomes of four round pairs
+    const uint32_t cp = tilemem::Rates<true>::deep_const(P.Tp), cq = tilemem::Rates<true>::deep_const(P.Tq);
+    auto below = [](uint32_t lo, uint32_t hi, uint32_t c) { return tilemem::deep_below(lo, hi, c, ~0u) & 0x80808080u; };
 #pragma unroll 1
     for (uint32_t rp = part * n; rp < part * n + n; ++rp) {
       const uint32_t c[4] = {(kTagPos << 28) | (lane << 3) | rp, (kTagAcc << 28) | (lane << 4) | (2u * rp),
@@ -108,8 +107,8 @@ __device__ __forceinline__ void draw_tile(const SweepParams& P, TileRand<kGenera
       B.acc[2u * rp][lane] = o[1];
       B.acc[2u * rp + 1u][lane] = o[2];
       const uint32_t j = 2u * (rp & 3u);
-      dp |= (deep_below(o[3].x, o[3].y, P.Tp) >> j) | (deep_below(o[3].z, o[3].w, P.Tp) >> (j + 1u));
-      dq |= (deep_below(o[3].x, o[3].y, P.Tq) >> j) | (deep_below(o[3].z, o[3].w, P.Tq) >> (j + 1u));
+      dp |= (below(o[3].x, o[3].y, cp) >> j) | (below(o[3].z, o[3].w, cp) >> (j + 1u));
+      dq |= (below(o[3].x, o[3].y, cq) >> j) | (below(o[3].z, o[3].w, cq) >> (j + 1u));
       if ((rp & 3u) == 3u) {
         B.deep[rp >> 2][lane] = make_uint2(dp, dq);
         dp = dq = 0u;
@@ -128,104 +127,43 @@ __device__ __forceinline__ void draw_tile(const SweepParams& P, TileRand<kGenera
   }
 }
 
-// Acceptance of a general-rate round from the drawn blocks (the rule of
-// rounds::one_round): the candidates' top four bits against their threshold
-// (Tp's bits for a minimum, Tq's for a maximum) by a majority chain, ties by
-// the low twelve bits. No votes: the numbers are there already.
-struct Rates {
-  uint32_t dpm, dqm, pall, qall, bp[4], bq[4];
-  __device__ __forceinline__ explicit Rates(const SweepParams& P) {
-    dpm = (P.Tp != 0u && P.Tp < 65536u) ? ~0u : 0u;
-    dqm = (P.Tq != 0u && P.Tq < 65536u) ? ~0u : 0u;
-    pall = (P.Tp >> 16) ? ~0u : 0u;
-    qall = (P.Tq >> 16) ? ~0u : 0u;
-#pragma unroll
-    for (uint32_t n = 0; n < 4u; ++n) {
-      bp[n] = 0u - ((P.Tp >> (15u - n)) & 1u);
-      bq[n] = 0u - ((P.Tq >> (15u - n)) & 1u);
-    }
-  }
-};
-// All ones where the top bit of byte k of w is set.
-template <int k>
-__device__ __forceinline__ uint32_t byte_mask(uint32_t w) {
-  uint32_t r;
-  asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r) : "r"(w), "n"(0x8888 + 0x1111 * k));
-  return r;
-}
-__device__ __forceinline__ uint32_t accept_cells(const SweepParams& P, const Rates& R, const TileCtx& tc, const uint4& A,
-                                                 const uint2& W, uint32_t lane, uint32_t r, uint32_t up, uint32_t uq) {
-  const uint32_t dm = (up & R.dpm) | (uq & R.dqm);   // candidates that need random bits
-  const uint32_t w[4] = {A.x, A.y, A.z, A.w};
-  uint32_t b[4];
-#pragma unroll
-  for (uint32_t n = 0; n < 4u; ++n) b[n] = (up & R.bp[n]) | (~up & R.bq[n]);
-  uint32_t lt = 0u;
-#pragma unroll
-  for (int n = 3; n >= 0; --n) lt = (~w[n] & lt) | (~w[n] & b[n]) | (lt & b[n]);
-  const uint32_t tie = (dm & ~(w[0] ^ b[0]) & ~(w[1] ^ b[1])) & (~(w[2] ^ b[2]) & ~(w[3] ^ b[3]));
-  uint32_t acc = (up & R.pall) | (uq & R.qall) | (lt & dm);
-  // The k-th tie from below takes the k-th outcome.
-  const uint32_t g0 = (up & byte_mask<0>(W.x)) | (~up & byte_mask<0>(W.y));
-  const uint32_t g1 = (up & byte_mask<1>(W.x)) | (~up & byte_mask<1>(W.y));
-  const uint32_t g2 = (up & byte_mask<2>(W.x)) | (~up & byte_mask<2>(W.y));
-  const uint32_t g3 = (up & byte_mask<3>(W.x)) | (~up & byte_mask<3>(W.y));
-  const uint32_t m1 = tie & (tie - 1u), m2 = m1 & (m1 - 1u), m3 = m2 & (m2 - 1u), m4 = m3 & (m3 - 1u);
-  acc |= (tie & ~m1 & g0) | (m1 & ~m2 & g1) | (m2 & ~m3 & g2) | (m3 & ~m4 & g3);
-  if (m4 != 0u) {   // more than four ties in a row: the overflow blocks of the round
-    uint4 X = make_uint4(0u, 0u, 0u, 0u);
-    uint32_t m = m4;
-    for (uint32_t k = 0u; m != 0u; ++k) {
-      const uint32_t bit = m & (0u - m);
-      m ^= bit;
-      if ((k & 7u) == 0u)
-        X = philox((kTagDeep << 28) | (lane << 8) | (r << 3) | (1u + (k >> 3)), tc.tid, tc.s, P.sample, P.k0, P.k1);
-      const uint32_t x = (k & 4u) ? ((k & 2u) ? X.w : X.z) : ((k & 2u) ? X.y : X.x);
-      const uint32_t h = ((k & 1u) ? (x >> 16) : x) & 0xFFFu;
-      acc |= (h < (((bit & up) ? P.Tp : P.Tq) & 0xFFFu)) ? bit : 0u;
-    }
-  }
-  return acc;
-}
-
 // The 16 single-hit rounds of the tile in m from its drawn numbers. The
 // offsets and numbers of a round are loaded one round ahead, so its chain is
 // quadrant in, logic, quadrant out.
 template <bool kGeneral, int kPar, bool kTrack>
-__device__ __forceinline__ int rounds_from(TileMem& m, const QuadTab& tab, uint32_t ghost, const SweepParams& P,
-                                           const TileCtx& tc, const tilemem::Origin& og, const TileRand<kGeneral>& B,
-                                           uint32_t lane) {
-  char* base = reinterpret_cast<char*>(&m) + lane * 8u;
+__device__ __forceinline__ int rounds_from(TileMem& m, const QuadTab& tab, const SweepParams& P, uint32_t tid, uint32_t s,
+                                           const tilemem::Origin& og, const TileRand<kGeneral>& B, uint32_t lane) {
+  const uint32_t base = (uint32_t)__cvta_generic_to_shared(&m) + lane * 8u;
+  const uint32_t one = *(const volatile uint32_t*)&tab.one, neg = *(const volatile uint32_t*)&tab.neg;
   int dh = 0;
-  const Rates R(P);
-  auto one = [&](const uint4& at, const uint4& sh, uint32_t X, uint32_t Y, uint32_t r, const uint4& A, const uint2& W) {
+  const tilemem::Rates<true> R(P, kPar != 0);
+  auto one_round = [&](const uint4& ofs, const uint4& sh, uint32_t X, uint32_t Y, uint32_t r, const uint4& A,
+                       uint32_t Wp, uint32_t Wq) {
     if constexpr (kGeneral)
-      tilemem::round_general<kPar, kTrack>(base, at, sh, ghost, X, Y, og, dh, [&](uint32_t up, uint32_t uq) {
-        return accept_cells(P, R, tc, A, W, lane, r, up, uq);
+      tilemem::round_general<kTrack>(base, ofs, sh, one, X, Y, kPar != 0, og, dh, [&](uint32_t same, uint32_t any) {
+        return tilemem::accept_cells<true>(P, R, tid, s, A, kPar ? Wq : Wp, kPar ? Wp : Wq, lane, r, same, any, one, neg);
       });
     else
-      tilemem::round_p1<kPar, kTrack>(base, at, sh, ghost, X, Y, og, dh);
+      tilemem::round_p1<kPar, kTrack>(base, ofs, sh, one, X, Y, og, dh);
   };
-  uint32_t setw = tc.setw;
-  uint4 at0 = tab.at[setw & 3u], sh0 = tab.sh[setw & 3u], pos = B.pos[0][lane];
+  uint4 at0 = B.at[0], sh0 = B.sh[0], pos = B.pos[0][lane];
   uint4 A0 = B.acc[0][kGeneral ? lane : 0u];
   uint2 W = B.deep[0][kGeneral ? lane : 0u];   // outcomes of the next eight rounds, shifted round by round
 #pragma unroll 1
   for (uint32_t rp = 0; rp < kRounds / 2; ++rp) {
-    const uint32_t k1 = (setw >> 2) & 3u, k2 = (setw >> 4) & 3u, nx = (rp + 1u) & 7u;
-    setw >>= 4;
-    const uint4 at1 = tab.at[k1], sh1 = tab.sh[k1];
+    const uint32_t nx = (rp + 1u) & 7u;
+    const uint4 at1 = B.at[2u * rp + 1u], sh1 = B.sh[2u * rp + 1u];
     uint4 A1 = A0;
     if constexpr (kGeneral) {
       A1 = B.acc[2u * rp + 1u][lane];
       if (rp == 4u) W = B.deep[1][lane];
     }
-    one(at0, sh0, pos.x, pos.y, 2u * rp, A0, W);
-    at0 = tab.at[k2];
-    sh0 = tab.sh[k2];
+    one_round(at0, sh0, pos.x, pos.y, 2u * rp, A0, W.x, W.y);
+    at0 = B.at[2u * nx];
+    sh0 = B.sh[2u * nx];
     const uint4 pn = B.pos[nx][lane];
     if constexpr (kGeneral) A0 = B.acc[2u * nx][lane];
-    one(at1, sh1, pos.z, pos.w, 2u * rp + 1u, A1, make_uint2(W.x << 1, W.y << 1));
+    one_round(at1, sh1, pos.z, pos.w, 2u * rp + 1u, A1, W.x << 1, W.y << 1);
     pos = pn;
     W.x <<= 2;
     W.y <<= 2;
@@ -333,28 +271,19 @@ __device__ __forceinline__ void tile_rounds(const SweepParams& P, Window& w, Til
                                             uint32_t oy, uint32_t tx, uint32_t ty) {
   const uint32_t L = P.g.L;
   const uint32_t Y0 = (oy + ty * kTile) & (L - 1u), X0 = (ox + tx * kTile) & (L - 1u);
-  TileCtx tc;   // what the overflow draws need
-  tc.tid = ty * P.ntx + tx;
-  tc.s = s;
-  tc.setw = B.setw[0];
+  const uint32_t tid = ty * P.ntx + tx;
   const uint32_t uo = (0u - X0) & (L - 1u), vo = (0u - Y0) & (L - 1u);
   const bool track = (uo < kTile) && (vo < kTile), odd = (X0 + Y0 + P.g.par) & 1u;
   const tilemem::Origin og(lane, uo, vo);
-  const uint32_t ghost = tilemem::put_tile<kLive>(m, lane, w.T, w.hx, w.hy, w.left, w.up);
+  tilemem::put_tile<kLive>(m, lane, w.T, w.hx, w.hy, w.left, w.up);
+  __syncwarp();
   int dh;
-  if (track) dh = odd ? rounds_from<kGeneral, 1, true>(m, tab, ghost, P, tc, og, B, lane)
-                      : rounds_from<kGeneral, 0, true>(m, tab, ghost, P, tc, og, B, lane);
-  else       dh = odd ? rounds_from<kGeneral, 1, false>(m, tab, ghost, P, tc, og, B, lane)
-                      : rounds_from<kGeneral, 0, false>(m, tab, ghost, P, tc, og, B, lane);
+  if (track) dh = odd ? rounds_from<kGeneral, 1, true>(m, tab, P, tid, s, og, B, lane)
+                      : rounds_from<kGeneral, 0, true>(m, tab, P, tid, s, og, B, lane);
+  else       dh = odd ? rounds_from<kGeneral, 1, false>(m, tab, P, tid, s, og, B, lane)
+                      : rounds_from<kGeneral, 0, false>(m, tab, P, tid, s, og, B, lane);
   if (track && dh != 0) atomicAdd(P.h00, (unsigned long long)(long long)dh);
-#pragma unroll
-  for (uint32_t y = 0; y < 4; ++y)
-#pragma unroll
-    for (uint32_t px = 0; px < 2; ++px) {
-      const uint2 v = m.w[y][px][1u + lane];
-      w.T[y][2 * px] = v.x;
-      w.T[y][2 * px + 1] = v.y;
-    }
+  tilemem::get_tile(m, lane, w.T);
 }
 
 // Set swept in phase `phase` of sweep s (the shuffle of kpz_tileset.cu).
@@ -470,7 +399,7 @@ __global__ void __launch_bounds__(320, 1) resident_grid_kernel(const SweepParams
   uint32_t s, tx, ty, ox = 0u, oy = 0u, px = 0u, py = 0u;
   if (maker) {
     place(0u, s, tx, ty);
-    if (live) draw_tile<kGeneral>(P, rnd[slot], ty * P.ntx + tx, s, lane, part, makers);
+    if (live) draw_tile<kGeneral>(P, tab, rnd[slot], ty * P.ntx + tx, s, lane, part, makers);
   }
   if (makers) bar_sync(3, blockDim.x - 32u);
   for (uint32_t k = 0; k <= nsteps; ++k) {
@@ -481,7 +410,7 @@ __global__ void __launch_bounds__(320, 1) resident_grid_kernel(const SweepParams
     if (maker) {
       if (k + 1u < nsteps && live) {
         place(k + 1u, s, tx, ty);
-        draw_tile<kGeneral>(P, rnd[((k + 1u) & 1u) * wpc + slot], ty * P.ntx + tx, s, lane, part, makers);
+        draw_tile<kGeneral>(P, tab, rnd[((k + 1u) & 1u) * wpc + slot], ty * P.ntx + tx, s, lane, part, makers);
       }
     } else {
       const uint32_t sw = kSets ? k >> 2 : k;    // sweeps before this step
@@ -493,7 +422,7 @@ __global__ void __launch_bounds__(320, 1) resident_grid_kernel(const SweepParams
         py = oy;
       }
       if (!makers) {
-        if (live && !back) draw_tile<kGeneral>(P, B, ty * P.ntx + tx, s, lane, 0u, 1u);
+        if (live && !back) draw_tile<kGeneral>(P, tab, B, ty * P.ntx + tx, s, lane, 0u, 1u);
         __syncwarp();
         if (k != 0u) {
           bar_sync(2, blockDim.x);
@@ -501,8 +430,8 @@ __global__ void __launch_bounds__(320, 1) resident_grid_kernel(const SweepParams
         }
       }
       if (!kSets || (k & 3u) == 0u) {
-        ox = back ? 0u : B.setw[1];
-        oy = back ? 0u : B.setw[2];
+        ox = back ? 0u : B.origin[0];
+        oy = back ? 0u : B.origin[1];
       }
       const GlobalLat from{sw == 0u ? P.lat : scratch + ((sw - 1u) & 1u) * words};
       const GlobalLat to{back ? P.lat : scratch + (sw & 1u) * words};
@@ -624,11 +553,12 @@ __global__ void __launch_bounds__(384, 1) resident_cluster_kernel(const SweepPar
   const bool maker = warp >= tpc;
   const uint32_t slot = maker ? (warp - tpc) & (tpc - 1u) : warp, part = maker ? (warp - tpc) >> lg : 0u;
   const uint32_t tile = blockIdx.x * tpc + slot, ty = tile / P.ntx, tx = tile - ty * P.ntx;
+  __syncthreads();
   uint32_t* own = frame + slot * (kPlanes * 32u) + lane;   // this lane's words, 32 apart; + the frame's offset
   const uint32_t half = tpc * kPlanes * 32u;               // words of one frame in this block
   Window w;
   if (maker) {
-    draw_tile<kGeneral>(P, rnd[slot], tile, t0, lane, part, makers);
+    draw_tile<kGeneral>(P, tab, rnd[slot], tile, t0, lane, part, makers);
   } else {
     const uint32_t o = tx * kPlanes * P.g.NR + ty * 32u + lane;
 #pragma unroll
@@ -639,10 +569,10 @@ __global__ void __launch_bounds__(384, 1) resident_cluster_kernel(const SweepPar
   for (uint32_t k = 0; k < n; ++k) {
     const uint32_t s = t0 + k, buf = k & 1u;
     if (maker) {
-      if (k + 1u < n) draw_tile<kGeneral>(P, rnd[(buf ^ 1u) * tpc + slot], tile, s + 1u, lane, part, makers);
+      if (k + 1u < n) draw_tile<kGeneral>(P, tab, rnd[(buf ^ 1u) * tpc + slot], tile, s + 1u, lane, part, makers);
     } else {
       const TileRand<kGeneral>& B = rnd[buf * tpc + slot];
-      const uint32_t ox = B.setw[1], oy = B.setw[2];
+      const uint32_t ox = B.origin[0], oy = B.origin[1];
       load_window_cluster<1>(P, smem_u32(frame + buf * half), lg, lane, (ox - px + tx * kTile) & (L - 1u),
                              (oy - py + ty * kTile) & (L - 1u), w);
       tile_rounds<kGeneral, false>(P, w, mem[slot], tab, B, lane, s, ox, oy, tx, ty);

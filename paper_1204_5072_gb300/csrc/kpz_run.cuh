@@ -36,6 +36,7 @@
 // warps work on tiles of both parities at once).
 #pragma once
 #include "kpz_rounds.cuh"
+#include "kpz_tilemem.cuh"
 
 namespace kpz {
 namespace run {
@@ -69,19 +70,32 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_al
 // column t+1 as read and Pf[t&1] receives t+2); Hf: lane 31's halo row, a
 // ring of three block columns.
 template <int CR>
-struct WarpStage {
+struct alignas(16) WarpStage {
   uint32_t M[CR][kPlanes][32];
   uint32_t Pf[2][CR][kPlanes][32];
   uint32_t Hf[3][4];
 };
+// The rounds of 128 x 128 tiles of 4 x 4 cells at general rates run from
+// shared memory.
+template <int CR>
+struct alignas(16) WarpStageMem : WarpStage<CR> {
+  tilemem::TileMem mem;
+};
 constexpr uint32_t kMaxWarpsPerCta = 8;
+// Rates: p = 1, q = 0; general; general with a rate of 0 or 1.
+enum Mode : int { kGrowth = 0, kInner = 1, kEdgeRate = 2 };
+inline Mode mode_of(const SweepParams& P) {
+  if (P.Tp == 65536u && P.Tq == 0u) return kGrowth;
+  return (P.Tp == 0u || P.Tp == 65536u || P.Tq == 0u || P.Tq == 65536u) ? kEdgeRate : kInner;
+}
 
 // One run: tiles tx0 .. tx0 + n - 1 of tile row ty (n <= ntx), left to right.
-template <bool kGeneral, int CR, bool kSK, bool kRtPar = false, bool kC2 = false>
-__device__ __forceinline__ void sweep_run(const SweepParams& P, WarpStage<CR>& ws, const uint4* rk,
+template <int kMode, int CR, bool kSK, bool kRtPar = false, bool kC2 = false, class Stage>
+__device__ __forceinline__ void sweep_run(const SweepParams& P, Stage& ws, const uint4* rk, const tilemem::QuadTab& tab,
                                           uint32_t lane,
                                           uint32_t s, uint32_t ox, uint32_t oy, uint32_t ty,
                                           uint32_t tx0, uint32_t n) {
+  constexpr bool kGeneral = kMode != kGrowth;
   constexpr uint32_t kTileY = kTile * CR;
   static_assert(!kC2 || CR == 1, "the C = 2 work-group layer holds one cell row per lane");
   const uint32_t L = P.g.L, NR = P.g.NR, NB = P.g.NB;
@@ -159,6 +173,7 @@ __device__ __forceinline__ void sweep_run(const SweepParams& P, WarpStage<CR>& w
 #pragma unroll
     for (uint32_t p = 0; p < kPlanes; ++p) ws.Pf[1][r][p][lane] = T[r][p >> 2][p & 3u];
   if (n > 1u) prefetch(2u);
+  __syncwarp();   // Hf
 
   TileCtx tc;
   tc.rk = rk;
@@ -168,23 +183,17 @@ __device__ __forceinline__ void sweep_run(const SweepParams& P, WarpStage<CR>& w
   tc.last_lane = last_lane;
   const uint32_t vo = (0u - Y0) & (L - 1u);
 
-  // Quadrant sets: with round keys in shared memory (kSK) lane l draws the set
-  // of tile t0 + l (t0 = t & ~31) and the warp broadcasts it, one draw per 32
-  // tiles; otherwise every lane draws the set of each tile.
+  // Quadrant sets: lane l draws the set of tile t0 + l (t0 = t & ~31) and the
+  // warp broadcasts it, one draw per 32 tiles.
   uint32_t set_lane = 0;
 #pragma unroll 1
   for (uint32_t t = 0; t < n; ++t) {
-    if (!kSK) {
-      tc.tid = ty * P.ntx + tx0 + t;
-      tc.setw = philox(kTagSet << 28, tc.tid, s, P.sample, P.k0, P.k1).x;
-    } else {
-      if ((t & 31u) == 0u) {
-        tc.tid = ty * P.ntx + tx0 + t + lane;
-        set_lane = philox_sk(kTagSet << 28, tc.tid, s, P.sample, rk).x;
-      }
-      tc.tid = ty * P.ntx + tx0 + t;
-      tc.setw = __shfl_sync(kFull, set_lane, t & 31u);
+    if ((t & 31u) == 0u) {
+      tc.tid = ty * P.ntx + tx0 + t + lane;
+      set_lane = rounds::draw<kSK>(P, tc, kTagSet << 28).x;
     }
+    tc.tid = ty * P.ntx + tx0 + t;
+    tc.setw = __shfl_sync(kFull, set_lane, t & 31u);
     const uint32_t uo = (0u - ((X0 + t * kTile) & (L - 1u))) & (L - 1u);
     tc.track = (uo < kTile) && (vo < kTileY);
     tc.xo = uo & 3u; tc.co = uo >> 2; tc.yo = vo & 3u; tc.cyo = vo >> 2;
@@ -195,10 +204,10 @@ __device__ __forceinline__ void sweep_run(const SweepParams& P, WarpStage<CR>& w
     for (int r = 0; r < CR; ++r)
 #pragma unroll
       for (uint32_t yq = 0; yq < 4; ++yq)   // bit 0 of window t+1 = bit shx[0] of block column t+1
-        hx[r][yq] = ((t == 0u ? ws.M[r][yq * 4][lane] : ws.Pf[(t + 1u) & 1u][r][yq * 4][lane]) >> shx[0]) & 1u;
+        hx[r][yq] = (t == 0u ? ws.M[r][yq * 4][lane] : ws.Pf[(t + 1u) & 1u][r][yq * 4][lane]) >> shx[0];   // bit 0
 #pragma unroll
     for (uint32_t xq = 0; xq < 4; ++xq)
-      hy[xq] = last_lane ? __funnelshift_r(ws.Hf[t % 3u][xq], ws.Hf[(t + 1u) % 3u][xq], shx[xq]) : 0u;
+      hy[xq] = __funnelshift_r(ws.Hf[t % 3u][xq], ws.Hf[(t + 1u) % 3u][xq], shx[xq]);   // lane 31 needs it
 
     const bool last = (t + 1u == n);
     const uint32_t keep = t == 0u ? 1u : (t & 1u);   // slot of the start copy
@@ -211,7 +220,16 @@ __device__ __forceinline__ void sweep_run(const SweepParams& P, WarpStage<CR>& w
 
     int dh = 0;
     // The one tile per sweep that holds site (0,0) also counts its moves.
-    if (kC2) {      // C = 2 work-group layer (one cell row per lane)
+    if constexpr (CR == 1 && !kC2 && kGeneral) {
+      tilemem::put_rounds(ws.mem, tab, lane, tc.setw);
+      tilemem::put_tile<false>(ws.mem, lane, T[0], hx[0], hy, hy, hy);
+      __syncwarp();
+      const tilemem::Origin og(lane, uo, vo);
+      auto draw_block = [&](uint32_t c0) { return rounds::draw<kSK>(P, tc, c0); };
+      dh = tc.track ? tilemem::rounds_drawn<kMode == kEdgeRate, true>(ws.mem, tab, P, tc.tid, s, par != 0, og, lane, draw_block)
+                    : tilemem::rounds_drawn<kMode == kEdgeRate, false>(ws.mem, tab, P, tc.tid, s, par != 0, og, lane, draw_block);
+      tilemem::get_tile(ws.mem, lane, T[0]);
+    } else if (kC2) {      // C = 2 work-group layer (one cell row per lane)
       auto& T0 = reinterpret_cast<uint32_t(&)[4][4]>(T[0]);
       if (tc.track) {
         if (par) rounds::tile_rounds_c2<kGeneral, 1, true, kSK>(T0, hx[0], hy, P, tc, lane, dh);
@@ -235,6 +253,7 @@ __device__ __forceinline__ void sweep_run(const SweepParams& P, WarpStage<CR>& w
 
     // Write back block column t and slide the window to tile t+1.
     cp_async_wait();
+    __syncwarp();   // Hf: lane 31's copies, read by all lanes
     if (t != 0u && !last) {
       // Interior tile: both words of each window row are this run's alone.
       // One wide multiply-add gives the word to store, carry | T << sh, and

@@ -7,6 +7,7 @@
 // shared memory instead of being advanced per draw.
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "kpz_run.cuh"
 
@@ -23,17 +24,29 @@ using run::kMaxWarpsPerCta;
 // Every warp makes exactly one fetch past the last chunk; the warp whose
 // fetch is the last of all (nchunks + W - 1) returns the counter to zero for
 // the next launch.
-template <bool kGeneral, int CR, bool kC2>
-__global__ void __launch_bounds__(256, CR == 1 ? (kGeneral ? 2 : 3) : (kGeneral ? 1 : 2))
+template <int kMode, int CR, bool kC2>
+struct StageOf {
+  using type = WarpStage<CR>;
+};
+template <int kMode>
+struct StageOf<kMode, 1, false> {
+  using type = std::conditional_t<kMode == run::kGrowth, WarpStage<1>, run::WarpStageMem<1>>;
+};
+template <int kMode, int CR, bool kC2>
+__global__ void __launch_bounds__(256, CR == 1 ? (kMode != run::kGrowth ? 2 : 3) : (kMode != run::kGrowth ? 1 : 2))
 sweep_kernel(const SweepParams P) {
+  constexpr bool kGeneral = kMode != run::kGrowth;
+  using Stage = typename StageOf<kMode, CR, kC2>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  WarpStage<CR>& ws = reinterpret_cast<WarpStage<CR>*>(smem_raw)[threadIdx.x >> 5];
+  Stage& ws = reinterpret_cast<Stage*>(smem_raw)[threadIdx.x >> 5];
   __shared__ uint4 rk[kPhiloxRounds / 2];   // Philox round keys of (k0, k1)
   if (!kGeneral && threadIdx.x < kPhiloxRounds / 2) {
     const uint32_t r = 2u * threadIdx.x;
     rk[threadIdx.x] = make_uint4(P.k0 + r * kPhiloxWeylA, P.k1 + r * kPhiloxWeylB,
                                  P.k0 + (r + 1u) * kPhiloxWeylA, P.k1 + (r + 1u) * kPhiloxWeylB);
   }
+  __shared__ tilemem::QuadTab tab;
+  if (kGeneral && threadIdx.x < 4u) tilemem::fill_quad_tab(tab, threadIdx.x);
   __syncthreads();
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t W = gridDim.x * (blockDim.x >> 5);
@@ -51,7 +64,7 @@ sweep_kernel(const SweepParams P) {
     uint32_t next = 0;
     if (lane == 0) next = atomicAdd(P.queue, 1u);
     const uint32_t ty = c / cpr;
-    run::sweep_run<kGeneral, CR, !kGeneral, false, kC2>(P, ws, rk, lane, s, ox, oy, ty, (c - ty * cpr) * P.run,
+    run::sweep_run<kMode, CR, !kGeneral, false, kC2>(P, ws, rk, tab, lane, s, ox, oy, ty, (c - ty * cpr) * P.run,
                                                        P.run);
     c = __shfl_sync(kFull, next, 0);
   }
@@ -59,7 +72,7 @@ sweep_kernel(const SweepParams P) {
 }
 
 // Resident CTAs per SM of one sweep kernel at wpc warps per CTA (cached per device).
-template <bool kGeneral, int CR, bool kC2>
+template <int kMode, int CR, bool kC2>
 cudaError_t resident_ctas(uint32_t wpc, uint32_t& ctas) {
   constexpr int kMaxDev = 64;
   static std::mutex mu;
@@ -69,12 +82,12 @@ cudaError_t resident_ctas(uint32_t wpc, uint32_t& ctas) {
   if (e != cudaSuccess) return e;
   std::lock_guard<std::mutex> lock(mu);
   if (dev < kMaxDev && cache[dev][wpc]) { ctas = cache[dev][wpc]; return cudaSuccess; }
-  const int bytes = (int)(kMaxWarpsPerCta * sizeof(WarpStage<CR>));
-  e = cudaFuncSetAttribute(sweep_kernel<kGeneral, CR, kC2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  const int bytes = (int)(kMaxWarpsPerCta * sizeof(typename StageOf<kMode, CR, kC2>::type));
+  e = cudaFuncSetAttribute(sweep_kernel<kMode, CR, kC2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e != cudaSuccess) return e;
   int per_sm = 0, sms = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sweep_kernel<kGeneral, CR, kC2>, (int)(wpc * 32u),
-                                                    wpc * sizeof(WarpStage<CR>));
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sweep_kernel<kMode, CR, kC2>, (int)(wpc * 32u),
+                                                    wpc * sizeof(typename StageOf<kMode, CR, kC2>::type));
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   ctas = (uint32_t)(per_sm > 0 ? per_sm : 1) * (uint32_t)(sms > 0 ? sms : 1);
@@ -82,15 +95,15 @@ cudaError_t resident_ctas(uint32_t wpc, uint32_t& ctas) {
   return cudaSuccess;
 }
 
-template <bool kGeneral, int CR, bool kC2 = false>
+template <int kMode, int CR, bool kC2 = false>
 cudaError_t launch_cr(const SweepParams& P, uint32_t wpc, cudaStream_t st) {
   uint32_t ctas = 0;
-  cudaError_t e = resident_ctas<kGeneral, CR, kC2>(wpc, ctas);
+  cudaError_t e = resident_ctas<kMode, CR, kC2>(wpc, ctas);
   if (e != cudaSuccess) return e;
   // One wave of resident warps, fewer if there are fewer tiles than warps.
   const uint64_t tiles = (uint64_t)P.ntx * P.nty;
   const uint64_t blocks = std::min<uint64_t>(ctas, (tiles + wpc - 1) / wpc);
-  sweep_kernel<kGeneral, CR, kC2><<<(unsigned)blocks, wpc * 32u, wpc * sizeof(WarpStage<CR>), st>>>(P);
+  sweep_kernel<kMode, CR, kC2><<<(unsigned)blocks, wpc * 32u, wpc * sizeof(typename StageOf<kMode, CR, kC2>::type), st>>>(P);
   return cudaSuccess;
 }
 
@@ -104,15 +117,18 @@ cudaError_t launch_sweep(const SweepParams& P, uint32_t warps_per_cta, cudaStrea
   if (wpc > kMaxWarpsPerCta) return cudaErrorInvalidValue;
   const uint32_t tile_y = P.g.L / P.nty;
   cudaError_t e;
-  const bool general = !(P.Tp == 65536u && P.Tq == 0u);
+  const run::Mode mode = run::mode_of(P);
+  const bool general = mode != run::kGrowth;   // the variants without TileMem have one general form
   if (P.cell == 2u && tile_y == kTile)
-    e = general ? launch_cr<true, 1, true>(P, wpc, st) : launch_cr<false, 1, true>(P, wpc, st);
+    e = general ? launch_cr<run::kEdgeRate, 1, true>(P, wpc, st) : launch_cr<run::kGrowth, 1, true>(P, wpc, st);
   else if (P.cell == 2u)
     return cudaErrorInvalidValue;
   else if (tile_y == kTile)
-    e = general ? launch_cr<true, 1>(P, wpc, st) : launch_cr<false, 1>(P, wpc, st);
+    e = mode == run::kInner ? launch_cr<run::kInner, 1>(P, wpc, st)
+        : general           ? launch_cr<run::kEdgeRate, 1>(P, wpc, st)
+                            : launch_cr<run::kGrowth, 1>(P, wpc, st);
   else if (tile_y == 2u * kTile)
-    e = general ? launch_cr<true, 2>(P, wpc, st) : launch_cr<false, 2>(P, wpc, st);
+    e = general ? launch_cr<run::kEdgeRate, 2>(P, wpc, st) : launch_cr<run::kGrowth, 2>(P, wpc, st);
   else
     return cudaErrorInvalidValue;
   if (e != cudaSuccess) return e;
