@@ -8,9 +8,9 @@
 #include <atomic>
 #include <new>
 #include <string>
-#include <thread>
 
 #include "kpz.h"
+#include "kpz_host.h"
 #include "kpz_internal.h"
 #include "kpz_observe.h"
 #include "kpz_resident.h"
@@ -143,35 +143,6 @@ cudaError_t io_prepare(kpz_ctx* c) {
   e = cudaEventRecord(c->io_ev[4], c->stream);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(c->io_stream, c->io_ev[4], 0);
   return e;
-}
-
-// Writes to every page of a caller's buffer that the call is about to fill.
-// Pages of a fresh allocation exist only once touched, and a GPU that is the
-// first to touch one waits some 55 us for each 64 KiB (heights at L = 2048 took
-// 28 ms into a fresh array, 1.2 ms into a touched one); the CPU takes 3.5 us a
-// page, and large buffers are split over a few threads.
-void touch_pages(void* p, size_t bytes) {
-  constexpr size_t kPage = 4096, kPart = size_t(4) << 20, kThreads = 8;
-  auto touch = [](char* a, char* b) {
-    for (; a < b; a += kPage) *(volatile char*)a = 0;
-  };
-  char* base = (char*)p;
-  const size_t parts = std::min(kThreads, bytes / kPart);
-  size_t done = 0;
-  std::thread th[kThreads];
-  size_t n = 0;
-  try {
-    for (; n + 1 < parts; ++n) {
-      const size_t end = done + bytes / parts / kPage * kPage;
-      th[n] = std::thread(touch, base + done, base + end);
-      done = end;
-    }
-  } catch (...) {   // no thread to be had: the rest is touched here
-  }
-  touch(base + done, base + bytes);
-  for (std::thread& t : th)
-    if (t.joinable()) t.join();
-  if (bytes) *(volatile char*)(base + bytes - 1) = 0;
 }
 
 // Rows per band when the staging band is used as two halves.
@@ -330,9 +301,7 @@ kpz_status kpz_init(kpz_ctx** out, uint32_t L, double p, double q, uint64_t seed
       return KPZ_ENOMEM;
     }
   }
-  int pageable = 0;
-  cudaDeviceGetAttribute(&pageable, cudaDevAttrPageableMemoryAccess, ctx->device);
-  ctx->direct_host = pageable != 0;
+  ctx->direct_host = reaches_pageable(ctx->device);
   char* base = (char*)ctx->buf;
   ctx->lat = (uint32_t*)(base + y.lat);
   ctx->t_dev = (uint64_t*)(base + y.small);

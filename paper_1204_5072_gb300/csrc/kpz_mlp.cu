@@ -1,7 +1,7 @@
 // kpz_mlp.cu -- the learned surrogate: a 4-128-128-128-1 GELU MLP with
 // bfloat16 weights and float32 arithmetic, trained with Adam by the kernels
-// below (forward and backward on the tcgen05 tensor cores, gradient
-// reduction, update).
+// below (forward and backward in one kernel on the tcgen05 tensor cores,
+// gradient reduction and update in another).
 //
 // The paper has no learned component. The network maps the features of a
 // realisation and a time (log2 L, log t, p, q, scaled) to log W^2; the
@@ -11,11 +11,13 @@
 // deterministic for a given data order.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <new>
 #include <vector>
 
 #include "kpz.h"
+#include "kpz_host.h"
 #include "kpz_internal.h"
 
 namespace kpz {
@@ -25,55 +27,98 @@ constexpr int kW = 128, kIn = 4;
 constexpr int oW1 = 0, oB1 = oW1 + kW * kIn, oW2 = oB1 + kW, oB2 = oW2 + kW * kW, oW3 = oB2 + kW,
               oB3 = oW3 + kW * kW, oW4 = oB3 + kW, oB4 = oW4 + kW, kParams = oB4 + 1;
 static_assert(kParams == 33793, "parameter count");
-constexpr int kPart = kParams + 1;   // per-tile gradient partial + squared-error sum
+constexpr int kPart = kParams + 3;   // partial of one block: gradient, squared-error sum; 16-byte multiple
+static_assert(kPart % 4 == 0 && oW2 % 4 == 0 && oW3 % 4 == 0, "16-byte stores of the weight gradients");
 
-__device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_grad(float z) {
-  return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * expf(-0.5f * z * z);
-}
 __device__ __forceinline__ float bf(const __nv_bfloat16* p, int i) { return __bfloat162float(p[i]); }
 
 // ---------------------------------------------------------------------------
-// The 128 x 128 layers on the 5th-generation tensor cores (tcgen05). A tile
-// is 128 samples, four threads per sample (each a quarter of the units). In
-// the forward pass the two 128 x 128 layers run as
-// D[s][j] = sum_k A[s][k] W[j][k] with M = N = K = 128: A (activations) and W
-// (weights) in shared memory in the canonical K-major layout without swizzle
-// (8-row x 16-byte core matrices, 128 B apart along K, 2048 B apart along the
-// rows), the float32 accumulator in tensor memory (lane = sample, column =
-// unit). The MMA takes bfloat16 operands; the weights are bfloat16 already,
-// each float32 activation a is split into hi = bf16(a) and lo = bf16(a - hi),
-// and two chains of MMAs (hi, then lo, 8 of K = 16 each) accumulate
-// sum_k (hi + lo) W, which agrees with the float32 product to about 2^-16
-// relative. One thread issues the MMAs and commits them to an mbarrier; every
-// wait on it is bounded in time (a timeout sets *err and the host reports it).
+// Forward and backward pass on the 5th-generation tensor cores (tcgen05). A
+// tile is 32 samples; units are the rows of every product (M = 128), samples
+// its columns, so one thread owns a unit and 8 samples of it: 16 warps, warp w
+// reads tensor-memory lanes 32 (w % 4) onwards and columns 8 (w / 4) onwards.
+// What bounds a minibatch is the chain of products and activations, not work:
+// a small tile spreads 128 samples over four SMs and leaves a thread 8
+// activations a layer (128-sample tiles with 32 took 19 us forward and 113 us
+// backward on one SM), and forward and backward share one kernel, which keeps
+// the activations' derivatives in registers instead of writing pre-activations
+// out and evaluating them three times over. Larger inputs loop over tiles in a
+// block per SM, with the weights staged once and the weight gradients
+// accumulated in tensor memory.
+// Whole calls from host arrays, before (forward, backward, reduction and Adam
+// in four kernels with 128-sample tiles, four copies): loss_grad of 128 samples
+// 217 -> 40 us, of 300000 2860 -> 470; predict of 251 47 -> 23 us, of 300000
+// 332 -> 240; 24 training steps of 128 samples 4.3 -> 0.64 ms.
+//
+// Operands are bfloat16 in shared memory without swizzle, core matrices of 8
+// rows x 16 bytes. The weights are bfloat16 already; activations h and errors
+// dz are split into a high and a low part, hi = bf16(a), lo = bf16(a - hi), and
+// every product takes the chains that matter (hi, lo with weights; hi.hi,
+// hi.lo, lo.hi between activations and errors), which agrees with the float32
+// product to about 2^-16 relative. One copy of each operand serves all its
+// products, as K-major or MN-major matrix:
+//   W [unit][k]        forward: A, K-major; input gradient: A = W^T, MN-major
+//   h, dz [unit][sample] (8 samples = 16 bytes): B, MN-major, of those two;
+//                      weight gradient dz h^T: A and B, K-major (K = samples).
+// One thread issues the products and commits them to an mbarrier; every wait
+// on one is bounded in time (a timeout sets *err and the host reports it).
 namespace tc {
 
-constexpr int kM = 128;                              // samples per tile (MMA M)
-constexpr int kQ = 4;                                // threads per sample: a quarter of the units each
-constexpr int kThreads = kM * kQ;                    // 16 warps; warp w reads tensor-memory lanes 32 (w % 4)
-constexpr uint32_t kOpBytes = (uint32_t)kW * kW * 2;  // one 128 x 128 bfloat16 operand
-constexpr size_t kSmem = 3 * (size_t)kOpBytes;       // A hi, A lo, W
-// Instruction descriptor of tcgen05.mma kind::f16: float32 accumulator
-// (bits 4-5 = 1), bfloat16 A and B (bits 7-9, 10-12 = 1), both K-major,
-// N / 8 at bits 17-22, M / 16 at bits 24-28.
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kW >> 3) << 17) |
-                            ((uint32_t)(kM >> 4) << 24);
-constexpr uint64_t kWaitNs = 1000000000ull;          // bound of every wait
+constexpr int kS = 32;                                // samples per tile
+constexpr int kThreads = 512;
+constexpr uint32_t kWBytes = (uint32_t)kW * kW * 2;   // a weight matrix
+constexpr uint32_t kHBytes = (uint32_t)kW * kS * 2;   // a high or low part of h or dz
+// Instruction descriptor of tcgen05.mma kind::f16: float32 accumulator, both
+// operands bfloat16, transpose bits (MN-major A, B), N / 8, M / 16.
+constexpr uint32_t idesc(bool ta, bool tb, int n) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((ta ? 1u : 0u) << 15) | ((tb ? 1u : 0u) << 16) |
+         ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kW >> 4) << 24);
+}
+constexpr uint64_t kWaitNs = 1000000000ull;           // bound of every wait
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// Byte offset of element (row, k) of a 128 x 128 bfloat16 operand.
-__device__ __forceinline__ uint32_t cm_off(int row, int k) {
-  return (uint32_t)(((row >> 3) * 16 + (k >> 3)) * 128 + (row & 7) * 16 + (k & 7) * 2);
-}
-
-// Shared-memory matrix descriptor: start address, leading-dimension byte
-// offset (between core matrices along K: 128), stride byte offset (between
-// 8-row groups: 2048), descriptor version 1 (bit 46), no swizzle.
-__device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
-  return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)(128u >> 4) << 16) | ((uint64_t)(2048u >> 4) << 32) |
+// Shared-memory matrix descriptor: start address, byte offsets between core
+// matrices along the leading dimension (K) and the other one, version 1 (bit
+// 46), no swizzle.
+__device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t along_k, uint32_t along_mn) {
+  return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)(along_k >> 4) << 16) | ((uint64_t)(along_mn >> 4) << 32) |
          (1ull << 46);
+}
+__device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t id, bool acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+      "l"(a), "l"(b), "r"(id), "r"((uint32_t)acc));
+}
+__device__ __forceinline__ void commit(uint32_t mbar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar) : "memory");
+}
+// D[j][s] = sum_k W[j][k] h[k][s].
+__device__ __forceinline__ void mma_forward(uint32_t d, uint32_t w, uint32_t hi, uint32_t lo) {
+#pragma unroll
+  for (int i = 0; i < 2 * (kW / 16); ++i) {
+    const int kk = i & 7;
+    mma(d, sdesc(w + kk * 256u, 128u, 2048u), sdesc((i < 8 ? hi : lo) + kk * 1024u, 512u, 128u), idesc(false, true, kS),
+        i != 0);
+  }
+}
+// D[k][s] = sum_u W[u][k] dz[u][s].
+__device__ __forceinline__ void mma_input(uint32_t d, uint32_t w, uint32_t hi, uint32_t lo) {
+#pragma unroll
+  for (int i = 0; i < 2 * (kW / 16); ++i) {
+    const int kk = i & 7;
+    mma(d, sdesc(w + kk * 4096u, 2048u, 128u), sdesc((i < 8 ? hi : lo) + kk * 1024u, 512u, 128u), idesc(true, true, kS),
+        i != 0);
+  }
+}
+// D[u][k] (+)= sum_s dz[u][s] h[k][s].
+__device__ __forceinline__ void mma_weight(uint32_t d, uint32_t dzhi, uint32_t dzlo, uint32_t hhi, uint32_t hlo, bool acc) {
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const uint32_t a = (i >= 4 ? dzlo : dzhi) + (i & 1) * 256u, b = ((i & 6) == 2 ? hlo : hhi) + (i & 1) * 256u;
+    mma(d, sdesc(a, 128u, 512u), sdesc(b, 128u, 512u), idesc(false, false, kW), acc || i != 0);
+  }
 }
 
 __device__ __forceinline__ uint64_t gtimer() {
@@ -81,42 +126,34 @@ __device__ __forceinline__ uint64_t gtimer() {
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
-
-// D (tensor memory) = (Ahi + Alo) W^T over K = 128, then commit to mbar.
-__device__ __forceinline__ void mma_chain(uint32_t taddr, uint32_t ahi, uint32_t alo, uint32_t b, uint32_t mbar) {
-#pragma unroll
-  for (int part = 0; part < 2; ++part) {
-#pragma unroll
-    for (int kk = 0; kk < kW / 16; ++kk) {
-      const uint64_t ad = sdesc((part ? alo : ahi) + kk * 256u);
-      const uint64_t bd = sdesc(b + kk * 256u);
-      const uint32_t acc = (part | kk) ? 1u : 0u;
-      asm volatile(
-          "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-          " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(taddr),
-          "l"(ad), "l"(bd), "r"(kIdesc), "r"(acc));
-    }
-  }
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
-               : "memory");
-}
-
 // Wait until phase `parity` of the mbarrier has completed; false on timeout.
 __device__ __forceinline__ bool wait_phase(uint32_t mbar, uint32_t parity) {
-  const uint64_t t0 = gtimer();
-  for (;;) {
+  uint64_t t0 = 0;
+  for (uint32_t it = 0;; ++it) {
     uint32_t done;
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.b32 %0, 1, 0, p;\n}\n"
         : "=r"(done)
         : "r"(mbar), "r"(parity)
         : "memory");
-    if (done) return true;
-    if (gtimer() - t0 > kWaitNs) return false;
+    if (done) break;
+    if (it == 0) t0 = gtimer();
+    else if (gtimer() - t0 > kWaitNs) return false;
   }
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  return true;
 }
 
-// 32 consecutive float32 columns of this warp's 32 tensor-memory lanes.
+// 8 and 32 consecutive float32 columns of this warp's 32 tensor-memory lanes.
+__device__ __forceinline__ void ld8(uint32_t ta, float (&v)[8]) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(ta));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
 __device__ __forceinline__ void ld32(uint32_t ta, float (&v)[32]) {
   uint32_t r[32];
   asm volatile(
@@ -132,28 +169,33 @@ __device__ __forceinline__ void ld32(uint32_t ta, float (&v)[32]) {
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// Eight activations h[0..7] of units j0..j0+7 (j0 % 8 == 0) of sample row s,
-// split into bfloat16 hi and lo parts, as one 16-byte core-matrix row each.
-__device__ __forceinline__ void put8(unsigned char* Ahi, unsigned char* Alo, int s, int j0, const float* h) {
+// Eight values of unit u and sample group g, as high and low parts.
+__device__ __forceinline__ void put8(unsigned char* Xhi, unsigned char* Xlo, int u, int g, const float (&v)[8]) {
   __align__(16) __nv_bfloat16 hi[8], lo[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    hi[i] = __float2bfloat16_rn(h[i]);
-    lo[i] = __float2bfloat16_rn(h[i] - __bfloat162float(hi[i]));
+    hi[i] = __float2bfloat16_rn(v[i]);
+    lo[i] = __float2bfloat16_rn(v[i] - __bfloat162float(hi[i]));
   }
-  *reinterpret_cast<uint4*>(Ahi + cm_off(s, j0)) = *reinterpret_cast<const uint4*>(hi);
-  *reinterpret_cast<uint4*>(Alo + cm_off(s, j0)) = *reinterpret_cast<const uint4*>(lo);
+  const uint32_t at = (uint32_t)(((u >> 3) * 4 + g) * 128 + (u & 7) * 16);
+  *reinterpret_cast<uint4*>(Xhi + at) = *reinterpret_cast<const uint4*>(hi);
+  *reinterpret_cast<uint4*>(Xlo + at) = *reinterpret_cast<const uint4*>(lo);
 }
 
-// W (128 x 128 bfloat16, row = output unit, K contiguous) into the operand layout.
+// W (128 x 128 bfloat16, row = output unit, K contiguous): 8-row x 16-byte core
+// matrices, 128 bytes apart along K, 2048 along the rows.
 __device__ __forceinline__ void stage_w(unsigned char* Bs, const __nv_bfloat16* W, int t) {
-#pragma unroll 4
-  for (int q = t; q < kW * kW / 8; q += kThreads) {
-    const int row = q >> 4, k0 = (q & 15) * 8;
-    *reinterpret_cast<uint4*>(Bs + cm_off(row, k0)) = *reinterpret_cast<const uint4*>(W + row * kW + k0);
+  uint4 v[kW * kW / 8 / kThreads];
+#pragma unroll
+  for (int i = 0; i < kW * kW / 8 / kThreads; ++i) v[i] = *reinterpret_cast<const uint4*>(W + (t + i * kThreads) * 8);
+#pragma unroll
+  for (int i = 0; i < kW * kW / 8 / kThreads; ++i) {
+    const int q = t + i * kThreads, row = q >> 4, k8 = q & 15;
+    *reinterpret_cast<uint4*>(Bs + ((row >> 3) * 16 + k8) * 128 + (row & 7) * 16) = v[i];
   }
 }
 
+// Shared-memory writes of all threads visible to the tensor cores.
 __device__ __forceinline__ void fence_to_mma() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -161,344 +203,271 @@ __device__ __forceinline__ void fence_to_mma() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
+// gelu(z) and, for training, its derivative (sharing the error function).
+template <bool kGrad>
+__device__ __forceinline__ float gelu(float z, float& d) {
+  const float c = 0.5f * (1.0f + erff(z * 0.70710678118654752f));
+  if (kGrad) d = c + z * 0.39894228040143268f * expf(-0.5f * z * z);
+  return z * c;
+}
+
+constexpr size_t kSmemPredict = 2 * (size_t)kWBytes + 2 * (size_t)kHBytes;   // W2, W3, h hi, h lo
+constexpr size_t kSmemGrad = 2 * (size_t)kWBytes + 8 * (size_t)kHBytes;      // h1, h2, dz3, dz2, hi and lo
+
 }  // namespace tc
 
-// Forward pass of a tile of 128 samples: y (and, for training, the
-// pre-activations z1..z3 in zsave). Thread (sample s, quarter q) handles units
-// 32 q .. 32 q + 31 of sample s; warps 4 q .. 4 q + 3 read columns 32 q ..
-// 32 q + 31 of the tensor-memory lanes of their samples.
-__global__ void __launch_bounds__(tc::kThreads, 1) fwd_kernel(const __nv_bfloat16* __restrict__ P,
-                                                              const float* __restrict__ x, int n,
-                                                              float* __restrict__ y, float* __restrict__ zsave,
-                                                              int* __restrict__ err) {
+// kGrad = false: y[i] = network(x[i]). kGrad = true: the gradient of the mean
+// squared error over the block's tiles (block b takes tiles b, b + gridDim.x,
+// ...) and the sum of squared errors into its slot of gpart. x, t and y may be
+// host memory the device reaches; the next tile's samples are read ahead.
+template <bool kGrad>
+__global__ void __launch_bounds__(tc::kThreads, kGrad ? 1 : 2)
+    net_kernel(const __nv_bfloat16* __restrict__ P, const float* __restrict__ x, const float* __restrict__ t, int n,
+               float inv_n, float* __restrict__ y, float* __restrict__ gpart, int* err) {
   extern __shared__ __align__(1024) unsigned char smem_tc[];
-  unsigned char* Ahi = smem_tc;
-  unsigned char* Alo = smem_tc + tc::kOpBytes;
-  unsigned char* Bs = smem_tc + 2 * tc::kOpBytes;
-  __shared__ __align__(8) uint64_t mbar;
+  unsigned char* Wb[2] = {smem_tc, smem_tc + tc::kWBytes};
+  unsigned char* Hb = smem_tc + 2 * tc::kWBytes;
+  // h1, h2 (predict: one pair of buffers, h2 replaces h1), dz3, dz2; hi and lo
+  auto buf = [&](int i) { return Hb + (size_t)i * tc::kHBytes; };
+  constexpr int iH1 = 0, iH2 = kGrad ? 2 : 0, iD3 = 4, iD2 = 6;
+  constexpr uint32_t kCols = kGrad ? 512u : 32u;   // tensor memory: products 0..31, dW3 32.., dW2 160..
+  __shared__ __align__(8) uint64_t mbar[2];
   __shared__ uint32_t taddr_s;
-  __shared__ float part[tc::kQ][tc::kM];
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int s = (warp & 3) * 32 + (tid & 31), q = warp >> 2, u0 = 32 * q;
-  const int gs = blockIdx.x * tc::kM + s;
-  const bool live = gs < n;
-  float xin[kIn];
+  __shared__ float xs[tc::kS * kIn], ts[tc::kS], part[4][tc::kS];
+  __shared__ float red[4][kW][kIn + 1];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int u = (warp & 3) * 32 + lane, g = warp >> 2, s0 = 8 * g;
+  const int ntiles = (n + tc::kS - 1) / tc::kS;
+  // Samples of a tile, one value a thread: inputs (threads 0..127), targets (128..159).
+  auto fetch = [&](int tile) -> float {
+    const long long i = (long long)tile * tc::kS;
+    if (tile >= ntiles) return 0.f;
+    if (tid < tc::kS * kIn) return i + (tid >> 2) < n ? x[i * kIn + tid] : 0.f;
+    if (kGrad && tid < tc::kS * (kIn + 1)) return i + (tid - tc::kS * kIn) < n ? t[i + (tid - tc::kS * kIn)] : 0.f;
+    return 0.f;
+  };
+  float ahead = fetch(blockIdx.x);
+  tc::stage_w(Wb[0], P + oW2, tid);
+  tc::stage_w(Wb[1], P + oW3, tid);
+  float w1[kIn];
 #pragma unroll
-  for (int c = 0; c < kIn; ++c) xin[c] = live ? x[(size_t)gs * kIn + c] : 0.f;
-  // Layer 1 (K = 4) on the CUDA cores, straight into the operand A.
-#pragma unroll 1
-  for (int j0 = u0; j0 < u0 + 32; j0 += 8) {
-    float h[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int j = j0 + i;
-      float z = bf(P + oB1, j);
-#pragma unroll
-      for (int c = 0; c < kIn; ++c) z += bf(P + oW1, j * kIn + c) * xin[c];
-      if (zsave && live) zsave[((size_t)gs * 3 + 0) * kW + j] = z;
-      h[i] = gelu(z);
-    }
-    tc::put8(Ahi, Alo, s, j0, h);
+  for (int c = 0; c < kIn; ++c) w1[c] = bf(P + oW1, u * kIn + c);
+  const float b1 = bf(P + oB1, u), b2 = bf(P + oB2, u), b3 = bf(P + oB3, u), w4 = bf(P + oW4, u), b4 = bf(P + oB4, 0);
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc::smem_u32(&mbar[0])));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc::smem_u32(&mbar[1])));
   }
-  tc::stage_w(Bs, P + oW2, tid);
-  if (tid == 0) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc::smem_u32(&mbar)));
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 128;" ::"r"(tc::smem_u32(&taddr_s)));
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc::smem_u32(&taddr_s)),
+                 "n"(kCols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   tc::fence_to_mma();
   const uint32_t taddr = taddr_s, lanes = taddr + ((uint32_t)((warp & 3) * 32) << 16);
-  const uint32_t mb = tc::smem_u32(&mbar);
+  const uint32_t mz = tc::smem_u32(&mbar[0]), mw = tc::smem_u32(&mbar[1]);
+  const uint32_t w2a = tc::smem_u32(Wb[0]), w3a = tc::smem_u32(Wb[1]);
+  uint32_t phase = 0, wphase = 0;
   bool ok = true;
-  const int oBl[2] = {oB2, oB3};
-  float out = 0.f;
+  float gw1[kIn] = {0.f, 0.f, 0.f, 0.f}, gb1 = 0.f, gb2 = 0.f, gb3 = 0.f, gw4 = 0.f, gb4 = 0.f, gsq = 0.f;
+  bool first = true;
 #pragma unroll 1
-  for (int layer = 0; layer < 2; ++layer) {
-    if (tid == 0) tc::mma_chain(taddr, tc::smem_u32(Ahi), tc::smem_u32(Alo), tc::smem_u32(Bs), mb);
-    ok = tc::wait_phase(mb, (uint32_t)layer) && ok;
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    float v[32];
-    tc::ld32(lanes + (uint32_t)u0, v);
-#pragma unroll
-    for (int g = 0; g < 32; g += 8) {
-      float h[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int j = u0 + g + i;
-        const float z = v[g + i] + bf(P + oBl[layer], j);
-        if (zsave && live) zsave[((size_t)gs * 3 + 1 + layer) * kW + j] = z;
-        h[i] = gelu(z);
-        if (layer == 1) out += bf(P + oW4, j) * h[i];
-      }
-      if (layer == 0) tc::put8(Ahi, Alo, s, u0 + g, h);
-    }
-    if (layer == 0) {
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncthreads();   // every lane read layer 2 and the MMAs are done with W2: restage
-      tc::stage_w(Bs, P + oW3, tid);
-      tc::fence_to_mma();
-    }
-  }
-  part[q][s] = out;
-  if (!ok) atomicExch(err, 1);
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  if (q == 0 && live) y[gs] = ((part[0][s] + part[1][s]) + part[2][s]) + part[3][s] + bf(P + oB4, 0);
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;" ::"r"(taddr));
-}
-
-namespace tc {
-
-// D (tensor memory) = sum over the npair operand pairs (a[i], b[i]) of
-// a[i] b[i]^T, K = 128 each, then commit to mbar.
-__device__ __forceinline__ void mma_pairs(uint32_t taddr, const uint32_t* a, const uint32_t* b, int npair,
-                                          uint32_t mbar) {
-#pragma unroll 1
-  for (int pr = 0; pr < npair; ++pr) {
-#pragma unroll
-    for (int kk = 0; kk < kW / 16; ++kk) {
-      const uint64_t ad = sdesc(a[pr] + kk * 256u);
-      const uint64_t bd = sdesc(b[pr] + kk * 256u);
-      const uint32_t acc = (pr | kk) ? 1u : 0u;
-      asm volatile(
-          "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-          " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(taddr),
-          "l"(ad), "l"(bd), "r"(kIdesc), "r"(acc));
-    }
-  }
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
-               : "memory");
-}
-
-// Element (row, k) of a pair of operands as bfloat16 hi and lo parts.
-__device__ __forceinline__ void put1(unsigned char* Xhi, unsigned char* Xlo, int row, int k, float v) {
-  const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-  *reinterpret_cast<__nv_bfloat16*>(Xhi + cm_off(row, k)) = hi;
-  *reinterpret_cast<__nv_bfloat16*>(Xlo + cm_off(row, k)) = __float2bfloat16_rn(v - __bfloat162float(hi));
-}
-__device__ __forceinline__ float get1(const unsigned char* Xhi, const unsigned char* Xlo, int row, int k) {
-  return __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(Xhi + cm_off(row, k))) +
-         __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(Xlo + cm_off(row, k)));
-}
-
-// W^T of a 128 x 128 bfloat16 weight matrix (row = output unit) into the
-// operand layout: element (k, u) = W[u][k].
-__device__ __forceinline__ void stage_wt(unsigned char* Bs, const __nv_bfloat16* W, int t) {
-#pragma unroll 2
-  for (int q = t; q < kW * kW / 8; q += kThreads) {
-    const int k = q & (kW - 1), u0 = (q >> 7) * 8;
-    __align__(16) __nv_bfloat16 v[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = W[(u0 + i) * kW + k];
-    *reinterpret_cast<uint4*>(Bs + cm_off(k, u0)) = *reinterpret_cast<const uint4*>(v);
-  }
-}
-
-}  // namespace tc
-
-// Backward pass of a tile of 128 samples: d(mean squared error)/d(parameters)
-// restricted to the tile's samples, written to its own slot of gpart (no
-// atomics). Per hidden layer (3, then 2) two tensor-core products: the weight
-// gradient dW[u][k] = sum_s dz[s][u] h[s][k] (M = units, K = samples; dz and h
-// split into bfloat16 hi and lo, three MMA chains hi.hi + hi.lo + lo.hi, in
-// tensor-memory columns 128..255) and the gradient at the layer's input
-// dh[s][k] = sum_u dz[s][u] W[u][k] (M = samples, K = units; two chains, in
-// columns 0..127). Thread (sample s, quarter q) handles units 32 q .. 32 q + 31
-// of sample s. Column sums over the samples (biases, the output and the first
-// layer) are taken per unit in four quarters of 32 samples, added in a fixed
-// order, so a call is deterministic.
-__global__ void __launch_bounds__(tc::kThreads, 1) bwd_kernel(const __nv_bfloat16* __restrict__ P,
-                                                              const float* __restrict__ x, const float* __restrict__ t,
-                                                              const float* __restrict__ y,
-                                                              const float* __restrict__ zsave, int n, float inv_n,
-                                                              float* __restrict__ gpart, int* __restrict__ err) {
-  extern __shared__ __align__(1024) unsigned char smem_tc[];
-  unsigned char* X0 = smem_tc;                       // operand buffers, 32 KB each
-  unsigned char* X1 = smem_tc + tc::kOpBytes;
-  unsigned char* X2 = smem_tc + 2 * tc::kOpBytes;
-  unsigned char* X3 = smem_tc + 3 * tc::kOpBytes;
-  float* dzT = reinterpret_cast<float*>(smem_tc);    // layer 1: dz1 as [unit][sample] float32 (X0, X1)
-  __shared__ float dy[tc::kM];
-  __shared__ float xs[tc::kM * kIn];
-  __shared__ float sq_part[4];
-  __shared__ float red[tc::kQ][tc::kM][kIn + 1];     // per-quarter column sums
-  __shared__ __align__(8) uint64_t mbar;
-  __shared__ uint32_t taddr_s;
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int s = (warp & 3) * 32 + (tid & 31), q = warp >> 2, u0 = 32 * q;   // sample role
-  const int uu = tid & (tc::kM - 1), qq = tid >> 7, k0 = 32 * qq;            // unit role: unit uu, samples k0..k0+31
-  const int s0 = blockIdx.x * tc::kM;
-  float* g = gpart + (size_t)blockIdx.x * kPart;
-  auto zval = [&](int smp, int layer, int u) -> float {   // zero beyond the last sample
-    return (s0 + smp < n) ? zsave[((size_t)(s0 + smp) * 3 + layer) * kW + u] : 0.f;
-  };
-  // Sum of the four quarters' partials of unit uu (fixed order), by the threads of quarter 0.
-  auto combine = [&](int c) -> float { return ((red[0][uu][c] + red[1][uu][c]) + red[2][uu][c]) + red[3][uu][c]; };
-  if (q == 0) {
-    const int gs = s0 + s;
-    const bool live = gs < n;
-#pragma unroll
-    for (int c = 0; c < kIn; ++c) xs[s * kIn + c] = live ? x[(size_t)gs * kIn + c] : 0.f;
-    const float r = live ? (y[gs] - t[gs]) : 0.f;
-    dy[s] = 2.f * r * inv_n;
-    float sq = r * r;
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, d);
-    if ((tid & 31) == 0) sq_part[warp] = sq;
-  }
-  if (tid == 0) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc::smem_u32(&mbar)));
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(tc::smem_u32(&taddr_s)));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t taddr = taddr_s, lanes = taddr + ((uint32_t)((warp & 3) * 32) << 16);
-  const uint32_t mb = tc::smem_u32(&mbar);
-  const uint32_t x0 = tc::smem_u32(X0), x1 = tc::smem_u32(X1), x2 = tc::smem_u32(X2), x3 = tc::smem_u32(X3);
-  uint32_t phase = 0;
-  bool ok = true;
-  if (tid == 0) g[kParams] = ((sq_part[0] + sq_part[1]) + sq_part[2]) + sq_part[3];
-  // Output layer: grads of w4 and b4.
-  {
-    float gw4 = 0.f, gb = 0.f;
-#pragma unroll
-    for (int k = k0; k < k0 + 32; ++k) {
-      gw4 += dy[k] * gelu(zval(k, 2, uu));
-      gb += dy[k];
-    }
-    red[qq][uu][0] = gw4;
-    red[qq][uu][1] = gb;
-  }
-  __syncthreads();
-  if (qq == 0) {
-    g[oW4 + uu] = combine(0);
-    if (uu == 0) g[oB4] = combine(1);
-  }
-  __syncthreads();
-  const int oW[2] = {oW3, oW2}, oB[2] = {oB3, oB2};
-#pragma unroll 1
-  for (int L = 0; L < 2; ++L) {
-    const int zl = 2 - L;   // pre-activation of this layer's output: z3, then z2
-    // dz (sample s, units u0..u0+31) -> X0/X1 transposed (row = unit), h at the
-    // layer's input -> X2/X3 transposed. Layer 3: dz3 = dy w4 gelu'(z3); layer 2:
-    // dz2 = dh2 gelu'(z2), dh2 from tensor memory.
-    {
-      float dh[32];
-      if (L == 1) tc::ld32(lanes + (uint32_t)u0, dh);
-#pragma unroll 16
-      for (int i = 0; i < 32; ++i) {
-        const int u = u0 + i;
-        const float d = (L == 0) ? dy[s] * bf(P + oW4, u) : dh[i];
-        tc::put1(X0, X1, u, s, d * gelu_grad(zval(s, zl, u)));
-        tc::put1(X2, X3, u, s, gelu(zval(s, zl - 1, u)));
-      }
-    }
-    tc::fence_to_mma();
-    // Bias gradient: column sum of dz over the samples.
-    {
-      float db = 0.f;
-#pragma unroll 8
-      for (int k = k0; k < k0 + 32; ++k) db += tc::get1(X0, X1, uu, k);
-      red[qq][uu][0] = db;
-    }
-    __syncthreads();   // every column read before X0/X1 are rewritten below
-    if (qq == 0) g[oB[L] + uu] = combine(0);
-    // dW[u][k] into columns 128..255.
-    if (tid == 0) {
-      const uint32_t a[3] = {x0, x0, x1}, b[3] = {x2, x3, x2};
-      tc::mma_pairs(taddr + 128u, a, b, 3, mb);
-    }
-    ok = tc::wait_phase(mb, phase) && ok;
-    phase ^= 1u;
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    {
-      float v[32];
-      tc::ld32(lanes + 128u + (uint32_t)u0, v);    // row = unit s, columns u0..u0+31
-      float* dst = g + oW[L] + s * kW + u0;        // a tile's slot is not 16-byte aligned: scalar stores
-#pragma unroll
-      for (int i = 0; i < 32; ++i) dst[i] = v[i];
-    }
-    // dz again, now as rows (sample s) in X0/X1; W^T in X2.
-    {
-      float dh[32];
-      if (L == 1) tc::ld32(lanes + (uint32_t)u0, dh);
-#pragma unroll
-      for (int g8 = 0; g8 < 32; g8 += 8) {
-        float d8[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int u = u0 + g8 + i;
-          const float d = (L == 0) ? dy[s] * bf(P + oW4, u) : dh[g8 + i];
-          d8[i] = d * gelu_grad(zval(s, zl, u));
-        }
-        tc::put8(X0, X1, s, u0 + g8, d8);
-      }
-    }
-    tc::stage_wt(X2, P + oW[L], tid);
-    tc::fence_to_mma();
-    // dh at the layer's input into columns 0..127.
-    if (tid == 0) {
-      const uint32_t a[2] = {x0, x1}, b[2] = {x2, x2};
-      tc::mma_pairs(taddr, a, b, 2, mb);
-    }
-    ok = tc::wait_phase(mb, phase) && ok;
-    phase ^= 1u;
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    if (tid < tc::kS * kIn) xs[tid] = ahead;
+    else if (kGrad && tid < tc::kS * (kIn + 1)) ts[tid - tc::kS * kIn] = ahead;
     __syncthreads();
-  }
-  // First layer: dz1 = dh1 gelu'(z1) into dzT[u][s], then per unit
-  // dW1[u][c] = sum_s dz1 x[s][c], db1[u] = sum_s dz1.
-  {
-    float dh[32];
-    tc::ld32(lanes + (uint32_t)u0, dh);
+    ahead = fetch(tile + (int)gridDim.x);
+    float h[8], d1[8], d2[8], d3[8], z[8];
+    // Layer 1 (K = 4) on the CUDA cores.
 #pragma unroll
-    for (int i = 0; i < 32; ++i) dzT[(u0 + i) * tc::kM + s] = dh[i] * gelu_grad(zval(s, 0, u0 + i));
-  }
-  __syncthreads();
-  {
-    float a[kIn] = {0.f, 0.f, 0.f, 0.f}, db = 0.f;
-#pragma unroll 8
-    for (int k = k0; k < k0 + 32; ++k) {
-      const float d = dzT[uu * tc::kM + k];
-      db += d;
+    for (int i = 0; i < 8; ++i) {
+      float v = b1;
 #pragma unroll
-      for (int c = 0; c < kIn; ++c) a[c] += d * xs[k * kIn + c];
+      for (int c = 0; c < kIn; ++c) v += w1[c] * xs[(s0 + i) * kIn + c];
+      h[i] = tc::gelu<kGrad>(v, d1[i]);
     }
+    tc::put8(buf(iH1), buf(iH1 + 1), u, g, h);
+    tc::fence_to_mma();
+    if (tid == 0) {
+      tc::mma_forward(taddr, w2a, tc::smem_u32(buf(iH1)), tc::smem_u32(buf(iH1 + 1)));
+      tc::commit(mz);
+    }
+    ok = tc::wait_phase(mz, phase) && ok;
+    phase ^= 1u;
+    tc::ld8(lanes + (uint32_t)s0, z);
 #pragma unroll
-    for (int c = 0; c < kIn; ++c) red[qq][uu][c] = a[c];
-    red[qq][uu][kIn] = db;
-  }
-  __syncthreads();
-  if (qq == 0) {
+    for (int i = 0; i < 8; ++i) h[i] = tc::gelu<kGrad>(z[i] + b2, d2[i]);
+    tc::put8(buf(iH2), buf(iH2 + 1), u, g, h);
+    tc::fence_to_mma();
+    if (tid == 0) {
+      tc::mma_forward(taddr, w3a, tc::smem_u32(buf(iH2)), tc::smem_u32(buf(iH2 + 1)));
+      tc::commit(mz);
+    }
+    ok = tc::wait_phase(mz, phase) && ok;
+    phase ^= 1u;
+    tc::ld8(lanes + (uint32_t)s0, z);
 #pragma unroll
-    for (int c = 0; c < kIn; ++c) g[oW1 + uu * kIn + c] = combine(c);
-    g[oB1 + uu] = combine(kIn);
+    for (int i = 0; i < 8; ++i) h[i] = tc::gelu<kGrad>(z[i] + b3, d3[i]);
+    // Output: sum over the units, 32 by shuffles, then the four warps of a sample group.
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      float o = w4 * h[i];
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1) o += __shfl_xor_sync(0xffffffffu, o, d);
+      if (lane == i) part[warp & 3][s0 + i] = o;
+    }
+    __syncthreads();
+    if (!kGrad) {
+      const int s = tile * tc::kS + tid;
+      if (tid < tc::kS && s < n) y[s] = ((part[0][tid] + part[1][tid]) + part[2][tid]) + part[3][tid] + b4;
+      __syncthreads();   // part is written again by the next tile
+      continue;
+    }
+    float dy[8];
+    float sg4 = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int s = s0 + i;
+      const float o = ((part[0][s] + part[1][s]) + part[2][s]) + part[3][s] + b4;
+      const float r = tile * tc::kS + s < n ? o - ts[s] : 0.f;
+      dy[i] = 2.f * r * inv_n;
+      sg4 += dy[i];
+      gsq += r * r;
+    }
+    gb4 += sg4;
+    // Layer 3: dz3 = dy w4 gelu'(z3); its products with h2 and W3.
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      gw4 += dy[i] * h[i];
+      h[i] = dy[i] * w4 * d3[i];
+      gb3 += h[i];
+    }
+    tc::put8(buf(iD3), buf(iD3 + 1), u, g, h);
+    tc::fence_to_mma();
+    if (tid == 0) {
+      tc::mma_input(taddr, w3a, tc::smem_u32(buf(iD3)), tc::smem_u32(buf(iD3 + 1)));
+      tc::commit(mz);
+      tc::mma_weight(taddr + 32u, tc::smem_u32(buf(iD3)), tc::smem_u32(buf(iD3 + 1)), tc::smem_u32(buf(iH2)),
+                     tc::smem_u32(buf(iH2 + 1)), !first);
+    }
+    ok = tc::wait_phase(mz, phase) && ok;
+    phase ^= 1u;
+    tc::ld8(lanes + (uint32_t)s0, z);
+    // Layer 2: dz2 = dh2 gelu'(z2).
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      h[i] = z[i] * d2[i];
+      gb2 += h[i];
+    }
+    tc::put8(buf(iD2), buf(iD2 + 1), u, g, h);
+    tc::fence_to_mma();
+    if (tid == 0) {
+      tc::mma_input(taddr, w2a, tc::smem_u32(buf(iD2)), tc::smem_u32(buf(iD2 + 1)));
+      tc::commit(mz);
+      tc::mma_weight(taddr + 160u, tc::smem_u32(buf(iD2)), tc::smem_u32(buf(iD2 + 1)), tc::smem_u32(buf(iH1)),
+                     tc::smem_u32(buf(iH1 + 1)), !first);
+      tc::commit(mw);
+    }
+    ok = tc::wait_phase(mz, phase) && ok;
+    phase ^= 1u;
+    tc::ld8(lanes + (uint32_t)s0, z);
+    // Layer 1: dz1 = dh1 gelu'(z1).
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float d = z[i] * d1[i];
+      gb1 += d;
+#pragma unroll
+      for (int c = 0; c < kIn; ++c) gw1[c] += d * xs[(s0 + i) * kIn + c];
+    }
+    ok = tc::wait_phase(mw, wphase) && ok;   // the operands of the weight products are free again
+    wphase ^= 1u;
+    first = false;
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();   // xs, ts and part are written again by the next tile
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   }
-  if (!ok) atomicExch(err, 1);
+  if (kGrad) {
+    float* o = gpart + (size_t)blockIdx.x * kPart;
+    // Sums over the four sample groups, in a fixed order.
+    auto combine = [&](int c) -> float { return ((red[0][u][c] + red[1][u][c]) + red[2][u][c]) + red[3][u][c]; };
+#pragma unroll
+    for (int c = 0; c < kIn; ++c) red[g][u][c] = gw1[c];
+    red[g][u][kIn] = gb1;
+    __syncthreads();
+    if (g == 0) {
+#pragma unroll
+      for (int c = 0; c < kIn; ++c) o[oW1 + u * kIn + c] = combine(c);
+      o[oB1 + u] = combine(kIn);
+    }
+    __syncthreads();
+    red[g][u][0] = gb2;
+    red[g][u][1] = gb3;
+    red[g][u][2] = gw4;
+    red[g][u][3] = gb4;   // the same for every unit of a group
+    red[g][u][4] = gsq;
+    __syncthreads();
+    if (g == 0) {
+      o[oB2 + u] = combine(0);
+      o[oB3 + u] = combine(1);
+      o[oW4 + u] = combine(2);
+      if (u == 0) {
+        o[oB4] = combine(3);
+        o[kParams] = combine(4);
+      }
+    }
+    // Weight gradients: row u, columns 32 g .. 32 g + 31 of each matrix.
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+      float v[32];
+      tc::ld32(lanes + (m ? 160u : 32u) + 32u * (uint32_t)g, v);
+      float4* dst = reinterpret_cast<float4*>(o + (m ? oW2 : oW3) + u * kW + 32 * g);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+    }
+  }
+  if (!ok) {
+    *(volatile int*)err = 1;
+    __threadfence_system();
+  }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(taddr));
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "n"(kCols));
 }
 
-// grad[i] = sum over tiles b of gpart[b][i], tiles in order (deterministic).
-__global__ void reduce_kernel(const float* __restrict__ gpart, int ntiles, float* __restrict__ grad) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= kPart) return;
+// Sum over the blocks' partials, in order (deterministic).
+__device__ __forceinline__ float reduce_one(const float* __restrict__ gpart, int nparts, int i) {
   float s = 0.f;
-  for (int b = 0; b < ntiles; ++b) s += gpart[(size_t)b * kPart + i];
-  grad[i] = s;
+  int b = 0;
+  for (; b + 8 <= nparts; b += 8) {
+    float v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = gpart[(size_t)(b + k) * kPart + i];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s += v[k];
+  }
+  for (; b < nparts; ++b) s += gpart[(size_t)b * kPart + i];
+  return s;
 }
 
-// Adam (Kingma and Ba): master weights in float32, bfloat16 copy for the passes.
-__global__ void adam_kernel(float* __restrict__ theta, float* __restrict__ m, float* __restrict__ v,
-                            const float* __restrict__ grad, __nv_bfloat16* __restrict__ P, float lr, float b1,
-                            float b2, float c1, float c2, float eps) {
+// grad[i] (may be null) and the sum of squared errors; both may be host memory.
+__global__ void reduce_kernel(const float* __restrict__ gpart, int nparts, float* __restrict__ grad, float* sq) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= kParams) return;
-  const float gi = grad[i];
+  if (i > kParams || (i < kParams && !grad)) return;
+  const float s = reduce_one(gpart, nparts, i);
+  if (i < kParams) grad[i] = s;
+  else *sq = s;
+}
+
+// Reduction and Adam (Kingma and Ba): master weights in float32, bfloat16 copy for the passes.
+__global__ void adam_kernel(const float* __restrict__ gpart, int nparts, float* __restrict__ theta, float* __restrict__ m,
+                            float* __restrict__ v, __nv_bfloat16* __restrict__ P, float* sq, float lr, float b1, float b2,
+                            float c1, float c2, float eps) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i > kParams) return;
+  const float gi = reduce_one(gpart, nparts, i);
+  if (i == kParams) {
+    *sq = gi;
+    return;
+  }
   const float mi = b1 * m[i] + (1.f - b1) * gi;
   const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
   m[i] = mi;
@@ -513,8 +482,6 @@ __global__ void to_bf16_kernel(const float* __restrict__ theta, __nv_bfloat16* _
   if (i < kParams) P[i] = __float2bfloat16_rn(theta[i]);
 }
 
-constexpr size_t kBwdSmem = 4 * (size_t)tc::kOpBytes;   // four tensor-core operand buffers
-
 }  // namespace mlp
 }  // namespace kpz
 
@@ -523,84 +490,89 @@ using namespace kpz::mlp;
 
 struct kpz_mlp {
   int device = 0;
+  int sms = 0;
+  bool direct_host = false;     // the GPU reads and writes pageable host memory itself
   cudaStream_t stream = nullptr;
   float* theta = nullptr;       // master parameters
   float* m = nullptr;
   float* v = nullptr;
-  float* grad = nullptr;        // kPart (last entry: squared-error sum)
   __nv_bfloat16* P = nullptr;   // bfloat16 copy
   uint64_t step = 0;
-  // per-call buffers: data (x, t) for `cap` samples, work (y, z, gpart) for `wcap`
-  float *x = nullptr, *t = nullptr, *y = nullptr, *z = nullptr, *gpart = nullptr;
-  size_t cap = 0, wcap = 0;
-  int* err = nullptr;           // set by the forward kernel when a tensor-core wait timed out
+  // per-call buffers: data (x, t, y) for `cap` samples, partials of `pcap` blocks, a gradient
+  float *x = nullptr, *t = nullptr, *y = nullptr, *gpart = nullptr, *grad = nullptr;
+  size_t cap = 0, pcap = 0;
+  struct Host { int err; float sq; };
+  Host* host = nullptr;         // pinned: set when a tensor-core wait timed out; sum of squared errors
 };
 
 namespace {
 
 void mlp_release(kpz_mlp* m) {
-  float* ptrs[] = {m->theta, m->m, m->v, m->grad, m->x, m->t, m->y, m->z, m->gpart};
+  float* ptrs[] = {m->theta, m->m, m->v, m->grad, m->x, m->t, m->y, m->gpart};
   for (float* p : ptrs) if (p) cudaFree(p);
   if (m->P) cudaFree(m->P);
-  if (m->err) cudaFree(m->err);
+  if (m->host) cudaFreeHost(m->host);
 }
 
-// KPZ_OK, or KPZ_ETIMEOUT when a forward kernel's tensor-core wait ran out
-// (the flag is then cleared); the stream is synchronised.
-kpz_status check_err(kpz_mlp* m) {
-  int e = 0;
-  if (cudaMemcpyAsync(&e, m->err, 4, cudaMemcpyDeviceToHost, m->stream) != cudaSuccess ||
-      cudaStreamSynchronize(m->stream) != cudaSuccess)
-    return KPZ_ECUDA;
-  if (e) {
-    cudaMemsetAsync(m->err, 0, 4, m->stream);
+// Synchronises the stream; KPZ_ETIMEOUT when a kernel's tensor-core wait ran
+// out (the flag is then cleared).
+kpz_status finish(kpz_mlp* m) {
+  if (cudaStreamSynchronize(m->stream) != cudaSuccess) return KPZ_ECUDA;
+  volatile kpz_mlp::Host* h = m->host;
+  if (h->err) {
+    h->err = 0;
     return KPZ_ETIMEOUT;
   }
   return KPZ_OK;
 }
 
-// Data buffers for n samples and work buffers for passes over w samples.
-kpz_status ensure(kpz_mlp* m, size_t n, size_t w) {
-  if (n > m->cap) {
-    if (m->x) cudaFree(m->x);
-    if (m->t) cudaFree(m->t);
-    m->x = m->t = nullptr;
-    m->cap = 0;
-    if (cudaMalloc(&m->x, n * kIn * 4) != cudaSuccess || cudaMalloc(&m->t, n * 4) != cudaSuccess) {
-      cudaGetLastError();
-      return KPZ_ENOMEM;
-    }
-    m->cap = n;
+// Device buffers for n samples.
+kpz_status ensure_data(kpz_mlp* m, size_t n) {
+  if (n <= m->cap) return KPZ_OK;
+  float** bufs[] = {&m->x, &m->t, &m->y};
+  for (float** p : bufs) {
+    if (*p) cudaFree(*p);
+    *p = nullptr;
   }
-  if (w > m->wcap) {
-    float* bufs[] = {m->y, m->z, m->gpart};
-    for (float* p : bufs) if (p) cudaFree(p);
-    m->y = m->z = m->gpart = nullptr;
-    m->wcap = 0;
-    const size_t tiles = (w + tc::kM - 1) / tc::kM;
-    if (cudaMalloc(&m->y, w * 4) != cudaSuccess || cudaMalloc(&m->z, w * 3 * kW * 4) != cudaSuccess ||
-        cudaMalloc(&m->gpart, tiles * kPart * 4) != cudaSuccess) {
-      cudaGetLastError();
-      return KPZ_ENOMEM;
-    }
-    m->wcap = w;
+  m->cap = 0;
+  if (cudaMalloc(&m->x, n * kIn * 4) != cudaSuccess || cudaMalloc(&m->t, n * 4) != cudaSuccess ||
+      cudaMalloc(&m->y, n * 4) != cudaSuccess) {
+    cudaGetLastError();
+    return KPZ_ENOMEM;
   }
+  m->cap = n;
   return KPZ_OK;
 }
 
-// Gradient of the mean squared error over samples [0, n) of the uploaded
-// data into m->grad; y and z are filled on the way.
-cudaError_t grad_pass(kpz_mlp* m, const float* x, const float* t, int n) {
-  const int tiles = (n + tc::kM - 1) / tc::kM;
-  fwd_kernel<<<tiles, tc::kThreads, tc::kSmem, m->stream>>>(m->P, x, n, m->y, m->z, m->err);
-  count_launch();
-  bwd_kernel<<<tiles, tc::kThreads, kBwdSmem, m->stream>>>(m->P, x, t, m->y, m->z, n, 1.f / (float)n, m->gpart,
-                                                      m->err);
-  count_launch();
-  reduce_kernel<<<(kPart + 255) / 256, 256, 0, m->stream>>>(m->gpart, tiles, m->grad);
-  count_launch();
-  return cudaGetLastError();
+int tiles_of(size_t n) { return (int)((n + tc::kS - 1) / tc::kS); }
+int grad_blocks(const kpz_mlp* m, size_t n) { return std::min(tiles_of(n), m->sms); }
+
+// Partials for gradients over n samples.
+kpz_status ensure_parts(kpz_mlp* m, size_t n) {
+  const size_t b = (size_t)grad_blocks(m, n);
+  if (b <= m->pcap) return KPZ_OK;
+  if (m->gpart) cudaFree(m->gpart);
+  m->gpart = nullptr;
+  m->pcap = 0;
+  if (cudaMalloc(&m->gpart, b * kPart * 4) != cudaSuccess) {
+    cudaGetLastError();
+    return KPZ_ENOMEM;
+  }
+  m->pcap = b;
+  return KPZ_OK;
 }
+
+// Partial gradients of the mean squared error over n samples; returns the
+// number of partials.
+int queue_grad(kpz_mlp* m, const float* x, const float* t, int n) {
+  const int blocks = grad_blocks(m, (size_t)n);
+  net_kernel<true><<<blocks, tc::kThreads, tc::kSmemGrad, m->stream>>>(m->P, x, t, n, 1.f / (float)n, nullptr, m->gpart,
+                                                                      &m->host->err);
+  count_launch();
+  return blocks;
+}
+
+constexpr unsigned kReduceBlocks = (kParams + 1 + 255) / 256;
 
 }  // namespace
 
@@ -614,18 +586,25 @@ kpz_status kpz_mlp_create(kpz_mlp** out, const float* params, void* stream) {
   kpz_mlp* m = new (std::nothrow) kpz_mlp();
   if (!m) return KPZ_ENOMEM;
   cudaGetDevice(&m->device);
+  cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, m->device);
+  m->sms = std::max(m->sms, 1);
+  m->direct_host = reaches_pageable(m->device);
   m->stream = (cudaStream_t)stream;
   if (cudaMalloc(&m->theta, kParams * 4) != cudaSuccess || cudaMalloc(&m->m, kParams * 4) != cudaSuccess ||
-      cudaMalloc(&m->v, kParams * 4) != cudaSuccess || cudaMalloc(&m->grad, kPart * 4) != cudaSuccess ||
-      cudaMalloc(&m->P, kParams * 2) != cudaSuccess || cudaMalloc(&m->err, 4) != cudaSuccess) {
+      cudaMalloc(&m->v, kParams * 4) != cudaSuccess || cudaMalloc(&m->grad, kParams * 4) != cudaSuccess ||
+      cudaMalloc(&m->P, kParams * 2) != cudaSuccess ||
+      cudaHostAlloc((void**)&m->host, sizeof(*m->host), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
     cudaGetLastError();
     mlp_release(m);
     delete m;
     return KPZ_ENOMEM;
   }
-  if (cudaFuncSetAttribute(bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBwdSmem) != cudaSuccess ||
-      cudaFuncSetAttribute(fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kSmem) != cudaSuccess ||
-      cudaMemsetAsync(m->err, 0, 4, m->stream) != cudaSuccess ||
+  m->host->err = 0;
+  m->host->sq = 0.f;
+  if (cudaFuncSetAttribute(net_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kSmemGrad) !=
+          cudaSuccess ||
+      cudaFuncSetAttribute(net_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kSmemPredict) !=
+          cudaSuccess ||
       cudaMemcpyAsync(m->theta, params, kParams * 4, cudaMemcpyHostToDevice, m->stream) != cudaSuccess ||
       cudaMemsetAsync(m->m, 0, kParams * 4, m->stream) != cudaSuccess ||
       cudaMemsetAsync(m->v, 0, kParams * 4, m->stream) != cudaSuccess) {
@@ -652,37 +631,59 @@ kpz_status kpz_mlp_params(kpz_mlp* m, float* params) {
   return KPZ_OK;
 }
 
+// Where the GPU reaches pageable host memory (its pages touched before it
+// writes them), predict and loss_grad read and write the caller's arrays in the
+// kernels: a launch or two and one synchronisation instead of four copies.
 kpz_status kpz_mlp_predict(kpz_mlp* m, const float* x, uint32_t n, float* y) {
   if (!m || !x || !y) return KPZ_EINVAL;
   if (n == 0) return KPZ_OK;
-  kpz_status st = ensure(m, n, n);
-  if (st) return st;
-  if (cudaMemcpyAsync(m->x, x, (size_t)n * kIn * 4, cudaMemcpyHostToDevice, m->stream) != cudaSuccess)
-    return KPZ_ECUDA;
-  fwd_kernel<<<(n + tc::kM - 1) / tc::kM, tc::kThreads, tc::kSmem, m->stream>>>(m->P, m->x, (int)n, m->y, nullptr,
-                                                                         m->err);
+  const float* xin = x;
+  float* yout = y;
+  if (m->direct_host) {
+    touch_pages(y, (size_t)n * 4);
+  } else {
+    kpz_status st = ensure_data(m, n);
+    if (st) return st;
+    if (cudaMemcpyAsync(m->x, x, (size_t)n * kIn * 4, cudaMemcpyHostToDevice, m->stream) != cudaSuccess) return KPZ_ECUDA;
+    xin = m->x;
+    yout = m->y;
+  }
+  net_kernel<false><<<std::min(tiles_of(n), 2 * m->sms), tc::kThreads, tc::kSmemPredict, m->stream>>>(
+      m->P, xin, nullptr, (int)n, 0.f, yout, nullptr, &m->host->err);
   count_launch();
   if (cudaGetLastError() != cudaSuccess ||
-      cudaMemcpyAsync(y, m->y, (size_t)n * 4, cudaMemcpyDeviceToHost, m->stream) != cudaSuccess)
+      (!m->direct_host && cudaMemcpyAsync(y, m->y, (size_t)n * 4, cudaMemcpyDeviceToHost, m->stream) != cudaSuccess))
     return KPZ_ECUDA;
-  return check_err(m);
+  return finish(m);
 }
 
 kpz_status kpz_mlp_loss_grad(kpz_mlp* m, const float* x, const float* t, uint32_t n, float* loss, float* grad) {
   if (!m || !x || !t || n == 0) return KPZ_EINVAL;
-  kpz_status st = ensure(m, n, n);
+  kpz_status st = ensure_parts(m, n);
   if (st) return st;
-  if (cudaMemcpyAsync(m->x, x, (size_t)n * kIn * 4, cudaMemcpyHostToDevice, m->stream) != cudaSuccess ||
-      cudaMemcpyAsync(m->t, t, (size_t)n * 4, cudaMemcpyHostToDevice, m->stream) != cudaSuccess ||
-      grad_pass(m, m->x, m->t, (int)n) != cudaSuccess)
+  const float *xin = x, *tin = t;
+  float* gout = grad;
+  if (m->direct_host) {
+    if (grad) touch_pages(grad, kParams * 4);
+  } else {
+    if ((st = ensure_data(m, n)) != KPZ_OK) return st;
+    if (cudaMemcpyAsync(m->x, x, (size_t)n * kIn * 4, cudaMemcpyHostToDevice, m->stream) != cudaSuccess ||
+        cudaMemcpyAsync(m->t, t, (size_t)n * 4, cudaMemcpyHostToDevice, m->stream) != cudaSuccess)
+      return KPZ_ECUDA;
+    xin = m->x;
+    tin = m->t;
+    gout = grad ? m->grad : nullptr;
+  }
+  const int parts = queue_grad(m, xin, tin, (int)n);
+  reduce_kernel<<<kReduceBlocks, 256, 0, m->stream>>>(m->gpart, parts, gout, &m->host->sq);
+  count_launch();
+  if (cudaGetLastError() != cudaSuccess ||
+      (grad && !m->direct_host &&
+       cudaMemcpyAsync(grad, m->grad, kParams * 4, cudaMemcpyDeviceToHost, m->stream) != cudaSuccess))
     return KPZ_ECUDA;
-  std::vector<float> h(kPart);
-  if (cudaMemcpyAsync(h.data(), m->grad, kPart * 4, cudaMemcpyDeviceToHost, m->stream) != cudaSuccess ||
-      cudaStreamSynchronize(m->stream) != cudaSuccess)
-    return KPZ_ECUDA;
-  if (grad) for (int i = 0; i < kParams; ++i) grad[i] = h[i];
-  if (loss) *loss = h[kParams] / (float)n;
-  return check_err(m);
+  st = finish(m);
+  if (loss) *loss = *(volatile float*)&m->host->sq / (float)n;
+  return st;
 }
 
 kpz_status kpz_mlp_train(kpz_mlp* m, const float* x, const float* t, uint32_t n, const uint32_t* order,
@@ -692,7 +693,8 @@ kpz_status kpz_mlp_train(kpz_mlp* m, const float* x, const float* t, uint32_t n,
   // step s uses samples order[s*batch .. s*batch + batch - 1] (indices < n).
   const size_t total = (size_t)steps * batch;
   for (size_t i = 0; i < total; ++i) if (order[i] >= n) return KPZ_EINVAL;
-  kpz_status st = ensure(m, total, batch);
+  kpz_status st = ensure_data(m, total);
+  if (st == KPZ_OK) st = ensure_parts(m, batch);
   if (st) return st;
   std::vector<float> xg(total * kIn), tg(total);
   for (size_t i = 0; i < total; ++i) {
@@ -703,22 +705,19 @@ kpz_status kpz_mlp_train(kpz_mlp* m, const float* x, const float* t, uint32_t n,
       cudaMemcpyAsync(m->t, tg.data(), total * 4, cudaMemcpyHostToDevice, m->stream) != cudaSuccess)
     return KPZ_ECUDA;
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+  m->host->sq = 0.f;
   for (uint32_t s = 0; s < steps; ++s) {
     ++m->step;
     const float c1 = 1.f - std::pow(b1, (float)m->step), c2 = 1.f - std::pow(b2, (float)m->step);
-    if (grad_pass(m, m->x + (size_t)s * batch * kIn, m->t + (size_t)s * batch, (int)batch) != cudaSuccess)
-      return KPZ_ECUDA;
-    adam_kernel<<<(kParams + 255) / 256, 256, 0, m->stream>>>(m->theta, m->m, m->v, m->grad, m->P, lr, b1, b2,
-                                                             c1, c2, eps);
+    const int parts = queue_grad(m, m->x + (size_t)s * batch * kIn, m->t + (size_t)s * batch, (int)batch);
+    adam_kernel<<<kReduceBlocks, 256, 0, m->stream>>>(m->gpart, parts, m->theta, m->m, m->v, m->P, &m->host->sq, lr, b1, b2,
+                                                      c1, c2, eps);
     count_launch();
   }
-  float sq = 0.f;
-  if (cudaGetLastError() != cudaSuccess ||
-      cudaMemcpyAsync(&sq, m->grad + kParams, 4, cudaMemcpyDeviceToHost, m->stream) != cudaSuccess ||
-      cudaStreamSynchronize(m->stream) != cudaSuccess)
-    return KPZ_ECUDA;
-  if (last_loss) *last_loss = sq / (float)batch;
-  return check_err(m);
+  if (cudaGetLastError() != cudaSuccess) return KPZ_ECUDA;
+  st = finish(m);
+  if (last_loss) *last_loss = *(volatile float*)&m->host->sq / (float)batch;
+  return st;
 }
 
 void kpz_mlp_free(kpz_mlp* m) {
