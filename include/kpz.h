@@ -102,9 +102,8 @@ typedef struct {
                              (attempt a at the site drawn from Philox tag 4),
                              run as rounds of non-neighbouring sites whose
                              next attempt is the earliest around them; needs
-                             L <= 8192, allocates about 20 L^2 bytes of
-                             scratch itself (not in kpz_device_bytes) and
-                             synchronises the stream every sweep.
+                             L <= 8192 and allocates 20 L^2 bytes of
+                             scratch itself (not in kpz_device_bytes).
                              2, 3 and 4 need 128 x 128 tiles                   */
     uint32_t cell;        /* work-group layer cell edge (Sec. 3.1): 4 (0 = 4):
                              4 x 4 cells, 2 x 2 quadrant sets, 16 rounds per

@@ -46,10 +46,10 @@ struct kpz_ctx {
   long long* sums = nullptr;           // pinned host memory: results of the roughness kernel
   uint32_t* hcar = nullptr;            // import: height of (0, j0) modulo 4
   uint32_t* queue = nullptr;           // sweep work queue (zero between launches)
-  ResidentSync* sync = nullptr;        // resident kernels: grid barrier and error flag
+  GridSync* sync = nullptr;            // persistent kernels: grid barrier and error flag
   uint32_t resident = 0;               // kpz_run's resident kernel (resident_kind), 0: one launch per sweep
   bool direct_host = false;            // the GPU reads and writes pageable host memory itself
-  bool unchecked = false;              // resident launches since the error flag was read
+  bool unchecked = false;              // persistent launches since the error flag was read
   int32_t* col0 = nullptr;             // h(0,j); roughness: the bands' partial sums
   void* io = nullptr;                  // staging band for host transfers
   size_t io_bytes = 0;
@@ -86,7 +86,7 @@ Layout layout(uint32_t L) {
   Layout y{};
   const size_t lat_bytes = (size_t)L * L / 8;   // 1 bit per site
   y.lat = 0;
-  y.small = align_up(lat_bytes);                 // t, h00, hcar, queue, ticket; at +128 ResidentSync
+  y.small = align_up(lat_bytes);                 // t, h00, hcar, queue, ticket; at +128 GridSync
   y.col0 = y.small + kAlign;
   y.io = y.col0 + align_up((size_t)L * 4);
   const size_t io_bytes = std::min(kIoMax, (size_t)L * L / 4);
@@ -151,7 +151,7 @@ uint32_t io_band_rows(const kpz_ctx* c, size_t row_bytes, size_t* half) {
   return (uint32_t)std::min<size_t>(c->g.L, *half / row_bytes) & ~3u;
 }
 
-// Reads the resident kernels' error flag if launches are outstanding; for
+// Reads the persistent kernels' error flag if launches are outstanding; for
 // calls that synchronise and do not read the block of small values anyway.
 kpz_status settle(kpz_ctx* ctx) {
   if (!ctx->unchecked) return KPZ_OK;
@@ -309,7 +309,7 @@ kpz_status kpz_init(kpz_ctx** out, uint32_t L, double p, double q, uint64_t seed
   ctx->ticket = (uint32_t*)(base + y.small + 56);
   ctx->hcar = (uint32_t*)(base + y.small + 40);
   ctx->queue = (uint32_t*)(base + y.small + 48);
-  ctx->sync = (ResidentSync*)(base + y.small + 128);
+  ctx->sync = (GridSync*)(base + y.small + 128);
   ctx->col0 = (int32_t*)(base + y.col0);
   ctx->io = base + y.io;
   ctx->io_bytes = y.total - y.io;
@@ -344,10 +344,13 @@ kpz_status kpz_run(kpz_ctx* ctx, uint64_t n_mcs) {
   SweepParams P = sweep_params(ctx);
   while (n_mcs > 0) {
     // A resident launch takes 65536 sweeps at most (0.15 to 1.4 s).
-    const uint32_t chunk = (uint32_t)std::min<uint64_t>(n_mcs, ctx->resident ? 1u << 16 : 1u << 20);
-    if (ctx->resident) {
+    // (random-sequential: 1024, 0.1 to 10 s)
+    const bool rsu = ctx->decomposition == 4u;
+    const uint32_t chunk = (uint32_t)std::min<uint64_t>(n_mcs, rsu ? 1u << 10 : ctx->resident ? 1u << 16 : 1u << 20);
+    if (rsu || ctx->resident) {
       ctx->unchecked = true;
-      KPZ_CUDA(launch_resident(P, ctx->decomposition == 1u, ctx->resident, chunk, (uint32_t*)ctx->io, ctx->sync, ctx->stream));
+      if (rsu) KPZ_CUDA(launch_rsu(P, chunk, ctx->rsu_scratch, ctx->sync, ctx->stream));
+      else KPZ_CUDA(launch_resident(P, ctx->decomposition == 1u, ctx->resident, chunk, (uint32_t*)ctx->io, ctx->sync, ctx->stream));
       ctx->t_host += chunk;
       n_mcs -= chunk;
       continue;
@@ -357,7 +360,6 @@ kpz_status kpz_run(kpz_ctx* ctx, uint64_t n_mcs) {
       if (ctx->decomposition == 1u)      KPZ_CUDA(launch_sweep_tilesets(P, ctx->stream));
       else if (ctx->decomposition == 2u) KPZ_CUDA(launch_sweep_colour(P, ctx->colour_m, ctx->stream));
       else if (ctx->decomposition == 3u) KPZ_CUDA(launch_sweep_db2(P, ctx->stream));
-      else if (ctx->decomposition == 4u) KPZ_CUDA(launch_sweep_rsu(P, ctx->rsu_scratch, ctx->stream));
       else                               KPZ_CUDA(launch_sweep(P, ctx->wpc, ctx->stream));
     }
     KPZ_CUDA(launch_advance(ctx->t_dev, chunk, ctx->stream));

@@ -256,9 +256,11 @@ __global__ void __launch_bounds__(kCol0Threads) col0_kernel(const uint32_t* __re
 // A1^2, so a run costs one table entry {8D << 16 | V, A1}, whose first word is
 // also the running height: m from one shift-add, m and m^2 accumulated.
 // The per-run unpacking of D, A1, A2 and the three-term update it replaces
-// took 2.57 instructions a site.
-constexpr uint32_t kBandRows = 32, kBandCells = kBandRows / 4u, kBandThreads = 256, kSegs = 8;
-constexpr size_t kRunTab2Bytes = 256u * 32u * sizeof(uint2);   // one copy per lane
+// took 2.57 instructions a site (0.43 ms at L = 2^16 and 0.05 for the column;
+// now 0.27 ms, 2.0 TB/s, waiting for loads; 0.33 with 3 blocks an SM, 0.32 with 5).
+constexpr uint32_t kBandRows = 32, kBandCells = kBandRows / 4u, kBandThreads = 256, kBandBlocks = 4, kSegs = 8;
+// One copy for lanes l and l + 16: 8-byte loads go by half warps.
+constexpr size_t kRunTab2Bytes = 256u * 16u * sizeof(uint2);
 
 // Table entry of run byte b (kpz_w2.cuh): {8 D << 16 | V, A1}.
 __device__ __forceinline__ uint2 run_entry2(uint32_t b) {
@@ -267,9 +269,9 @@ __device__ __forceinline__ uint2 run_entry2(uint32_t b) {
   return make_uint2((uint32_t)(8 * D * 65536 + 8 * A2 - A1 * A1), (uint32_t)A1);
 }
 
-__global__ void __launch_bounds__(kBandThreads, 3) roughness_kernel(const uint32_t* __restrict__ lat, Geometry g,
+__global__ void __launch_bounds__(kBandThreads, kBandBlocks) roughness_kernel(const uint32_t* __restrict__ lat, Geometry g,
                                                                     long long* __restrict__ part, RoughOut out) {
-  extern __shared__ __align__(16) uint2 tab2[];   // [256][32]
+  extern __shared__ __align__(16) uint2 tab2[];   // [256][16]
   __shared__ long long seg_s1[kBandRows][kSegs], seg_s2[kBandRows][kSegs];
   __shared__ int seg_dh[kBandRows][kSegs];
   __shared__ bool last;
@@ -277,13 +279,15 @@ __global__ void __launch_bounds__(kBandThreads, 3) roughness_kernel(const uint32
   {
     const uint2 e = run_entry2(threadIdx.x);   // kBandThreads = 256 entries; a warp writes its 32 side by side
 #pragma unroll 8
-    for (uint32_t i = 0; i < 32u; ++i)
-      tab2[(warp * 32u + i) * 32u + lane] =
-          make_uint2(__shfl_sync(0xffffffffu, e.x, i), __shfl_sync(0xffffffffu, e.y, i));
+    for (uint32_t i = 0; i < 16u; ++i) {
+      const uint32_t k = 2u * i + (lane >> 4);
+      const uint2 v = make_uint2(__shfl_sync(0xffffffffu, e.x, k), __shfl_sync(0xffffffffu, e.y, k));
+      tab2[(warp * 32u + k) * 16u + (lane & 15u)] = v;
+    }
   }
   __syncthreads();
   const char* tl = reinterpret_cast<const char*>(tab2);
-  const uint32_t lane8 = lane * 8u;
+  const uint32_t lane8 = (lane & 15u) * 8u;
   const uint32_t y4 = warp & 3u, rr = lane & 7u, q = (warp >> 2) * 4u + (lane >> 3);
   const uint32_t seg = (g.NB + kSegs - 1u) / kSegs, K0 = min(g.NB, q * seg), K1 = min(g.NB, K0 + seg);
   const uint32_t nb = g.L / kBandRows;
@@ -311,8 +315,8 @@ __global__ void __launch_bounds__(kBandThreads, 3) roughness_kernel(const uint32
         for (uint32_t m = 0; m < 4; ++m)
 #pragma unroll
           for (uint32_t k = 0; k < 4; ++k) {
-            const uint32_t v = m == 0u ? u[k] << 8 : u[k] >> (8u * m - 8u);
-            const uint2 e = *reinterpret_cast<const uint2*>(tl + ((v & 0xFF00u) | lane8));
+            const uint32_t v = m == 0u ? u[k] << 7 : u[k] >> (8u * m - 7u);
+            const uint2 e = *reinterpret_cast<const uint2*>(tl + ((v & 0x7F80u) | lane8));
             const int32_t mm = (run >> 16) + (int32_t)e.y;
             sm += mm;
             sq += mm * mm;

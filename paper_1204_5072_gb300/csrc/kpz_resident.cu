@@ -301,31 +301,12 @@ __device__ __forceinline__ uint32_t phase_set(const SweepParams& P, uint32_t s, 
   return phase == 0u ? perm[0] : phase == 1u ? perm[1] : phase == 2u ? perm[2] : perm[3];
 }
 
-__device__ __forceinline__ uint64_t now_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
-  uint32_t v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ uint32_t add_release(uint32_t* p, uint32_t v) {
-  uint32_t old;
-  asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
-  return old;
-}
-__device__ __forceinline__ void red_release(uint32_t* p) {
-  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
-}
 __device__ __forceinline__ void bar_sync(uint32_t id, uint32_t n) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 __device__ __forceinline__ void bar_arrive(uint32_t id, uint32_t n) {
   asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
-constexpr uint64_t kWaitNs = 10000000000ull;   // bound of every grid wait
 
 // Grid version. A step is a sweep, or one tile set of a sweep (kSets); every
 // tile of a step has a tile warp of its own. Warps of a block: wpc tile warps,
@@ -338,7 +319,7 @@ constexpr uint64_t kWaitNs = 10000000000ull;   // bound of every grid wait
 template <bool kGeneral, bool kSets>
 __global__ void __launch_bounds__(320, 1) resident_grid_kernel(const SweepParams P, uint32_t n, uint32_t tiles,
                                                                uint32_t wpc, uint32_t makers, uint32_t* scratch,
-                                                               ResidentSync* sync) {
+                                                               GridSync* sync) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TileRand<kGeneral>* rnd = reinterpret_cast<TileRand<kGeneral>*>(smem_raw);   // [1 or 2][wpc]
   TileMem* mem = reinterpret_cast<TileMem*>(rnd + (makers ? 2u : 1u) * wpc);   // [wpc]
@@ -353,18 +334,8 @@ __global__ void __launch_bounds__(320, 1) resident_grid_kernel(const SweepParams
     for (uint32_t k = 1; k <= nsteps; ++k) {
       bar_sync(1, blockDim.x);
       if (lane == 0) {
-        red_release(&sync->arrived);
-        const uint32_t want = k * gridDim.x;
-        if (ld_acquire(&sync->arrived) < want) {
-          const uint64_t t0 = now_ns();
-          for (uint32_t it = 1; ld_acquire(&sync->arrived) < want; ++it) {
-            if ((it & 63u) == 0u && (now_ns() - t0 > kWaitNs || *(volatile uint32_t*)&sync->err)) {
-              atomicExch(&sync->err, 1u);
-              stop = 1u;
-              break;
-            }
-          }
-        }
+        gridsync::red_release(&sync->arrived);
+        if (!gridsync::wait_for(sync, k * gridDim.x)) stop = 1u;
       }
       __syncwarp();
       bar_sync(2, blockDim.x);
@@ -374,7 +345,7 @@ __global__ void __launch_bounds__(320, 1) resident_grid_kernel(const SweepParams
     // The last block out resets the counters and advances the sweep count.
     if (lane == 0) {
       __threadfence();
-      if (add_release(&sync->finished, 1u) == gridDim.x - 1u) {
+      if (gridsync::add_acq_rel(&sync->finished, 1u) == gridDim.x - 1u) {
         sync->arrived = 0u;
         sync->finished = 0u;
         *const_cast<uint64_t*>(P.t_dev) += n;
@@ -696,7 +667,7 @@ uint32_t resident_kind(const SweepParams& P, bool tilesets) {
 }
 
 cudaError_t launch_resident(const SweepParams& P, bool tilesets, uint32_t kind, uint32_t n, uint32_t* scratch,
-                            ResidentSync* sync, cudaStream_t st) {
+                            GridSync* sync, cudaStream_t st) {
   const bool general = is_general(P);
   const Shape h = shape_of(P, tilesets, general, kind == 2u);
   if (h.wpc == 0u) return cudaErrorInvalidValue;
