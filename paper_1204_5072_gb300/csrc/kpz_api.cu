@@ -6,8 +6,10 @@
 #include <cstring>
 #include <algorithm>
 #include <atomic>
+#include <mutex>
 #include <new>
 #include <string>
+#include <vector>
 
 #include "kpz.h"
 #include "kpz_host.h"
@@ -21,6 +23,55 @@ using namespace kpz;
 namespace kpz {
 static std::atomic<uint64_t> g_launches{0};
 void count_launch(uint64_t n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
+
+// Pinned slots of all contexts and networks of the process: one allocation (20
+// us) for up to 64 of them instead of one each.
+namespace {
+struct Slab {
+  char* base;
+  uint64_t used;   // bit i: slot i
+};
+std::mutex g_slab_mu;
+std::vector<Slab> g_slabs;
+}  // namespace
+
+void* host_slot() {
+  std::lock_guard<std::mutex> lock(g_slab_mu);
+  Slab* s = nullptr;
+  for (Slab& x : g_slabs)
+    if (~x.used) { s = &x; break; }
+  if (!s) {
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, 64 * kHostSlot, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    try {
+      g_slabs.push_back(Slab{(char*)p, 0u});
+    } catch (...) {
+      cudaFreeHost(p);
+      return nullptr;
+    }
+    s = &g_slabs.back();
+  }
+  const int i = __builtin_ctzll(~s->used);
+  s->used |= 1ull << i;
+  memset(s->base + i * kHostSlot, 0, kHostSlot);
+  return s->base + i * kHostSlot;
+}
+
+void host_slot_free(void* p) {
+  if (!p) return;
+  std::lock_guard<std::mutex> lock(g_slab_mu);
+  bool any = false;
+  for (Slab& x : g_slabs) {
+    if ((char*)p >= x.base && (char*)p < x.base + 64 * kHostSlot) x.used &= ~(1ull << (((char*)p - x.base) / kHostSlot));
+    any = any || x.used;
+  }
+  if (any) return;
+  for (Slab& x : g_slabs) cudaFreeHost(x.base);
+  g_slabs.clear();
+}
 }  // namespace kpz
 
 struct kpz_ctx {
@@ -43,7 +94,7 @@ struct kpz_ctx {
   uint64_t* t_dev = nullptr;           // sweep counter
   unsigned long long* h00 = nullptr;   // absolute height of site (0,0)
   uint32_t* ticket = nullptr;          // roughness: blocks that have finished (zero between launches)
-  long long* sums = nullptr;           // pinned host memory: results of the roughness kernel
+  long long* sums = nullptr;           // pinned host slot: results of the roughness kernel
   uint32_t* hcar = nullptr;            // import: height of (0, j0) modulo 4
   uint32_t* queue = nullptr;           // sweep work queue (zero between launches)
   GridSync* sync = nullptr;            // persistent kernels: grid barrier and error flag
@@ -284,9 +335,8 @@ kpz_status kpz_init(kpz_ctx** out, uint32_t L, double p, double q, uint64_t seed
     ctx->own_buf = true;
     ctx->buf_bytes = y.total;
   }
-  if (cudaHostAlloc((void**)&ctx->sums, 8 * sizeof(long long), cudaHostAllocMapped | cudaHostAllocPortable) !=
-      cudaSuccess) {
-    cudaGetLastError();
+  ctx->sums = (long long*)host_slot();
+  if (!ctx->sums) {
     if (ctx->own_buf) cudaFree(ctx->buf);
     delete ctx;
     return KPZ_ENOMEM;
@@ -295,7 +345,7 @@ kpz_status kpz_init(kpz_ctx** out, uint32_t L, double p, double q, uint64_t seed
     cudaError_t e = cudaMalloc(&ctx->rsu_scratch, rsu_scratch_bytes(L));
     if (e != cudaSuccess) {
       cudaGetLastError();
-      cudaFreeHost(ctx->sums);
+      host_slot_free(ctx->sums);
       if (ctx->own_buf) cudaFree(ctx->buf);
       delete ctx;
       return KPZ_ENOMEM;
@@ -657,7 +707,7 @@ void kpz_free(kpz_ctx* ctx) {
   }
   if (ctx->sums) {
     cudaStreamSynchronize(ctx->stream);
-    cudaFreeHost(ctx->sums);
+    host_slot_free(ctx->sums);
   }
   delete ctx;
 }

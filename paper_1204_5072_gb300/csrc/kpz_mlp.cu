@@ -502,7 +502,7 @@ struct kpz_mlp {
   float *x = nullptr, *t = nullptr, *y = nullptr, *gpart = nullptr, *grad = nullptr;
   size_t cap = 0, pcap = 0;
   struct Host { int err; float sq; };
-  Host* host = nullptr;         // pinned: set when a tensor-core wait timed out; sum of squared errors
+  Host* host = nullptr;         // pinned slot: set when a tensor-core wait timed out; sum of squared errors
 };
 
 namespace {
@@ -511,7 +511,7 @@ void mlp_release(kpz_mlp* m) {
   float* ptrs[] = {m->theta, m->m, m->v, m->grad, m->x, m->t, m->y, m->gpart};
   for (float* p : ptrs) if (p) cudaFree(p);
   if (m->P) cudaFree(m->P);
-  if (m->host) cudaFreeHost(m->host);
+  host_slot_free(m->host);
 }
 
 // Synchronises the stream; KPZ_ETIMEOUT when a kernel's tensor-core wait ran
@@ -592,15 +592,12 @@ kpz_status kpz_mlp_create(kpz_mlp** out, const float* params, void* stream) {
   m->stream = (cudaStream_t)stream;
   if (cudaMalloc(&m->theta, kParams * 4) != cudaSuccess || cudaMalloc(&m->m, kParams * 4) != cudaSuccess ||
       cudaMalloc(&m->v, kParams * 4) != cudaSuccess || cudaMalloc(&m->grad, kParams * 4) != cudaSuccess ||
-      cudaMalloc(&m->P, kParams * 2) != cudaSuccess ||
-      cudaHostAlloc((void**)&m->host, sizeof(*m->host), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+      cudaMalloc(&m->P, kParams * 2) != cudaSuccess || !(m->host = (kpz_mlp::Host*)host_slot())) {
     cudaGetLastError();
     mlp_release(m);
     delete m;
     return KPZ_ENOMEM;
   }
-  m->host->err = 0;
-  m->host->sq = 0.f;
   if (cudaFuncSetAttribute(net_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kSmemGrad) !=
           cudaSuccess ||
       cudaFuncSetAttribute(net_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kSmemPredict) !=

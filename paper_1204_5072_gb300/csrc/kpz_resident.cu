@@ -21,13 +21,14 @@
 //     Two scratch lattices take turns; the last step writes the fixed frame.
 // Microseconds per sweep, p = 1 / p = 0.95, against one launch per sweep with
 // runs of 8 tiles (and of one tile, the fastest there): L = 256 2.1 / 3.3
-// against 12.4 / 22.8 (10.2 / 15.9), L = 1024 2.7 / 4.6 against 25 / 63 (10.2 /
-// 17.7), L = 4096 3.8 / 7.9 against 29 / 80 (14.1 / 25.8); tile sets at
-// L = 2048 13.8 / 19.3 against 44 at p = 1. At L = 512 (one tile a block, one
-// tile warp a scheduler) the 16 rounds take 2000 / 4300 cycles of a sweep's
-// 4400 / 7000; the rest is the window's trip and the barrier. At L = 4096 and
-// general rates the eight tiles of an SM bind it (logic and Philox pipes).
+// against 12.4 / 22.8 (10.2 / 15.9), L = 1024 2.9 / 4.3 against 25 / 63 (10.2 /
+// 17.7), L = 4096 4.0 / 8.0 against 29 / 80 (14.1 / 25.8); tile sets at L = 2048
+// 12.2 / 19.1 against 44 at p = 1. At L = 512 (one tile a block, one tile warp
+// a scheduler) the 16 rounds take 2000 / 4300 cycles of a sweep's 4400 / 7000;
+// the rest is the window's trip and the barrier. At L = 4096 and general rates
+// the eight tiles of an SM bind it (logic and Philox pipes).
 #include <algorithm>
+#include <mutex>
 
 #include "kpz_resident.h"
 #include "kpz_tilemem.cuh"
@@ -438,11 +439,11 @@ __global__ void __launch_bounds__(320, 1) resident_grid_kernel(const SweepParams
   }
 }
 
-// Cluster version (L <= 1024): one cluster of 1 to 16 blocks holds the whole
-// lattice in its shared memory, two frames of it by turns, a block the words
-// of its `tpc` tiles; windows are read over distributed shared memory and the
-// hardware's cluster barrier ends a sweep. Warps of a block: tpc tile warps,
-// makers * tpc drawing warps.
+// Cluster version (up to 64 tiles at a time): one cluster of 1 to 16 blocks
+// holds the whole lattice in its shared memory, two frames of it by turns;
+// windows are read over distributed shared memory and the hardware's cluster
+// barrier ends a step. Warps of a block: a tile warp for each of its units,
+// `makers` drawing warps for each.
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ uint32_t map_to(uint32_t addr, uint32_t cta) {
   uint32_t r;
@@ -458,44 +459,61 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// load_window over the cluster: `lat` = shared address of the frame in every
-// block ([tpc][16 planes][32 lanes] words), tpc = 1 << lg tiles per block.
-template <int kHalo>
-__device__ __forceinline__ void load_window_cluster(const SweepParams& P, uint32_t lat, uint32_t lg, uint32_t lane,
-                                                    uint32_t X0, uint32_t Y0, Window& w) {
-  const uint32_t NR = P.g.NR, NB = P.g.NB;
-  const uint32_t by = Y0 & 3u, Rb = Y0 >> 2, bx = X0 & 3u, a = X0 >> 2, K = a >> 5;
-  // Address of plane 0 of block columns K, K + 1, K + 2 at cell rows Rb + lane,
-  // Rb + lane + 1 and Rb + 32.
-  uint32_t at[3][3];
-#pragma unroll
-  for (uint32_t i = 0; i < (kHalo ? 3u : 2u); ++i) {
-    const uint32_t R = (Rb + (i == 2u ? 32u : lane + i)) & (NR - 1u);
-#pragma unroll
-    for (uint32_t j = 0; j < 3u; ++j) {
-      const uint32_t t = (R >> 5) * P.ntx + ((K + j) & (NB - 1u));
-      at[i][j] = map_to(lat + (t & ((1u << lg) - 1u)) * (kPlanes * 128u) + (R & 31u) * 4u, t >> lg);
-    }
+// The lattice over the cluster: a block's frame holds 1 << lg units of one
+// tile, or (kSets) of 2 x 2 tiles, one of each set, each tile as [16 planes][32
+// cell rows] words.
+template <bool kSets>
+struct ClusterLat {
+  uint32_t frame;   // shared address of the frame in every block
+  uint32_t lg, NR, NB, ntx;
+  // Address of plane 0 of block column K at cell row R (both wrapped).
+  __device__ __forceinline__ uint32_t at(uint32_t K, uint32_t R) const {
+    K &= NB - 1u;
+    R &= NR - 1u;
+    const uint32_t ty = R >> 5;
+    const uint32_t unit = kSets ? (ty >> 1) * (ntx >> 1) + (K >> 1) : ty * ntx + K;
+    const uint32_t q = kSets ? (K & 1u) + 2u * (ty & 1u) : 0u;
+    const uint32_t slot = (unit & ((1u << lg) - 1u)) * (kSets ? 4u : 1u) + q;
+    return map_to(frame + slot * (kPlanes * 128u) + (R & 31u) * 4u, unit >> lg);
   }
-  uint32_t C[4][4], N[4][4], H[4][2], sh[4];
+};
+
+// load_window over the cluster.
+template <int kHalo, bool kSets>
+__device__ __forceinline__ void load_window_cluster(const ClusterLat<kSets>& lat, uint32_t lane, uint32_t X0, uint32_t Y0,
+                                                    Window& w) {
+  const uint32_t L = lat.NR * 4u;
+  X0 &= L - 1u;
+  Y0 &= L - 1u;
+  const uint32_t by = Y0 & 3u, Rb = Y0 >> 2, bx = X0 & 3u, a = X0 >> 2, K = a >> 5;
+  // Plane 0 of block columns K, K + 1, K + 2 at cell rows Rb + lane, Rb + lane
+  // + 1, of the row below the tile (lane 31 needs it) and the one above (lane 0).
+  uint32_t at[4][3];
+#pragma unroll
+  for (uint32_t i = 0; i < (kHalo == 2 ? 4u : kHalo ? 3u : 2u); ++i) {
+    const uint32_t R = i == 3u ? Rb - 1u + ((by + 3u) >> 2) : Rb + (i == 2u ? 32u : lane + i);
+#pragma unroll
+    for (uint32_t j = 0; j < 3u; ++j) at[i][j] = lat.at(K + j, R);
+  }
+  uint32_t C[4][4], N[4][4], H[4][2], U[4][2], B3[4], sh[4];
 #pragma unroll
   for (uint32_t xq = 0; xq < 4; ++xq) {
     const uint32_t st = a + ((bx + xq) >> 2), x4 = (bx + xq) & 3u;
     sh[xq] = st & 31u;
     const bool next = (st >> 5) != K;   // carried into the next block column
+    auto two = [&](uint32_t r0, uint32_t r1, uint32_t r2, uint32_t p, uint32_t& c, uint32_t& n) {
+      c = ld_cluster((next ? r1 : r0) + p);
+      n = ld_cluster((next ? r2 : r1) + p);
+    };
 #pragma unroll
     for (uint32_t yq = 0; yq < 4; ++yq) {
       const uint32_t y4 = (by + yq) & 3u, p = plane(y4, x4) * 128u;
       const bool wrap = by + yq >= 4u;
-      const uint32_t a0 = wrap ? at[1][0] : at[0][0], a1 = wrap ? at[1][1] : at[0][1], a2 = wrap ? at[1][2] : at[0][2];
-      C[yq][xq] = ld_cluster((next ? a1 : a0) + p);
-      N[yq][xq] = ld_cluster((next ? a2 : a1) + p);
+      two(wrap ? at[1][0] : at[0][0], wrap ? at[1][1] : at[0][1], wrap ? at[1][2] : at[0][2], p, C[yq][xq], N[yq][xq]);
+      if (kHalo == 2 && xq == 3) B3[yq] = ld_cluster(lat.at((st >> 5) - 1u, Rb + lane + (wrap ? 1u : 0u)) + p);
     }
-    if (kHalo) {
-      const uint32_t p = plane(by, x4) * 128u;
-      H[xq][0] = ld_cluster((next ? at[2][1] : at[2][0]) + p);
-      H[xq][1] = ld_cluster((next ? at[2][2] : at[2][1]) + p);
-    }
+    if (kHalo) two(at[2][0], at[2][1], at[2][2], plane(by, x4) * 128u, H[xq][0], H[xq][1]);
+    if (kHalo == 2) two(at[3][0], at[3][1], at[3][2], plane((by + 3u) & 3u, x4) * 128u, U[xq][0], U[xq][1]);
   }
 #pragma unroll
   for (uint32_t xq = 0; xq < 4; ++xq) {
@@ -503,62 +521,124 @@ __device__ __forceinline__ void load_window_cluster(const SweepParams& P, uint32
     for (uint32_t yq = 0; yq < 4; ++yq) {
       w.T[yq][xq] = __funnelshift_r(C[yq][xq], N[yq][xq], sh[xq]);
       if (kHalo && xq == 0) w.hx[yq] = (N[yq][0] >> sh[0]) & 1u;
+      if (kHalo == 2 && xq == 3) w.left[yq] = ((sh[3] ? C[yq][3] : B3[yq]) >> ((sh[3] + 31u) & 31u)) & 1u;
     }
     if (kHalo) w.hy[xq] = __funnelshift_r(H[xq][0], H[xq][1], sh[xq]);
+    if (kHalo == 2) w.up[xq] = __funnelshift_r(U[xq][0], U[xq][1], sh[xq]);
   }
 }
 
-template <bool kGeneral>
+// load_tile over the cluster; own: this lane's words of the tile, 32 apart.
+__device__ __forceinline__ void load_tile_cluster(const ClusterLat<true>& lat, const uint32_t* own, uint32_t lane,
+                                                  uint32_t tx, uint32_t ty, Window& w) {
+  const uint32_t R = ty * 32u + lane;
+  const uint32_t l = lat.at(tx - 1u, R), r = lat.at(tx + 1u, R), u = lat.at(tx, ty * 32u - 1u), d = lat.at(tx, ty * 32u + 32u);
+#pragma unroll
+  for (uint32_t y = 0; y < 4; ++y) {
+    w.left[y] = ld_cluster(l + plane(y, 3) * 128u) >> 31;
+    w.hx[y] = ld_cluster(r + plane(y, 0) * 128u) & 1u;
+  }
+#pragma unroll
+  for (uint32_t x = 0; x < 4; ++x) {
+    w.hy[x] = ld_cluster(d + plane(0, x) * 128u);
+    w.up[x] = ld_cluster(u + plane(3, x) * 128u);
+  }
+#pragma unroll
+  for (uint32_t p = 0; p < kPlanes; ++p) w.T[p >> 2][p & 3u] = own[p * 32u];
+}
+
+template <bool kGeneral, bool kSets>
 __global__ void __launch_bounds__(384, 1) resident_cluster_kernel(const SweepParams P, uint32_t n, uint32_t lg,
                                                                   uint32_t makers) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const uint32_t tpc = 1u << lg;
-  TileRand<kGeneral>* rnd = reinterpret_cast<TileRand<kGeneral>*>(smem_raw);   // [2][tpc]
-  TileMem* mem = reinterpret_cast<TileMem*>(rnd + 2u * tpc);                   // [tpc]
-  uint32_t* frame = reinterpret_cast<uint32_t*>(mem + tpc);                    // [2][tpc][16][32]
+  constexpr uint32_t kTiles = kSets ? 4u : 1u, kTileWords = kPlanes * 32u;   // tiles of a unit
+  const uint32_t units = 1u << lg;
+  TileRand<kGeneral>* rnd = reinterpret_cast<TileRand<kGeneral>*>(smem_raw);   // [2][units]
+  TileMem* mem = reinterpret_cast<TileMem*>(rnd + 2u * units);                 // [units]
+  uint32_t* frame = reinterpret_cast<uint32_t*>(mem + units);                  // [2][units][tiles][16][32]
   __shared__ QuadTab tab;
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   const uint32_t t0 = (uint32_t)(*(const volatile uint64_t*)P.t_dev) + P.s_add;
-  const uint32_t L = P.g.L;
   if (threadIdx.x < 4u) tilemem::fill_quad_tab(tab, threadIdx.x);
-  const bool maker = warp >= tpc;
-  const uint32_t slot = maker ? (warp - tpc) & (tpc - 1u) : warp, part = maker ? (warp - tpc) >> lg : 0u;
-  const uint32_t tile = blockIdx.x * tpc + slot, ty = tile / P.ntx, tx = tile - ty * P.ntx;
+  const bool maker = warp >= units;
+  const uint32_t slot = maker ? (warp - units) & (units - 1u) : warp, part = maker ? (warp - units) >> lg : 0u;
+  const uint32_t unit = blockIdx.x * units + slot, across = P.ntx / (kSets ? 2u : 1u);
+  const uint32_t uy = unit / across, ux = unit - uy * across;
   __syncthreads();
-  uint32_t* own = frame + slot * (kPlanes * 32u) + lane;   // this lane's words, 32 apart; + the frame's offset
-  const uint32_t half = tpc * kPlanes * 32u;               // words of one frame in this block
+  uint32_t* own = frame + slot * kTiles * kTileWords + lane;   // this lane's words, 32 apart; + the frame's and the tile's offset
+  const uint32_t half = units * kTiles * kTileWords;           // words of one frame in this block
+  const uint32_t nsteps = n * kTiles;
+  // Sweep, set and tile of step k.
+  auto place = [&](uint32_t k, uint32_t& s, uint32_t& q, uint32_t& tx, uint32_t& ty) {
+    s = t0 + k / kTiles;
+    q = kSets ? phase_set(P, s, k & 3u) : 0u;
+    tx = kSets ? 2u * ux + (q & 1u) : ux;
+    ty = kSets ? 2u * uy + (q >> 1) : uy;
+  };
   Window w;
+  uint32_t s, q, tx, ty;
   if (maker) {
-    draw_tile<kGeneral>(P, tab, rnd[slot], tile, t0, lane, part, makers);
+    place(0u, s, q, tx, ty);
+    draw_tile<kGeneral>(P, tab, rnd[slot], ty * P.ntx + tx, s, lane, part, makers);
   } else {
-    const uint32_t o = tx * kPlanes * P.g.NR + ty * 32u + lane;
+#pragma unroll 1
+    for (uint32_t i = 0; i < kTiles; ++i) {
+      const uint32_t x = kSets ? 2u * ux + (i & 1u) : ux, y = kSets ? 2u * uy + (i >> 1) : uy;
+      const uint32_t o = x * kPlanes * P.g.NR + y * 32u + lane;
 #pragma unroll
-    for (uint32_t p = 0; p < kPlanes; ++p) own[p * 32u] = __ldcg(P.lat + o + p * P.g.NR);
+      for (uint32_t p = 0; p < kPlanes; ++p) own[i * kTileWords + p * 32u] = __ldcg(P.lat + o + p * P.g.NR);
+    }
   }
-  uint32_t px = 0u, py = 0u;
-  cluster_sync();
-  for (uint32_t k = 0; k < n; ++k) {
-    const uint32_t s = t0 + k, buf = k & 1u;
-    if (maker) {
-      if (k + 1u < n) draw_tile<kGeneral>(P, tab, rnd[(buf ^ 1u) * tpc + slot], tile, s + 1u, lane, part, makers);
-    } else {
-      const TileRand<kGeneral>& B = rnd[buf * tpc + slot];
-      const uint32_t ox = B.origin[0], oy = B.origin[1];
-      load_window_cluster<1>(P, smem_u32(frame + buf * half), lg, lane, (ox - px + tx * kTile) & (L - 1u),
-                             (oy - py + ty * kTile) & (L - 1u), w);
-      tile_rounds<kGeneral, false>(P, w, mem[slot], tab, B, lane, s, ox, oy, tx, ty);
-      uint32_t* to = own + (buf ^ 1u) * half;
+  uint32_t px = 0u, py = 0u, ox = 0u, oy = 0u;
+  auto lattice = [&](uint32_t sweep) {   // as it stands after `sweep` sweeps of this launch
+    return ClusterLat<kSets>{smem_u32(frame + (sweep & 1u) * half), lg, P.g.NR, P.g.NB, P.ntx};
+  };
+  auto put = [&](uint32_t* to) {
 #pragma unroll
-      for (uint32_t p = 0; p < kPlanes; ++p) to[p * 32u] = w.T[p >> 2][p & 3u];
-      px = ox;
-      py = oy;
+    for (uint32_t p = 0; p < kPlanes; ++p) to[p * 32u] = w.T[p >> 2][p & 3u];
+  };
+  cluster_sync();
+  for (uint32_t k = 0; k < nsteps; ++k) {
+    const uint32_t buf = k & 1u, sw = k / kTiles;
+    if (maker) {
+      if (k + 1u < nsteps) {
+        place(k + 1u, s, q, tx, ty);
+        draw_tile<kGeneral>(P, tab, rnd[(buf ^ 1u) * units + slot], ty * P.ntx + tx, s, lane, part, makers);
+      }
+    } else {
+      const TileRand<kGeneral>& B = rnd[buf * units + slot];
+      place(k, s, q, tx, ty);
+      uint32_t* to = own + ((sw + 1u) & 1u) * half;
+      if (!kSets || (k & 3u) == 0u) {   // the sweep's first step: the frame changes
+        px = ox;
+        py = oy;
+        ox = B.origin[0];
+        oy = B.origin[1];
+        if (kSets) {
+#pragma unroll 1
+          for (uint32_t i = 0; i < 4u; ++i) {
+            if (i == q) continue;
+            load_window_cluster<0>(lattice(sw), lane, ox - px + (2u * ux + (i & 1u)) * kTile,
+                                   oy - py + (2u * uy + (i >> 1)) * kTile, w);
+            put(to + i * kTileWords);
+          }
+        }
+        load_window_cluster<kSets ? 2 : 1>(lattice(sw), lane, ox - px + tx * kTile, oy - py + ty * kTile, w);
+      } else if constexpr (kSets) {
+        load_tile_cluster(lattice(sw + 1u), to + q * kTileWords, lane, tx, ty, w);
+      }
+      tile_rounds<kGeneral, kSets>(P, w, mem[slot], tab, B, lane, s, ox, oy, tx, ty);
+      put(to + q * kTileWords);
     }
     cluster_sync();
   }
   if (!maker) {
-    load_window_cluster<0>(P, smem_u32(frame + (n & 1u) * half), lg, lane, (tx * kTile - px) & (L - 1u),
-                           (ty * kTile - py) & (L - 1u), w);
-    store_tile(P.g, GlobalLat{P.lat}, lane, tx, ty, w.T);
+#pragma unroll 1
+    for (uint32_t i = 0; i < kTiles; ++i) {
+      const uint32_t x = kSets ? 2u * ux + (i & 1u) : ux, y = kSets ? 2u * uy + (i >> 1) : uy;
+      load_window_cluster<0>(lattice(n), lane, x * kTile - ox, y * kTile - oy, w);
+      store_tile(P.g, GlobalLat{P.lat}, lane, x, y, w.T);
+    }
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) *const_cast<uint64_t*>(P.t_dev) += n;
   cluster_sync();   // no block leaves while its shared memory is read
@@ -576,22 +656,24 @@ struct Shape {
 // 120 cycles, an SM's quarter in 80 (the wide multiplies), so drawing warps
 // pay while an SM has at most two tiles; with eight they take the issue slots
 // the tile warps need (L = 4096 at p = 0.95: 9.0 us a sweep with them, 7.9
-// without). The cluster serves up to 64 tiles, four a block: there it takes
-// 2.7 / 4.6 us a sweep against 3.3 / 5.4 on a grid of 64 blocks, at 16 tiles
-// 2.1 / 3.4 against 3.2 / 5.4. Beyond 1024 tiles an SM would have more than
-// two tiles a scheduler, and work, not latency, is the bound.
+// without). The cluster has 16 SMs: at p = 1 it serves four tiles each (L =
+// 1024 2.9 us a sweep, 3.1 on a grid; tile sets at L = 2048 12.2, 13.8), at
+// general rates one (L = 512 3.4, L = 1024 4.7 against 4.3 on a grid; tile sets
+// at L = 1024 14.4 against 19.0, at L = 2048 21.0 against 19.1). Beyond 1024
+// tiles an SM would have more than two tiles a scheduler, and work, not
+// latency, is the bound.
 Shape shape_of(const SweepParams& P, bool tilesets, bool general, bool cluster) {
   Shape h{};
   const size_t rnd = general ? sizeof(TileRand<true>) : sizeof(TileRand<false>);
   const uint32_t all = P.ntx * P.nty;
   if (cluster) {
-    if (tilesets || all > 64u) return h;
+    h.tiles = tilesets ? all / 4u : all;
+    if (h.tiles > (general ? 16u : 64u)) return Shape{};
     h.cluster = true;
-    h.tiles = all;
-    h.grid = std::min(all, 16u);
-    h.wpc = all / h.grid;
+    h.grid = std::min(h.tiles, 16u);
+    h.wpc = h.tiles / h.grid;
     h.makers = general ? 2u : 1u;
-    h.smem = h.wpc * (2u * rnd + sizeof(TileMem) + 2u * kPlanes * 32u * sizeof(uint32_t));
+    h.smem = h.wpc * (2u * rnd + sizeof(TileMem) + (tilesets ? 8u : 2u) * kPlanes * 32u * sizeof(uint32_t));
     return h;
   }
   h.tiles = tilesets ? all / 4u : all;
@@ -604,8 +686,11 @@ Shape shape_of(const SweepParams& P, bool tilesets, bool general, bool cluster) 
 }
 
 const void* kernel_of(const Shape& h, bool tilesets, bool general) {
+  if (h.cluster && tilesets)
+    return general ? (const void*)resident_cluster_kernel<true, true> : (const void*)resident_cluster_kernel<false, true>;
   if (h.cluster)
-    return general ? (const void*)resident_cluster_kernel<true> : (const void*)resident_cluster_kernel<false>;
+    return general ? (const void*)resident_cluster_kernel<true, false>
+                   : (const void*)resident_cluster_kernel<false, false>;
   if (tilesets)
     return general ? (const void*)resident_grid_kernel<true, true> : (const void*)resident_grid_kernel<false, true>;
   return general ? (const void*)resident_grid_kernel<true, false> : (const void*)resident_grid_kernel<false, false>;
@@ -662,8 +747,21 @@ bool is_general(const SweepParams& P) { return !(P.Tp == 65536u && P.Tq == 0u); 
 uint32_t resident_kind(const SweepParams& P, bool tilesets) {
   if (P.cell == 2u || P.nty * kTile != P.g.L) return 0u;
   const bool general = is_general(P);
-  if (fits(shape_of(P, tilesets, general, true), tilesets, general)) return 2u;
-  return fits(shape_of(P, tilesets, general, false), tilesets, general) ? 1u : 0u;
+  // The answer for a device, size and kernel is kept (the queries take 10 us).
+  constexpr int kMaxDev = 64;
+  static std::mutex mu;
+  static uint8_t known[kMaxDev][32][2][2] = {};   // kind + 1
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0u;
+  std::lock_guard<std::mutex> lock(mu);
+  uint8_t other = 0u;
+  uint8_t& k = dev < kMaxDev ? known[dev][__builtin_ctz(P.g.L)][tilesets][general] : other;
+  if (k) return k - 1u;
+  const uint32_t kind = fits(shape_of(P, tilesets, general, true), tilesets, general)    ? 2u
+                        : fits(shape_of(P, tilesets, general, false), tilesets, general) ? 1u
+                                                                                          : 0u;
+  k = (uint8_t)(kind + 1u);
+  return kind;
 }
 
 cudaError_t launch_resident(const SweepParams& P, bool tilesets, uint32_t kind, uint32_t n, uint32_t* scratch,

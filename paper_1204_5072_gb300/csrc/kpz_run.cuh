@@ -24,16 +24,18 @@
 // shuffles). The right neighbour of the last cell column and the row below
 // the last lane belong to the next tiles' dead borders, which no one changes
 // during the sweep: they are read once as halos. The next block column is
-// copied into shared memory (cp.async) one tile ahead.
+// copied into shared memory (cp.async) one tile ahead. At general rates a
+// 128 x 128 tile of 4 x 4 cells goes to shared memory for its rounds
+// (kpz_tilemem.cuh) and comes back to registers for the write-back.
 //
 // A run is tiles tx0 .. tx0 + n - 1 of one tile row, swept left to right with a
 // sliding two-word window per plane. The words a run shares with the runs to
 // its left and right are written back as XOR deltas against the tile's start
 // copy, so a run never reads memory another run may be changing. With kSK the
-// Philox round keys come from shared memory (rk) and each lane draws the
-// quadrant sets of a different tile. With kRtPar the tile parity is a run-time
-// value, so one copy of the round code serves every tile (callers whose
-// warps work on tiles of both parities at once).
+// Philox round keys come from shared memory (rk). With kRtPar the tile parity
+// of the register rounds is a run-time value, so one copy of the round code
+// serves every tile (callers whose warps work on tiles of both parities at
+// once).
 #pragma once
 #include "kpz_rounds.cuh"
 #include "kpz_tilemem.cuh"

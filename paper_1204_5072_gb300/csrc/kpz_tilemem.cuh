@@ -268,16 +268,17 @@ __device__ __forceinline__ uint32_t accept_cells(const SweepParams& P, const Rat
   for (int n = 0; n < 4; ++n) tie &= ~(w[n] ^ b[n]);
   uint32_t acc = lt & dm;
   if (kEdge) acc |= any & ((same & R.all_a) | (~same & R.all_b));
-  // The k-th tie from below takes the k-th outcome.
+  // The k-th tie from below takes the k-th outcome; a row has a fourth one in
+  // seven rounds of a thousand, so three are taken without a branch.
   const uint32_t g0 = (same & byte_mask<0>(Wa)) | (~same & byte_mask<0>(Wb));
   const uint32_t g1 = (same & byte_mask<1>(Wa)) | (~same & byte_mask<1>(Wb));
   const uint32_t g2 = (same & byte_mask<2>(Wa)) | (~same & byte_mask<2>(Wb));
-  const uint32_t g3 = (same & byte_mask<3>(Wa)) | (~same & byte_mask<3>(Wb));
-  const uint32_t m1 = tie & add_fma(tie, one, neg), m2 = m1 & add_fma(m1, one, neg), m3 = m2 & add_fma(m2, one, neg),
-                 m4 = m3 & add_fma(m3, one, neg);
+  const uint32_t m1 = tie & add_fma(tie, one, neg), m2 = m1 & add_fma(m1, one, neg), m3 = m2 & add_fma(m2, one, neg);
   acc |= (tie & ~m1 & g0) | (m1 & ~m2 & g1);
-  acc |= (m2 & ~m3 & g2) | (m3 & ~m4 & g3);
-  if (m4 != 0u) {   // more than four ties in a row: the overflow blocks of the round
+  acc |= m2 & ~m3 & g2;
+  if (m3 != 0u) {   // the fourth, and from the fifth on the overflow blocks of the round
+    const uint32_t m4 = m3 & (m3 - 1u);
+    acc |= m3 & ~m4 & ((same & byte_mask<3>(Wa)) | (~same & byte_mask<3>(Wb)));
     uint4 X = make_uint4(0u, 0u, 0u, 0u);
     uint32_t m = m4;
     for (uint32_t k = 0u; m != 0u; ++k) {
