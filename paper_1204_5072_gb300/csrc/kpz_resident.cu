@@ -720,10 +720,15 @@ cudaLaunchConfig_t config_of(const Shape& h, cudaLaunchAttribute* attr, cudaStre
 // Whether the current device holds all blocks of the kernel at once.
 bool fits(const Shape& h, bool tilesets, bool general) {
   if (h.wpc == 0u) return false;
-  int dev = 0, per_sm = 0, sms = 0, coop = 0;
+  int dev = 0, per_sm = 0, sms = 0, coop = 0, most = 0;
   const void* f = kernel_of(h, tilesets, general);
-  bool ok = cudaGetDevice(&dev) == cudaSuccess &&
-            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h.smem) == cudaSuccess;
+  cudaFuncAttributes fa{};
+  // The kernel's limit is the device's, not this shape's: it stays for every
+  // later launch, and lattices of other sizes share the kernel.
+  bool ok = cudaGetDevice(&dev) == cudaSuccess && cudaFuncGetAttributes(&fa, f) == cudaSuccess &&
+            cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
+            (most -= (int)fa.sharedSizeBytes) >= (int)h.smem &&
+            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess;
   if (ok && h.cluster) {
     if (h.grid > 8u) ok = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
     cudaLaunchAttribute attr;

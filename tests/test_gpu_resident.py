@@ -47,3 +47,15 @@ def test_against_launch_per_sweep(eng, L, p, q, decomposition):
         assert np.array_equal(lat.slopes(), ref.slopes())
     lat.close()
     ref.close()
+
+
+@pytest.mark.parametrize("decomposition", [0, 1])
+def test_lattices_of_several_sizes_share_a_kernel(eng, decomposition):
+    # A larger lattice still runs after smaller ones have been made, in any order.
+    for p, q in ((1.0, 0.0), (0.95, 0.05)):
+        lats = [eng.Lattice(L, p, q, seed=4, decomposition=decomposition) for L in (4096, 2048, 1024, 512, 256, 4096)]
+        for lat in lats:
+            lat.run(3)
+        assert lats[0].roughness() == lats[-1].roughness()
+        for lat in lats:
+            lat.close()
