@@ -20,11 +20,11 @@
 //     read-modify-write; red.xor took 45 cycles each, 1400 to 2400 a tile).
 //     Two scratch lattices take turns; the last step writes the fixed frame.
 // Microseconds per sweep, p = 1 / p = 0.95, against one launch per sweep with
-// runs of 8 tiles (and of one tile, the fastest there): L = 256 2.1 / 3.3
-// against 12.4 / 22.8 (10.2 / 15.9), L = 1024 2.9 / 4.3 against 25 / 63 (10.2 /
-// 17.7), L = 4096 4.0 / 8.0 against 29 / 80 (14.1 / 25.8); tile sets at L = 2048
-// 12.2 / 19.1 against 44 at p = 1. At L = 512 (one tile a block, one tile warp
-// a scheduler) the 16 rounds take 2000 / 4300 cycles of a sweep's 4400 / 7000;
+// runs of 8 tiles (and of one tile, the fastest there): L = 256 1.9 / 3.1
+// against 12.4 / 22.8 (10.2 / 15.9), L = 1024 2.7 / 4.3 against 25 / 63 (10.2 /
+// 17.7), L = 4096 3.9 / 7.9 against 29 / 80 (14.1 / 25.8); tile sets at L = 2048
+// 11.7 / 18.4 against 44 at p = 1. At L = 512 (one tile a block, one tile warp
+// a scheduler) the 16 rounds take 2000 / 4300 cycles of a sweep's 3900 / 6400;
 // the rest is the window's trip and the barrier. At L = 4096 and general rates
 // the eight tiles of an SM bind it (logic and Philox pipes).
 #include <algorithm>
@@ -45,7 +45,7 @@ using tilemem::TileMem;
 // 7 - r % 8 of byte k of deep[r / 8].x (.y) is set when the k-th tie of the row
 // in round r is accepted as a minimum (maximum) (streams as in
 // kpz_rounds.cuh), the rounds' quadrant offsets (tilemem::QuadTab) and the
-// sweep's origin.
+// next sweep's origin.
 template <bool kGeneral>
 struct TileRand {
   uint4 pos[kRounds / 2][32];
@@ -80,18 +80,24 @@ __device__ __forceinline__ void philox4(const uint32_t (&ctr)[4], uint32_t c1, u
   for (int i = 0; i < 4; ++i) out[i] = make_uint4(x[i], y[i], z[i], w[i]);
 }
 
+// Origin of the tile grid of sweep s.
+__device__ __forceinline__ uint2 origin_of(const SweepParams& P, uint32_t s) {
+  const uint4 o = philox(kTagOrigin << 28, 0u, s, P.sample, P.k0, P.k1);
+  return make_uint2(o.x & (P.g.L - 1u), o.y & (P.g.L - 1u));
+}
+
 // Draws part `part` of `parts` (1 or 2) of a tile's blocks.
 template <bool kGeneral>
 __device__ __forceinline__ void draw_tile(const SweepParams& P, const QuadTab& tab, TileRand<kGeneral>& B,
                                           uint32_t tid, uint32_t s, uint32_t lane, uint32_t part, uint32_t parts) {
   if (part == 0u) {
     const uint32_t w = philox(kTagSet << 28, tid, s, P.sample, P.k0, P.k1).x;
-    const uint4 o = philox(kTagOrigin << 28, 0u, s, P.sample, P.k0, P.k1);
+    const uint2 o = origin_of(P, s + 1u);
     if (lane < kRounds) {
       B.at[lane] = tab.at[(w >> (2u * lane)) & 3u];
       B.sh[lane] = tab.sh[(w >> (2u * lane)) & 3u];
     }
-    if (lane == 0u) { B.origin[0] = o.x & (P.g.L - 1u); B.origin[1] = o.y & (P.g.L - 1u); }
+    if (lane == 0u) { B.origin[0] = o.x; B.origin[1] = o.y; }
   }
   uint4 o[4];
   if constexpr (kGeneral) {
@@ -184,16 +190,27 @@ struct Window {
   uint32_t T[4][4], hx[4], hy[4], left[4], up[4];
 };
 
+// Where a window's words are (word indices of a lattice in global memory, or
+// shared addresses over a cluster): they depend on the origins alone, so they
+// are worked out while the barrier before the step is pending. For plane row
+// y, column x of the window: c the word its bits start in, n the next block
+// column's, sh the bit they start at; h the row below (lane 31 needs it), u the
+// row above (lane 0) and b3 the block column left of column 3's (kHalo = 2).
+struct WinAddr {
+  uint32_t c[4][4], n[4][4], h[4][2], u[4][2], b3[4], sh[4];
+};
+
 // The window whose site (0,0) is site (X0, Y0) of the frame the lattice is
 // held in (geometry as in run::sweep_run, kpz_run.cuh). kHalo: 0 the tile
 // alone, 1 with the column right of it (hx) and the row below it (hy), 2 also
 // the column left of it and the row above.
 template <int kHalo>
-__device__ __forceinline__ void load_window(const Geometry& g, const GlobalLat lat, uint32_t lane, uint32_t X0,
-                                            uint32_t Y0, Window& w) {
+__device__ __forceinline__ void window_at(const Geometry& g, uint32_t lane, uint32_t X0, uint32_t Y0, WinAddr& w) {
   const uint32_t NR = g.NR, NB = g.NB;
+  X0 &= g.L - 1u;
+  Y0 &= g.L - 1u;
   const uint32_t by = Y0 & 3u, Rb = Y0 >> 2, bx = X0 & 3u, a = X0 >> 2;
-  uint32_t offY[4], sh[4], w0[4], w1[4], wm3 = 0u;
+  uint32_t offY[4];
 #pragma unroll
   for (uint32_t yq = 0; yq < 4; ++yq)
     offY[yq] = ((by + yq) & 3u) * 4u * NR + ((Rb + lane + ((by + yq) >> 2)) & (NR - 1u));
@@ -201,35 +218,44 @@ __device__ __forceinline__ void load_window(const Geometry& g, const GlobalLat l
   const uint32_t offU = ((by + 3u) & 3u) * 4u * NR + ((Rb - 1u + ((by + 3u) >> 2)) & (NR - 1u));   // row above
 #pragma unroll
   for (uint32_t xq = 0; xq < 4; ++xq) {
-    const uint32_t st = (a + ((bx + xq) >> 2)) & (g.L / 4u - 1u);
-    const uint32_t kx = st >> 5, offX = ((bx + xq) & 3u) * NR;
-    sh[xq] = st & 31u;
-    w0[xq] = kx * kPlanes * NR + offX;
-    w1[xq] = ((kx + 1u) & (NB - 1u)) * kPlanes * NR + offX;
-    if (xq == 3) wm3 = ((kx + NB - 1u) & (NB - 1u)) * kPlanes * NR + offX;
+    const uint32_t st = (a + ((bx + xq) >> 2)) & (g.L / 4u - 1u), kx = st >> 5, offX = ((bx + xq) & 3u) * NR;
+    const uint32_t w0 = kx * kPlanes * NR + offX, w1 = ((kx + 1u) & (NB - 1u)) * kPlanes * NR + offX;
+    w.sh[xq] = st & 31u;
+#pragma unroll
+    for (uint32_t yq = 0; yq < 4; ++yq) {
+      w.c[yq][xq] = w0 + offY[yq];
+      w.n[yq][xq] = w1 + offY[yq];
+      if (kHalo == 2 && xq == 3) w.b3[yq] = ((kx + NB - 1u) & (NB - 1u)) * kPlanes * NR + offX + offY[yq];
+    }
+    if (kHalo >= 1) { w.h[xq][0] = w0 + offH; w.h[xq][1] = w1 + offH; }
+    if (kHalo == 2) { w.u[xq][0] = w0 + offU; w.u[xq][1] = w1 + offU; }
   }
+}
+
+template <int kHalo, class Load>
+__device__ __forceinline__ void fetch_window(const WinAddr& a, Load ld, Window& w) {
   uint32_t C[4][4], N[4][4], H[4][2], U[4][2], B3[4];
 #pragma unroll
   for (uint32_t xq = 0; xq < 4; ++xq) {
 #pragma unroll
     for (uint32_t yq = 0; yq < 4; ++yq) {
-      C[yq][xq] = lat.ld(w0[xq] + offY[yq]);
-      N[yq][xq] = lat.ld(w1[xq] + offY[yq]);
-      if (kHalo == 2 && xq == 3) B3[yq] = lat.ld(wm3 + offY[yq]);
+      C[yq][xq] = ld(a.c[yq][xq]);
+      N[yq][xq] = ld(a.n[yq][xq]);
+      if (kHalo == 2 && xq == 3) B3[yq] = ld(a.b3[yq]);
     }
-    if (kHalo >= 1) { H[xq][0] = lat.ld(w0[xq] + offH); H[xq][1] = lat.ld(w1[xq] + offH); }   // lane 31 needs it
-    if (kHalo == 2) { U[xq][0] = lat.ld(w0[xq] + offU); U[xq][1] = lat.ld(w1[xq] + offU); }   // lane 0 needs it
+    if (kHalo >= 1) { H[xq][0] = ld(a.h[xq][0]); H[xq][1] = ld(a.h[xq][1]); }
+    if (kHalo == 2) { U[xq][0] = ld(a.u[xq][0]); U[xq][1] = ld(a.u[xq][1]); }
   }
 #pragma unroll
   for (uint32_t xq = 0; xq < 4; ++xq) {
 #pragma unroll
     for (uint32_t yq = 0; yq < 4; ++yq) {
-      w.T[yq][xq] = __funnelshift_r(C[yq][xq], N[yq][xq], sh[xq]);
-      if (kHalo >= 1 && xq == 0) w.hx[yq] = (N[yq][0] >> sh[0]) & 1u;
-      if (kHalo == 2 && xq == 3) w.left[yq] = ((sh[3] ? C[yq][3] : B3[yq]) >> ((sh[3] + 31u) & 31u)) & 1u;
+      w.T[yq][xq] = __funnelshift_r(C[yq][xq], N[yq][xq], a.sh[xq]);
+      if (kHalo >= 1 && xq == 0) w.hx[yq] = (N[yq][0] >> a.sh[0]) & 1u;
+      if (kHalo == 2 && xq == 3) w.left[yq] = ((a.sh[3] ? C[yq][3] : B3[yq]) >> ((a.sh[3] + 31u) & 31u)) & 1u;
     }
-    if (kHalo >= 1) w.hy[xq] = __funnelshift_r(H[xq][0], H[xq][1], sh[xq]);
-    if (kHalo == 2) w.up[xq] = __funnelshift_r(U[xq][0], U[xq][1], sh[xq]);
+    if (kHalo >= 1) w.hy[xq] = __funnelshift_r(H[xq][0], H[xq][1], a.sh[xq]);
+    if (kHalo == 2) w.up[xq] = __funnelshift_r(U[xq][0], U[xq][1], a.sh[xq]);
   }
 }
 
@@ -302,6 +328,11 @@ __device__ __forceinline__ uint32_t phase_set(const SweepParams& P, uint32_t s, 
   return phase == 0u ? perm[0] : phase == 1u ? perm[1] : phase == 2u ? perm[2] : perm[3];
 }
 
+// A step of a tile warp: sweep, set (kSets) and tile.
+struct Step {
+  uint32_t s, q, tx, ty;
+};
+
 __device__ __forceinline__ void bar_sync(uint32_t id, uint32_t n) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
@@ -360,89 +391,107 @@ __global__ void __launch_bounds__(320, 1) resident_grid_kernel(const SweepParams
   const uint32_t c = blockIdx.x * wpc + slot;    // this warp's tile of every step
   const uint32_t across = kSets ? P.ntx / 2u : P.ntx, cy = c / across, cx = c - cy * across;
   const bool live = c < tiles;
-  // Sweep and tile of step k.
-  auto place = [&](uint32_t k, uint32_t& s, uint32_t& tx, uint32_t& ty) {
-    s = t0 + (kSets ? k >> 2 : k);
-    const uint32_t set = kSets ? phase_set(P, s, k & 3u) : 0u;
-    tx = kSets ? 2u * cx + (set & 1u) : cx;
-    ty = kSets ? 2u * cy + (set >> 1) : cy;
-  };
   const uint32_t L = P.g.L, words = L * L / 32u;
-  uint32_t s, tx, ty, ox = 0u, oy = 0u, px = 0u, py = 0u;
+  Step st;
+  // Sweep and tile of step k.
+  auto place = [&](uint32_t k) {
+    st.s = t0 + (kSets ? k >> 2 : k);
+    st.q = kSets ? phase_set(P, st.s, k & 3u) : 0u;
+    st.tx = kSets ? 2u * cx + (st.q & 1u) : cx;
+    st.ty = kSets ? 2u * cy + (st.q >> 1) : cy;
+  };
   if (maker) {
-    place(0u, s, tx, ty);
-    if (live) draw_tile<kGeneral>(P, tab, rnd[slot], ty * P.ntx + tx, s, lane, part, makers);
+    place(0u);
+    if (live) draw_tile<kGeneral>(P, tab, rnd[slot], st.ty * P.ntx + st.tx, st.s, lane, part, makers);
+    bar_sync(3, blockDim.x - 32u);
+    for (uint32_t k = 0; k <= nsteps; ++k) {
+      if (k != 0u) {
+        bar_sync(2, blockDim.x);
+        if (*(volatile uint32_t*)&stop) return;
+      }
+      if (k + 1u < nsteps && live) {
+        place(k + 1u);
+        draw_tile<kGeneral>(P, tab, rnd[((k + 1u) & 1u) * wpc + slot], st.ty * P.ntx + st.tx, st.s, lane, part, makers);
+      }
+      bar_arrive(1, blockDim.x);
+    }
+    return;
   }
+  // The window's addresses ahead of the barrier: L = 2048, p = 1 2.96 us a sweep
+  // against 3.05; general rates gain nothing (L = 4096 7.97 against 7.89).
+  constexpr bool kEarly = !kSets && !kGeneral;
+  WinAddr at;
+  uint32_t ox = 0u, oy = 0u, rx = 0u, ry = 0u;   // origin; its offset in the frame before
+  // All that can be known of step k before the barrier in front of it.
+  auto plan = [&](uint32_t k) {
+    const bool back = k == nsteps;               // the fixed frame again
+    place(k);
+    if (!kSets || (k & 3u) == 0u) {
+      const uint32_t* o = rnd[(makers ? ((k - 1u) & 1u) * wpc : 0u) + slot].origin;
+      const uint2 next = back ? make_uint2(0u, 0u) : k == 0u ? origin_of(P, t0) : make_uint2(o[0], o[1]);
+      rx = next.x - ox;
+      ry = next.y - oy;
+      ox = next.x;
+      oy = next.y;
+    }
+    if (!makers) {
+      __syncwarp();
+      if (live && !back) draw_tile<kGeneral>(P, tab, rnd[slot], st.ty * P.ntx + st.tx, st.s, lane, 0u, 1u);
+      __syncwarp();
+    }
+    if constexpr (kEarly) window_at<1>(P.g, lane, rx + st.tx * kTile, ry + st.ty * kTile, at);
+  };
   if (makers) bar_sync(3, blockDim.x - 32u);
+  plan(0u);
   for (uint32_t k = 0; k <= nsteps; ++k) {
-    if (k != 0u && makers) {
+    const uint32_t sw = kSets ? k >> 2 : k;      // sweeps before this step
+    const bool back = k == nsteps;
+    const TileRand<kGeneral>& B = rnd[(makers ? (k & 1u) * wpc : 0u) + slot];
+    if (k != 0u) {
       bar_sync(2, blockDim.x);
       if (*(volatile uint32_t*)&stop) return;
     }
-    if (maker) {
-      if (k + 1u < nsteps && live) {
-        place(k + 1u, s, tx, ty);
-        draw_tile<kGeneral>(P, tab, rnd[((k + 1u) & 1u) * wpc + slot], ty * P.ntx + tx, s, lane, part, makers);
-      }
-    } else {
-      const uint32_t sw = kSets ? k >> 2 : k;    // sweeps before this step
-      const bool back = k == nsteps;             // the fixed frame again
-      TileRand<kGeneral>& B = rnd[(makers ? (k & 1u) * wpc : 0u) + slot];
-      place(k, s, tx, ty);
-      if (!kSets || (k & 3u) == 0u) {
-        px = ox;
-        py = oy;
-      }
-      if (!makers) {
-        if (live && !back) draw_tile<kGeneral>(P, tab, B, ty * P.ntx + tx, s, lane, 0u, 1u);
-        __syncwarp();
-        if (k != 0u) {
-          bar_sync(2, blockDim.x);
-          if (*(volatile uint32_t*)&stop) return;
-        }
-      }
-      if (!kSets || (k & 3u) == 0u) {
-        ox = back ? 0u : B.origin[0];
-        oy = back ? 0u : B.origin[1];
-      }
-      const GlobalLat from{sw == 0u ? P.lat : scratch + ((sw - 1u) & 1u) * words};
-      const GlobalLat to{back ? P.lat : scratch + (sw & 1u) * words};
-      if (live) {
-        Window w;
-        const uint32_t rx = ox - px, ry = oy - py;   // new frame in the old one
-        if (kSets && (back || (k & 3u) == 0u)) {     // the four tiles of this warp change frames
+    const GlobalLat from{sw == 0u ? P.lat : scratch + ((sw - 1u) & 1u) * words};
+    const GlobalLat to{back ? P.lat : scratch + (sw & 1u) * words};
+    auto ld = [&](uint32_t i) { return from.ld(i); };
+    if (live) {
+      Window w;
+      if (kSets && (back || (k & 3u) == 0u)) {   // the four tiles of this warp change frames
 #pragma unroll 1
-          for (uint32_t q = 0; q < 4u; ++q) {
-            const uint32_t qx = 2u * cx + (q & 1u), qy = 2u * cy + (q >> 1);
-            if (!back && qx == tx && qy == ty) continue;
-            load_window<0>(P.g, from, lane, (rx + qx * kTile) & (L - 1u), (ry + qy * kTile) & (L - 1u), w);
-            store_tile(P.g, to, lane, qx, qy, w.T);
-          }
+        for (uint32_t q = 0; q < 4u; ++q) {
+          if (!back && q == st.q) continue;
+          const uint32_t qx = 2u * cx + (q & 1u), qy = 2u * cy + (q >> 1);
+          WinAddr aq;
+          window_at<0>(P.g, lane, rx + qx * kTile, ry + qy * kTile, aq);
+          fetch_window<0>(aq, ld, w);
+          store_tile(P.g, to, lane, qx, qy, w.T);
         }
-        if (kSets) {
-          if (!back) {
-            if ((k & 3u) == 0u)
-              load_window<2>(P.g, from, lane, (rx + tx * kTile) & (L - 1u), (ry + ty * kTile) & (L - 1u), w);
-            else
-              load_tile(P.g, to, lane, tx, ty, w);
-            tile_rounds<kGeneral, true>(P, w, mem[slot], tab, B, lane, s, ox, oy, tx, ty);
-            store_tile(P.g, to, lane, tx, ty, w.T);
-          }
+      }
+      if (!(kSets && back)) {
+        if constexpr (!kSets) {
+          if constexpr (!kEarly) window_at<1>(P.g, lane, rx + st.tx * kTile, ry + st.ty * kTile, at);
+          fetch_window<1>(at, ld, w);
+        } else if ((k & 3u) == 0u) {
+          window_at<2>(P.g, lane, rx + st.tx * kTile, ry + st.ty * kTile, at);
+          fetch_window<2>(at, ld, w);
         } else {
-          load_window<1>(P.g, from, lane, (rx + tx * kTile) & (L - 1u), (ry + ty * kTile) & (L - 1u), w);
-          if (!back) tile_rounds<kGeneral, false>(P, w, mem[slot], tab, B, lane, s, ox, oy, tx, ty);
-          store_tile(P.g, to, lane, tx, ty, w.T);
+          load_tile(P.g, to, lane, st.tx, st.ty, w);
         }
+        if (!back) tile_rounds<kGeneral, kSets>(P, w, mem[slot], tab, B, lane, st.s, ox, oy, st.tx, st.ty);
+        store_tile(P.g, to, lane, st.tx, st.ty, w.T);
       }
     }
     bar_arrive(1, blockDim.x);
+    if (k < nsteps) plan(k + 1u);
   }
 }
 
 // Cluster version (up to 64 tiles at a time): one cluster of 1 to 16 blocks
 // holds the whole lattice in its shared memory, two frames of it by turns;
 // windows are read over distributed shared memory and the hardware's cluster
-// barrier ends a step. Warps of a block: a tile warp for each of its units,
+// barrier ends a step; between arriving and waiting the tile warps work out the
+// next window's addresses (L = 512, p = 1: 2.18 -> 1.95 us a sweep; an mbarrier
+// in each block, raised by every tile warp of the cluster, took 2.06). Warps of a block: a tile warp for each of its units,
 // `makers` drawing warps for each.
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ uint32_t map_to(uint32_t addr, uint32_t cta) {
@@ -455,8 +504,11 @@ __device__ __forceinline__ uint32_t ld_cluster(uint32_t addr) {
   asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
   return v;
 }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  cluster_arrive();
+  cluster_wait();
 }
 
 // The lattice over the cluster: a block's frame holds 1 << lg units of one
@@ -478,16 +530,16 @@ struct ClusterLat {
   }
 };
 
-// load_window over the cluster.
+// window_at over the cluster.
 template <int kHalo, bool kSets>
-__device__ __forceinline__ void load_window_cluster(const ClusterLat<kSets>& lat, uint32_t lane, uint32_t X0, uint32_t Y0,
-                                                    Window& w) {
+__device__ __forceinline__ void window_at_cluster(const ClusterLat<kSets>& lat, uint32_t lane, uint32_t X0, uint32_t Y0,
+                                                  WinAddr& w) {
   const uint32_t L = lat.NR * 4u;
   X0 &= L - 1u;
   Y0 &= L - 1u;
   const uint32_t by = Y0 & 3u, Rb = Y0 >> 2, bx = X0 & 3u, a = X0 >> 2, K = a >> 5;
   // Plane 0 of block columns K, K + 1, K + 2 at cell rows Rb + lane, Rb + lane
-  // + 1, of the row below the tile (lane 31 needs it) and the one above (lane 0).
+  // + 1, of the row below the tile and the one above.
   uint32_t at[4][3];
 #pragma unroll
   for (uint32_t i = 0; i < (kHalo == 2 ? 4u : kHalo ? 3u : 2u); ++i) {
@@ -495,44 +547,38 @@ __device__ __forceinline__ void load_window_cluster(const ClusterLat<kSets>& lat
 #pragma unroll
     for (uint32_t j = 0; j < 3u; ++j) at[i][j] = lat.at(K + j, R);
   }
-  uint32_t C[4][4], N[4][4], H[4][2], U[4][2], B3[4], sh[4];
 #pragma unroll
   for (uint32_t xq = 0; xq < 4; ++xq) {
     const uint32_t st = a + ((bx + xq) >> 2), x4 = (bx + xq) & 3u;
-    sh[xq] = st & 31u;
+    w.sh[xq] = st & 31u;
     const bool next = (st >> 5) != K;   // carried into the next block column
-    auto two = [&](uint32_t r0, uint32_t r1, uint32_t r2, uint32_t p, uint32_t& c, uint32_t& n) {
-      c = ld_cluster((next ? r1 : r0) + p);
-      n = ld_cluster((next ? r2 : r1) + p);
-    };
 #pragma unroll
     for (uint32_t yq = 0; yq < 4; ++yq) {
-      const uint32_t y4 = (by + yq) & 3u, p = plane(y4, x4) * 128u;
+      const uint32_t p = plane((by + yq) & 3u, x4) * 128u;
       const bool wrap = by + yq >= 4u;
-      two(wrap ? at[1][0] : at[0][0], wrap ? at[1][1] : at[0][1], wrap ? at[1][2] : at[0][2], p, C[yq][xq], N[yq][xq]);
-      if (kHalo == 2 && xq == 3) B3[yq] = ld_cluster(lat.at((st >> 5) - 1u, Rb + lane + (wrap ? 1u : 0u)) + p);
+      w.c[yq][xq] = (wrap ? (next ? at[1][1] : at[1][0]) : (next ? at[0][1] : at[0][0])) + p;
+      w.n[yq][xq] = (wrap ? (next ? at[1][2] : at[1][1]) : (next ? at[0][2] : at[0][1])) + p;
+      if (kHalo == 2 && xq == 3) w.b3[yq] = lat.at((st >> 5) - 1u, Rb + lane + (wrap ? 1u : 0u)) + p;
     }
-    if (kHalo) two(at[2][0], at[2][1], at[2][2], plane(by, x4) * 128u, H[xq][0], H[xq][1]);
-    if (kHalo == 2) two(at[3][0], at[3][1], at[3][2], plane((by + 3u) & 3u, x4) * 128u, U[xq][0], U[xq][1]);
-  }
-#pragma unroll
-  for (uint32_t xq = 0; xq < 4; ++xq) {
-#pragma unroll
-    for (uint32_t yq = 0; yq < 4; ++yq) {
-      w.T[yq][xq] = __funnelshift_r(C[yq][xq], N[yq][xq], sh[xq]);
-      if (kHalo && xq == 0) w.hx[yq] = (N[yq][0] >> sh[0]) & 1u;
-      if (kHalo == 2 && xq == 3) w.left[yq] = ((sh[3] ? C[yq][3] : B3[yq]) >> ((sh[3] + 31u) & 31u)) & 1u;
+    if (kHalo) {
+      const uint32_t p = plane(by, x4) * 128u;
+      w.h[xq][0] = (next ? at[2][1] : at[2][0]) + p;
+      w.h[xq][1] = (next ? at[2][2] : at[2][1]) + p;
     }
-    if (kHalo) w.hy[xq] = __funnelshift_r(H[xq][0], H[xq][1], sh[xq]);
-    if (kHalo == 2) w.up[xq] = __funnelshift_r(U[xq][0], U[xq][1], sh[xq]);
+    if (kHalo == 2) {
+      const uint32_t p = plane((by + 3u) & 3u, x4) * 128u;
+      w.u[xq][0] = (next ? at[3][1] : at[3][0]) + p;
+      w.u[xq][1] = (next ? at[3][2] : at[3][1]) + p;
+    }
   }
 }
 
 // load_tile over the cluster; own: this lane's words of the tile, 32 apart.
-__device__ __forceinline__ void load_tile_cluster(const ClusterLat<true>& lat, const uint32_t* own, uint32_t lane,
-                                                  uint32_t tx, uint32_t ty, Window& w) {
+__device__ __forceinline__ void load_tile_cluster(const ClusterLat<true>& lat, uint32_t lane, uint32_t tx, uint32_t ty,
+                                                  const uint32_t* own, Window& w) {
   const uint32_t R = ty * 32u + lane;
-  const uint32_t l = lat.at(tx - 1u, R), r = lat.at(tx + 1u, R), u = lat.at(tx, ty * 32u - 1u), d = lat.at(tx, ty * 32u + 32u);
+  const uint32_t l = lat.at(tx - 1u, R), r = lat.at(tx + 1u, R);
+  const uint32_t u = lat.at(tx, ty * 32u - 1u), d = lat.at(tx, ty * 32u + 32u);
 #pragma unroll
   for (uint32_t y = 0; y < 4; ++y) {
     w.left[y] = ld_cluster(l + plane(y, 3) * 128u) >> 31;
@@ -568,28 +614,37 @@ __global__ void __launch_bounds__(384, 1) resident_cluster_kernel(const SweepPar
   uint32_t* own = frame + slot * kTiles * kTileWords + lane;   // this lane's words, 32 apart; + the frame's and the tile's offset
   const uint32_t half = units * kTiles * kTileWords;           // words of one frame in this block
   const uint32_t nsteps = n * kTiles;
-  // Sweep, set and tile of step k.
-  auto place = [&](uint32_t k, uint32_t& s, uint32_t& q, uint32_t& tx, uint32_t& ty) {
-    s = t0 + k / kTiles;
-    q = kSets ? phase_set(P, s, k & 3u) : 0u;
-    tx = kSets ? 2u * ux + (q & 1u) : ux;
-    ty = kSets ? 2u * uy + (q >> 1) : uy;
+  Step st;
+  auto place = [&](uint32_t k) {
+    st.s = t0 + k / kTiles;
+    st.q = kSets ? phase_set(P, st.s, k & 3u) : 0u;
+    st.tx = kSets ? 2u * ux + (st.q & 1u) : ux;
+    st.ty = kSets ? 2u * uy + (st.q >> 1) : uy;
   };
-  Window w;
-  uint32_t s, q, tx, ty;
   if (maker) {
-    place(0u, s, q, tx, ty);
-    draw_tile<kGeneral>(P, tab, rnd[slot], ty * P.ntx + tx, s, lane, part, makers);
-  } else {
-#pragma unroll 1
-    for (uint32_t i = 0; i < kTiles; ++i) {
-      const uint32_t x = kSets ? 2u * ux + (i & 1u) : ux, y = kSets ? 2u * uy + (i >> 1) : uy;
-      const uint32_t o = x * kPlanes * P.g.NR + y * 32u + lane;
-#pragma unroll
-      for (uint32_t p = 0; p < kPlanes; ++p) own[i * kTileWords + p * 32u] = __ldcg(P.lat + o + p * P.g.NR);
+    place(0u);
+    draw_tile<kGeneral>(P, tab, rnd[slot], st.ty * P.ntx + st.tx, st.s, lane, part, makers);
+    cluster_sync();
+    for (uint32_t k = 0; k < nsteps; ++k) {
+      if (k + 1u < nsteps) {
+        place(k + 1u);
+        draw_tile<kGeneral>(P, tab, rnd[((k + 1u) & 1u) * units + slot], st.ty * P.ntx + st.tx, st.s, lane, part, makers);
+      }
+      cluster_sync();
     }
+    cluster_sync();
+    return;
   }
-  uint32_t px = 0u, py = 0u, ox = 0u, oy = 0u;
+#pragma unroll 1
+  for (uint32_t i = 0; i < kTiles; ++i) {
+    const uint32_t x = kSets ? 2u * ux + (i & 1u) : ux, y = kSets ? 2u * uy + (i >> 1) : uy;
+    const uint32_t o = x * kPlanes * P.g.NR + y * 32u + lane;
+#pragma unroll
+    for (uint32_t p = 0; p < kPlanes; ++p) own[i * kTileWords + p * 32u] = __ldcg(P.lat + o + p * P.g.NR);
+  }
+  Window w;
+  WinAddr at;
+  uint32_t ox = 0u, oy = 0u, rx = 0u, ry = 0u;   // origin; its offset in the frame before
   auto lattice = [&](uint32_t sweep) {   // as it stands after `sweep` sweeps of this launch
     return ClusterLat<kSets>{smem_u32(frame + (sweep & 1u) * half), lg, P.g.NR, P.g.NB, P.ntx};
   };
@@ -597,48 +652,54 @@ __global__ void __launch_bounds__(384, 1) resident_cluster_kernel(const SweepPar
 #pragma unroll
     for (uint32_t p = 0; p < kPlanes; ++p) to[p * 32u] = w.T[p >> 2][p & 3u];
   };
+  // All that can be known of step k before the barrier in front of it.
+  auto plan = [&](uint32_t k) {
+    place(k);
+    if (!kSets || (k & 3u) == 0u) {
+      const uint32_t* o = rnd[((k - 1u) & 1u) * units + slot].origin;
+      const uint2 next = k == 0u ? origin_of(P, t0) : make_uint2(o[0], o[1]);
+      rx = next.x - ox;
+      ry = next.y - oy;
+      ox = next.x;
+      oy = next.y;
+      if constexpr (!kSets) window_at_cluster<1>(lattice(k), lane, rx + st.tx * kTile, ry + st.ty * kTile, at);
+    }
+  };
+  auto ld = [](uint32_t a) { return ld_cluster(a); };
   cluster_sync();
+  plan(0u);
   for (uint32_t k = 0; k < nsteps; ++k) {
-    const uint32_t buf = k & 1u, sw = k / kTiles;
-    if (maker) {
-      if (k + 1u < nsteps) {
-        place(k + 1u, s, q, tx, ty);
-        draw_tile<kGeneral>(P, tab, rnd[(buf ^ 1u) * units + slot], ty * P.ntx + tx, s, lane, part, makers);
-      }
-    } else {
-      const TileRand<kGeneral>& B = rnd[buf * units + slot];
-      place(k, s, q, tx, ty);
-      uint32_t* to = own + ((sw + 1u) & 1u) * half;
-      if (!kSets || (k & 3u) == 0u) {   // the sweep's first step: the frame changes
-        px = ox;
-        py = oy;
-        ox = B.origin[0];
-        oy = B.origin[1];
-        if (kSets) {
+    const uint32_t sw = k / kTiles;
+    const TileRand<kGeneral>& B = rnd[(k & 1u) * units + slot];
+    uint32_t* to = own + ((sw + 1u) & 1u) * half;
+    if (!kSets || (k & 3u) == 0u) {   // the sweep's first step: the frame changes
+      if (kSets) {
 #pragma unroll 1
-          for (uint32_t i = 0; i < 4u; ++i) {
-            if (i == q) continue;
-            load_window_cluster<0>(lattice(sw), lane, ox - px + (2u * ux + (i & 1u)) * kTile,
-                                   oy - py + (2u * uy + (i >> 1)) * kTile, w);
-            put(to + i * kTileWords);
-          }
+        for (uint32_t i = 0; i < 4u; ++i) {
+          if (i == st.q) continue;
+          WinAddr aq;
+          window_at_cluster<0>(lattice(sw), lane, rx + (2u * ux + (i & 1u)) * kTile, ry + (2u * uy + (i >> 1)) * kTile, aq);
+          fetch_window<0>(aq, ld, w);
+          put(to + i * kTileWords);
         }
-        load_window_cluster<kSets ? 2 : 1>(lattice(sw), lane, ox - px + tx * kTile, oy - py + ty * kTile, w);
-      } else if constexpr (kSets) {
-        load_tile_cluster(lattice(sw + 1u), to + q * kTileWords, lane, tx, ty, w);
       }
-      tile_rounds<kGeneral, kSets>(P, w, mem[slot], tab, B, lane, s, ox, oy, tx, ty);
-      put(to + q * kTileWords);
+      if (kSets) window_at_cluster<2>(lattice(sw), lane, rx + st.tx * kTile, ry + st.ty * kTile, at);
+      fetch_window<kSets ? 2 : 1>(at, ld, w);
+    } else if constexpr (kSets) {
+      load_tile_cluster(lattice(sw + 1u), lane, st.tx, st.ty, to + st.q * kTileWords, w);
     }
-    cluster_sync();
+    tile_rounds<kGeneral, kSets>(P, w, mem[slot], tab, B, lane, st.s, ox, oy, st.tx, st.ty);
+    put(to + st.q * kTileWords);
+    cluster_arrive();
+    if (k + 1u < nsteps) plan(k + 1u);
+    cluster_wait();
   }
-  if (!maker) {
 #pragma unroll 1
-    for (uint32_t i = 0; i < kTiles; ++i) {
-      const uint32_t x = kSets ? 2u * ux + (i & 1u) : ux, y = kSets ? 2u * uy + (i >> 1) : uy;
-      load_window_cluster<0>(lattice(n), lane, x * kTile - ox, y * kTile - oy, w);
-      store_tile(P.g, GlobalLat{P.lat}, lane, x, y, w.T);
-    }
+  for (uint32_t i = 0; i < kTiles; ++i) {   // the fixed frame again
+    const uint32_t x = kSets ? 2u * ux + (i & 1u) : ux, y = kSets ? 2u * uy + (i >> 1) : uy;
+    window_at_cluster<0>(lattice(n), lane, x * kTile - ox, y * kTile - oy, at);
+    fetch_window<0>(at, ld, w);
+    store_tile(P.g, GlobalLat{P.lat}, lane, x, y, w.T);
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) *const_cast<uint64_t*>(P.t_dev) += n;
   cluster_sync();   // no block leaves while its shared memory is read
@@ -657,9 +718,9 @@ struct Shape {
 // pay while an SM has at most two tiles; with eight they take the issue slots
 // the tile warps need (L = 4096 at p = 0.95: 9.0 us a sweep with them, 7.9
 // without). The cluster has 16 SMs: at p = 1 it serves four tiles each (L =
-// 1024 2.9 us a sweep, 3.1 on a grid; tile sets at L = 2048 12.2, 13.8), at
-// general rates one (L = 512 3.4, L = 1024 4.7 against 4.3 on a grid; tile sets
-// at L = 1024 14.4 against 19.0, at L = 2048 21.0 against 19.1). Beyond 1024
+// 1024 2.7 us a sweep, 2.9 on a grid; tile sets at L = 2048 11.6, 13.4), at
+// general rates one (L = 512 3.15, on a grid 4.2; L = 1024 4.5 against 4.3; tile
+// sets at L = 1024 13.5 against 18.1, at L = 2048 20.2 against 18.6). Beyond 1024
 // tiles an SM would have more than two tiles a scheduler, and work, not
 // latency, is the bound.
 Shape shape_of(const SweepParams& P, bool tilesets, bool general, bool cluster) {
