@@ -619,7 +619,7 @@ def main():
         roofline_general = {"bound": "alu", "achieved": ach, "peak": alu_peak, "unit": "Top/s",
                             "frac": ach / alu_peak,
                             "traffic": measured_traffic(L, "sweep_kernel_general_L65536.md"),
-                            "kernel": "sweep_kernel (general rates)", "p": 0.95, "q": 0.05,
+                            "kernel": "sweep_chain_kernel (general rates)", "p": 0.95, "q": 0.05,
                             "alg_ops_per_attempt": K_ALG_ALU_GENERAL, "candidate_density": C_CAND,
                             "launch_ms": per_g * 1e3, "sweeps_timed": ng, "start": "t = 5 from the flat start",
                             "attempts_per_s": L * L / per_g,

@@ -73,7 +73,8 @@ typedef struct {
                              execution only. With run and warps_per_cta both 0,
                              lattices of 128 x 128 tiles and 4 x 4 cells up to
                              L = 4096 (tile sets: L = 8192) run all sweeps of a
-                             kpz_run call in one launch instead of one each      */
+                             kpz_run call in one launch instead of one each; four
+                             or more sweeps of larger ones are chained in a launch */
     void* stream;         /* cudaStream_t to queue work on (NULL = default stream)  */
     void* dev_buf;        /* optional caller-owned device memory for the lattice and
                              its scratch; at least kpz_device_bytes(L) bytes,

@@ -79,7 +79,7 @@ struct kpz_ctx {
   uint32_t Tp = 0, Tq = 0, nlev = 0, sample = 0;
   double p = 0.0, q = 0.0;             // as given to kpz_init (checkpoint header)
   uint64_t seed = 0;
-  uint32_t run = 1, wpc = 8;
+  uint32_t run = 1, run_many = 1, wpc = 8;
   uint32_t tile_y = 128;               // tile height in sites (128 or 256)
   uint32_t decomposition = 0;          // device layer: 0 dead border, 1 tile sets
   uint32_t cell = 4;                   // work-group cell edge: 4 or 2
@@ -98,7 +98,7 @@ struct kpz_ctx {
   uint32_t* hcar = nullptr;            // import: height of (0, j0) modulo 4
   uint32_t* queue = nullptr;           // sweep work queue (zero between launches)
   GridSync* sync = nullptr;            // persistent kernels: grid barrier and error flag
-  uint32_t resident = 0;               // kpz_run's resident kernel (resident_kind), 0: one launch per sweep
+  uint32_t resident = 0;               // kpz_run's resident kernel (resident_kind), 0: the work queue
   bool direct_host = false;            // the GPU reads and writes pageable host memory itself
   bool unchecked = false;              // persistent launches since the error flag was read
   int32_t* col0 = nullptr;             // h(0,j); roughness: the bands' partial sums
@@ -307,19 +307,25 @@ kpz_status kpz_init(kpz_ctx** out, uint32_t L, double p, double q, uint64_t seed
   ctx->cell = o.cell ? o.cell : 4u;
   ctx->colour_m = o.colour_sparsity ? o.colour_sparsity : 3u;
   // Default schedule of the work-queue sweep, measured on GB300 (results do not
-  // depend on it): about 8192 runs, two to three for each resident warp, but
-  // none longer than 1/32 of a tile row, which keeps the last wave short. A
-  // longer run saves window prologues, start copies and edge write-backs, a
-  // shorter one fills the GPU: us per sweep at p = 1 / 0.95 with runs of 1, 2,
-  // 4, 8 tiles, L = 8192: 24 / 37, 25 / 50, 30 / -, 37 / 128; L = 16384: 55 / 107,
-  // 47 / 102, 63 / 115, 62 / 200; L = 32768: 178 / -, 155 / -, 142 / 349, 138 /
-  // 340; L = 65536: runs of 8 482 / 1270, 16 465 / 1270. From L = 65536 4-warp
-  // CTAs for 128-row tiles (465 against 485 at p = 1), below it 8-warp ones.
+  // depend on it). A longer run saves window prologues, start copies and edge
+  // write-backs, a shorter one fills the GPU. Sweeps that follow one another in
+  // a launch: about 4096 runs, none longer than 1/32 of a tile row; us per sweep
+  // at p = 1 / 0.95 with runs of 1, 2, 4, 8, 16 tiles, L = 8192: 14.3 / 24.7,
+  // 16.7 / 28.7, 17.3 / 33, - , -; L = 16384: - , 38 / 87, 37 / 81, 44 / 92, - ;
+  // L = 32768: - , - , 136 / 324, 120 / 310, 120 / 349; L = 65536: 8 487 / 1245, 16
+  // 462 / 1226. A sweep alone ends with a wave of its own and wants it short:
+  // about 8192 runs (L = 16384, p = 1: 47 with runs of 2, 63 with 4). From L =
+  // 65536 4-warp CTAs for 128-row tiles (462 against 485 at p = 1), below it
+  // 8-warp ones (L = 8192 14.3 against 14.4 and 22.9, L = 16384 37 against 38).
   const bool wide = ntx >= 512u;
   const uint32_t tiles = ntx * (L / ctx->tile_y);
-  uint32_t auto_run = 1u;
-  while (2u * auto_run <= std::min(tiles / 8192u, ntx / 32u)) auto_run *= 2u;
-  ctx->run = o.run ? o.run : auto_run;   // tiles per work-queue chunk
+  auto run_rule = [&](uint32_t runs) {
+    uint32_t r = 1u;
+    while (2u * r <= std::min(tiles / runs, ntx / 32u)) r *= 2u;
+    return r;
+  };
+  ctx->run = o.run ? o.run : run_rule(8192u);        // tiles per work-queue chunk
+  ctx->run_many = o.run ? o.run : run_rule(4096u);   // the same with sweeps chained (calls of four or more)
   ctx->wpc = o.warps_per_cta ? o.warps_per_cta : (wide && ctx->tile_y == kTile ? 4u : 8u);
   ctx->stream = (cudaStream_t)o.stream;
   if (o.dev_buf) {
@@ -405,12 +411,23 @@ kpz_status kpz_run(kpz_ctx* ctx, uint64_t n_mcs) {
       n_mcs -= chunk;
       continue;
     }
-    for (uint32_t i = 0; i < chunk; ++i) {
+    uint32_t most = 1u;   // sweeps of one launch
+    if (ctx->decomposition == 0u && chunk >= 4u) {
+      P.run = ctx->run_many;
+      P.runs_x = P.ntx / P.run;
+      most = sweeps_per_launch(P);
+      if (most > 1u) ctx->unchecked = true;   // the sweeps wait for one another
+    }
+    if (most == 1u) {
+      P.run = ctx->run;
+      P.runs_x = P.ntx / P.run;
+    }
+    for (uint32_t i = 0; i < chunk; i += most) {
       P.s_add = i;
       if (ctx->decomposition == 1u)      KPZ_CUDA(launch_sweep_tilesets(P, ctx->stream));
       else if (ctx->decomposition == 2u) KPZ_CUDA(launch_sweep_colour(P, ctx->colour_m, ctx->stream));
       else if (ctx->decomposition == 3u) KPZ_CUDA(launch_sweep_db2(P, ctx->stream));
-      else                               KPZ_CUDA(launch_sweep(P, ctx->wpc, ctx->stream));
+      else KPZ_CUDA(launch_sweep(P, ctx->wpc, std::min(most, chunk - i), (uint32_t*)ctx->io, ctx->sync, ctx->stream));
     }
     KPZ_CUDA(launch_advance(ctx->t_dev, chunk, ctx->stream));
     ctx->t_host += chunk;

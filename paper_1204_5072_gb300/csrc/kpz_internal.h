@@ -51,7 +51,12 @@ inline void set_philox_key(SweepParams& P, uint64_t seed) {
   P.k1 = (uint32_t)(seed >> 32);
 }
 
-cudaError_t launch_sweep(const SweepParams& P, uint32_t warps_per_cta, cudaStream_t st);
+// n sweeps from *t_dev + s_add on, 1 <= n <= sweeps_per_launch(P). For n > 1 done
+// is scratch for nty words, and a wait that runs out of time sets sync->err.
+struct GridSync;
+uint32_t sweeps_per_launch(const SweepParams& P);
+cudaError_t launch_sweep(const SweepParams& P, uint32_t warps_per_cta, uint32_t n, uint32_t* done, GridSync* sync,
+                         cudaStream_t st);
 cudaError_t launch_advance(uint64_t* t_dev, uint32_t n, cudaStream_t st);
 // One sweep of the tile-set variant of the device layer (kpz_tileset.cu):
 // four launches, one per tile set, in the order drawn for the sweep.
