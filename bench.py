@@ -18,7 +18,7 @@ measured pipe peak and the DRAM traffic of the committed ncu capture),
 path), `cpu_baseline` / `cpu_all_cores` / `cpu_rsu` (the oracle on a bounded
 sample), `clocks`, `gpu_launches`, `batch` (the 512-realisation batched
 workload at its 10^5-sweep cap in one persistent launch, with construction-free
-baselines -- one launch per realisation, one launch per sweep -- on a
+baselines -- one launch per realisation, one lattice after another -- on a
 stratified subset, per L bucket) and `surrogate` (trained on that batch's own
 curves with one size held out; held-out errors, planned run lengths against
 4 L^1.6, saturation times).
@@ -326,7 +326,7 @@ def _timed(fn):
 
 
 def _per_sweep_run(eng, lat, n, times):
-    """One realisation by one launch per sweep (kpz_run), W^2 at its sample times."""
+    """One realisation as a lattice of its own (kpz_run), W^2 at its sample times."""
     tp = 0
     for t in times:
         if t > n:

@@ -151,7 +151,7 @@ kpz_status kpz_reset(kpz_ctx* ctx);
 
 /* Queue n_mcs sweeps (n_mcs * L*L attempts) on the context's stream and
  * return; errors of the queued work surface at the next synchronising call
- * (KPZ_ETIMEOUT if a device-side barrier of a one-launch run gave up).      */
+ * (KPZ_ETIMEOUT if a device-side wait of the run gave up).      */
 kpz_status kpz_run(kpz_ctx* ctx, uint64_t n_mcs);
 
 /* Exact height sums and W^2 at the current time (eq. Wdef, Sec. 2.1).

@@ -210,7 +210,7 @@ kpz_status settle(kpz_ctx* ctx) {
   KPZ_CUDA(cudaMemcpyAsync(&err, &ctx->sync->err, sizeof(err), cudaMemcpyDeviceToHost, ctx->stream));
   KPZ_CUDA(cudaStreamSynchronize(ctx->stream));
   ctx->unchecked = false;
-  return err ? fail(ctx, KPZ_ETIMEOUT, "a grid barrier of kpz_run timed out") : KPZ_OK;
+  return err ? fail(ctx, KPZ_ETIMEOUT, "a device-side wait of kpz_run timed out") : KPZ_OK;
 }
 
 SweepParams sweep_params(const kpz_ctx* c) {
@@ -448,7 +448,7 @@ kpz_status kpz_roughness(kpz_ctx* ctx, kpz_rough* out) {
   const unsigned long long host[4] = {(unsigned long long)res[0], (unsigned long long)res[1],
                                       (unsigned long long)res[2], (unsigned long long)res[3]};
   ctx->unchecked = false;
-  if (res[4]) return fail(ctx, KPZ_ETIMEOUT, "a grid barrier of kpz_run timed out");
+  if (res[4]) return fail(ctx, KPZ_ETIMEOUT, "a device-side wait of kpz_run timed out");
   const uint64_t N = (uint64_t)ctx->g.L * ctx->g.L;
   out->t_mcs = ctx->t_host;
   out->n_sites = N;

@@ -1,6 +1,7 @@
-// kpz_gridsync.cuh -- building blocks of bounded grid-wide barriers in
-// cooperative launches: a counter that every block raises once a step, release
-// to acquire, with a wait that gives up after kWaitNs.
+// kpz_gridsync.cuh -- building blocks of bounded waits between blocks, release
+// to acquire: grid-wide barriers in cooperative launches (a counter that every
+// block raises once a step) and the row counters of chained sweeps; a wait
+// gives up after kWaitNs.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
