@@ -22,11 +22,11 @@
 // Microseconds per sweep, p = 1 / p = 0.95, against one launch per sweep with
 // runs of 8 tiles (and of one tile, the fastest there): L = 256 1.9 / 3.1
 // against 12.4 / 22.8 (10.2 / 15.9), L = 1024 2.7 / 4.3 against 25 / 63 (10.2 /
-// 17.7), L = 4096 3.9 / 7.9 against 29 / 80 (14.1 / 25.8); tile sets at L = 2048
+// 17.7), L = 4096 3.7 / 7.8 against 29 / 80 (14.1 / 25.8); tile sets at L = 2048
 // 11.7 / 18.4 against 44 at p = 1. At L = 512 (one tile a block, one tile warp
 // a scheduler) the 16 rounds take 2000 / 4300 cycles of a sweep's 3900 / 6400;
 // the rest is the window's trip and the barrier. At L = 4096 and general rates
-// the eight tiles of an SM bind it (logic and Philox pipes).
+// the seven tiles of an SM bind it (logic and Philox pipes).
 #include <algorithm>
 #include <mutex>
 
@@ -712,17 +712,21 @@ struct Shape {
   size_t smem;
 };
 
+constexpr uint32_t kSms = 152;   // GB300; where fewer are to be had, fits() says no
+
 // How a lattice is laid over the chip (wpc = 0: not served). p = 1 draws 8
 // blocks a tile and sweep, general rates 32; one warp draws a block in about
 // 120 cycles, an SM's quarter in 80 (the wide multiplies), so drawing warps
-// pay while an SM has at most two tiles; with eight they take the issue slots
+// pay while an SM has at most two tiles; with seven or eight they take the issue slots
 // the tile warps need (L = 4096 at p = 0.95: 9.0 us a sweep with them, 7.9
 // without). The cluster has 16 SMs: at p = 1 it serves four tiles each (L =
 // 1024 2.7 us a sweep, 2.9 on a grid; tile sets at L = 2048 11.6, 13.4), at
 // general rates one (L = 512 3.15, on a grid 4.2; L = 1024 4.5 against 4.3; tile
 // sets at L = 1024 13.5 against 18.1, at L = 2048 20.2 against 18.6). Beyond 1024
 // tiles an SM would have more than two tiles a scheduler, and work, not
-// latency, is the bound.
+// latency, is the bound. 1024 tiles go to 147 blocks of seven tile warps: with
+// eight on 128 of the 152 SMs L = 4096 took 3.94 us a sweep at p = 1 against 3.73
+// (the tiles of an SM share its LSU), tile sets at L = 8192 17.8 against 17.0.
 Shape shape_of(const SweepParams& P, bool tilesets, bool general, bool cluster) {
   Shape h{};
   const size_t rnd = general ? sizeof(TileRand<true>) : sizeof(TileRand<false>);
@@ -739,7 +743,7 @@ Shape shape_of(const SweepParams& P, bool tilesets, bool general, bool cluster) 
   }
   h.tiles = tilesets ? all / 4u : all;
   if (h.tiles > 1024u) return h;
-  h.wpc = std::max(1u, h.tiles / 128u);      // up to 128 blocks of 1 to 8 tile warps
+  h.wpc = std::max(1u, (h.tiles + kSms - 1u) / kSms);   // blocks of 1 to 7 tile warps, one on an SM
   h.grid = (h.tiles + h.wpc - 1u) / h.wpc;
   h.makers = h.wpc > 2u ? 0u : (general ? 2u : 1u);
   h.smem = h.wpc * ((h.makers ? 2u : 1u) * rnd + sizeof(TileMem));

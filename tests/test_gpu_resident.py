@@ -1,6 +1,6 @@
 """Lattices swept by the resident kernels (no execution knobs given, up to 1024
 tiles at a time): every layout -- one block, clusters of 4 and 16 blocks with
-one and four tiles each, grids with one, two and eight tile warps per block --
+one and four tiles each, grids with one, two and seven tile warps per block --
 against the oracle where it is quick and against the launch-per-sweep
 kernels elsewhere, bit for bit; runs split over calls, odd start parity, tile sets."""
 import numpy as np
