@@ -333,10 +333,16 @@ struct Step {
   uint32_t s, q, tx, ty;
 };
 
+// bar.* and barrier.cluster.*.aligned are only defined for a warp whose lanes
+// arrive together; divergent code comes before most of them (the atomic add of
+// the tile that holds site (0,0), a lane that draws origins), so the lanes are
+// brought together here.
 __device__ __forceinline__ void bar_sync(uint32_t id, uint32_t n) {
+  __syncwarp();
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 __device__ __forceinline__ void bar_arrive(uint32_t id, uint32_t n) {
+  __syncwarp();
   asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
@@ -504,8 +510,14 @@ __device__ __forceinline__ uint32_t ld_cluster(uint32_t addr) {
   asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
   return v;
 }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void cluster_sync() {
   cluster_arrive();
   cluster_wait();
