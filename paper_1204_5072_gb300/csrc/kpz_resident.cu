@@ -664,12 +664,11 @@ __global__ void __launch_bounds__(384, 1) resident_cluster_kernel(const SweepPar
 #pragma unroll
     for (uint32_t p = 0; p < kPlanes; ++p) to[p * 32u] = w.T[p >> 2][p & 3u];
   };
-  // All that can be known of step k before the barrier in front of it.
-  auto plan = [&](uint32_t k) {
+  // All that can be known of step k before the barrier in front of it; next:
+  // the origin of its sweep.
+  auto plan = [&](uint32_t k, const uint2 next) {
     place(k);
     if (!kSets || (k & 3u) == 0u) {
-      const uint32_t* o = rnd[((k - 1u) & 1u) * units + slot].origin;
-      const uint2 next = k == 0u ? origin_of(P, t0) : make_uint2(o[0], o[1]);
       rx = next.x - ox;
       ry = next.y - oy;
       ox = next.x;
@@ -679,7 +678,7 @@ __global__ void __launch_bounds__(384, 1) resident_cluster_kernel(const SweepPar
   };
   auto ld = [](uint32_t a) { return ld_cluster(a); };
   cluster_sync();
-  plan(0u);
+  plan(0u, origin_of(P, t0));
   for (uint32_t k = 0; k < nsteps; ++k) {
     const uint32_t sw = k / kTiles;
     const TileRand<kGeneral>& B = rnd[(k & 1u) * units + slot];
@@ -702,8 +701,11 @@ __global__ void __launch_bounds__(384, 1) resident_cluster_kernel(const SweepPar
     }
     tile_rounds<kGeneral, kSets>(P, w, mem[slot], tab, B, lane, st.s, ox, oy, st.tx, st.ty);
     put(to + st.q * kTileWords);
+    // Once every warp has arrived, the drawing warp may go on to overwrite this
+    // step's numbers, so the origin they hold is read before.
+    const uint2 next = make_uint2(B.origin[0], B.origin[1]);
     cluster_arrive();
-    if (k + 1u < nsteps) plan(k + 1u);
+    if (k + 1u < nsteps) plan(k + 1u, next);
     cluster_wait();
   }
 #pragma unroll 1

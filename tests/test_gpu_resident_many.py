@@ -32,3 +32,13 @@ def same_after(eng, L, p, q, decomposition, counts):
     (2048, 0.95, 0.05, 1), (4096, 1.0, 0.0, 1), (4096, 0.6, 0.3, 1)])
 def test_grid(eng, L, p, q, decomposition):
     same_after(eng, L, p, q, decomposition, (1000, 501))
+
+
+# One block, a cluster of 4 and of 16 blocks with one and four units each; the
+# drawing warps of a step run beside the tile warps of the step before.
+@pytest.mark.parametrize("L,p,q,decomposition", [
+    (128, 1.0, 0.0, 0), (256, 1.0, 0.0, 0), (512, 1.0, 0.0, 0), (1024, 1.0, 0.0, 0),
+    (128, 0.95, 0.05, 0), (256, 0.6, 0.3, 0), (512, 0.95, 0.05, 0),
+    (256, 1.0, 0.0, 1), (512, 0.95, 0.05, 1), (1024, 0.6, 0.3, 1), (1024, 1.0, 0.0, 1), (2048, 1.0, 0.0, 1)])
+def test_cluster(eng, L, p, q, decomposition):
+    same_after(eng, L, p, q, decomposition, (4000, 1501))
