@@ -55,14 +55,20 @@ using run::kMaxWarpsPerCta;
 
 // One warp: waits until the rows that ordered row i depends on have `want` chunks
 // done, and reports a chunk of row `prev` (~0: none) meanwhile; false when the
-// wait ran out of time.
+// wait ran out of time. Lanes 0..2 acquire the counters; a vote orders no memory,
+// so the warp is synchronised before the others read what the counters stand
+// for. That order is also what keeps the cp.async copies through L1 (kpz_run.cuh)
+// fresh now that sweeps share a launch.
 __device__ __forceinline__ bool rows_done(uint32_t* done, uint32_t i, uint32_t nty, uint32_t want, uint32_t prev,
                                           uint32_t lane, GridSync* sync) {
   const uint32_t* d = done + ((i + lane) & (nty - 1u));
   auto ready = [&] { return __all_sync(kFull, lane > 2u || gridsync::ld_acquire(d) >= want); };
   const bool ok = ready();
   if (lane == 0u && prev != ~0u) gridsync::red_release(done + prev);
-  if (ok) return true;
+  if (ok) {
+    __syncwarp();
+    return true;
+  }
   const uint64_t t0 = gridsync::now_ns();
   for (uint32_t it = 1; !ready(); ++it) {
     if ((it & 63u) == 0u &&
@@ -71,6 +77,7 @@ __device__ __forceinline__ bool rows_done(uint32_t* done, uint32_t i, uint32_t n
       return false;
     }
   }
+  __syncwarp();
   return true;
 }
 
