@@ -145,8 +145,11 @@ __device__ __forceinline__ bool wait_phase(uint32_t mbar, uint32_t parity) {
 }
 
 // 8 and 32 consecutive float32 columns of this warp's 32 tensor-memory lanes.
+// The aligned forms are only defined for a converged warp; lanes leave the wait
+// before one at a time.
 __device__ __forceinline__ void ld8(uint32_t ta, float (&v)[8]) {
   uint32_t r[8];
+  __syncwarp();
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                : "r"(ta));
@@ -156,6 +159,7 @@ __device__ __forceinline__ void ld8(uint32_t ta, float (&v)[8]) {
 }
 __device__ __forceinline__ void ld32(uint32_t ta, float (&v)[32]) {
   uint32_t r[32];
+  __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
       "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
@@ -258,6 +262,7 @@ __global__ void __launch_bounds__(tc::kThreads, kGrad ? 1 : 2)
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc::smem_u32(&mbar[1])));
   }
   if (warp == 0) {
+    __syncwarp();
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc::smem_u32(&taddr_s)),
                  "n"(kCols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
