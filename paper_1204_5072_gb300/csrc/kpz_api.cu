@@ -470,7 +470,9 @@ kpz_status kpz_heights(kpz_ctx* ctx, int64_t* host_out, int absolute) {
   const uint32_t L = ctx->g.L;
   KPZ_CUDA(launch_col0(ctx->lat, ctx->g, ctx->col0, ctx->stream));
   touch_pages(host_out, (size_t)L * L * 8);
-  if (ctx->direct_host) {   // the kernel stores to the caller's buffer itself
+  // The kernel stores to the caller's buffer itself, 16 bytes at a time; an
+  // int64 array may start at any multiple of 8, and such a one is copied to.
+  if (ctx->direct_host && ((uintptr_t)host_out & 15u) == 0) {
     KPZ_CUDA(launch_heights(ctx->lat, ctx->g, ctx->col0, 0, L, absolute ? ctx->h00 : nullptr, host_out, ctx->stream));
     KPZ_CUDA(cudaStreamSynchronize(ctx->stream));
     return settle(ctx);
