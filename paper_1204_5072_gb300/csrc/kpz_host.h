@@ -2,6 +2,7 @@
 #pragma once
 #include <algorithm>
 #include <cstddef>
+#include <cstdint>
 #include <cuda_runtime.h>
 
 #include <thread>
@@ -49,6 +50,24 @@ void host_slot_free(void* p);
 inline bool reaches_pageable(int device) {
   int v = 0;
   return cudaDeviceGetAttribute(&v, cudaDevAttrPageableMemoryAccess, device) == cudaSuccess && v != 0;
+}
+
+// Whether kernels may use the caller's float arrays in place: `in` (n_in of
+// them) read and `out` (may be null) written, sizes in bytes.
+// They need the type's alignment, which a copy does not, and an output apart
+// from every input: the call may read an input after it has begun to write.
+struct HostSpan {
+  const void* p;
+  size_t bytes;
+};
+inline bool usable_in_place(const HostSpan* in, int n_in, HostSpan out) {
+  const uintptr_t o = (uintptr_t)out.p;
+  bool ok = o % alignof(float) == 0;
+  for (int i = 0; i < n_in; ++i) {
+    const uintptr_t a = (uintptr_t)in[i].p;
+    ok = ok && a % alignof(float) == 0 && (!o || a + in[i].bytes <= o || o + out.bytes <= a);
+  }
+  return ok;
 }
 
 }  // namespace kpz

@@ -636,12 +636,15 @@ kpz_status kpz_mlp_params(kpz_mlp* m, float* params) {
 // Where the GPU reaches pageable host memory (its pages touched before it
 // writes them), predict and loss_grad read and write the caller's arrays in the
 // kernels: a launch or two and one synchronisation instead of four copies.
+// Arrays that are not aligned, or an output that overlaps an input, are copied.
 kpz_status kpz_mlp_predict(kpz_mlp* m, const float* x, uint32_t n, float* y) {
   if (!m || !x || !y) return KPZ_EINVAL;
   if (n == 0) return KPZ_OK;
   const float* xin = x;
   float* yout = y;
-  if (m->direct_host) {
+  const HostSpan in = {x, (size_t)n * kIn * 4};
+  const bool direct = m->direct_host && usable_in_place(&in, 1, HostSpan{y, (size_t)n * 4});
+  if (direct) {
     touch_pages(y, (size_t)n * 4);
   } else {
     kpz_status st = ensure_data(m, n);
@@ -654,7 +657,7 @@ kpz_status kpz_mlp_predict(kpz_mlp* m, const float* x, uint32_t n, float* y) {
       m->P, xin, nullptr, (int)n, 0.f, yout, nullptr, &m->host->err);
   count_launch();
   if (cudaGetLastError() != cudaSuccess ||
-      (!m->direct_host && cudaMemcpyAsync(y, m->y, (size_t)n * 4, cudaMemcpyDeviceToHost, m->stream) != cudaSuccess))
+      (!direct && cudaMemcpyAsync(y, m->y, (size_t)n * 4, cudaMemcpyDeviceToHost, m->stream) != cudaSuccess))
     return KPZ_ECUDA;
   return finish(m);
 }
@@ -665,7 +668,9 @@ kpz_status kpz_mlp_loss_grad(kpz_mlp* m, const float* x, const float* t, uint32_
   if (st) return st;
   const float *xin = x, *tin = t;
   float* gout = grad;
-  if (m->direct_host) {
+  const HostSpan in[2] = {{x, (size_t)n * kIn * 4}, {t, (size_t)n * 4}};
+  const bool direct = m->direct_host && usable_in_place(in, 2, HostSpan{grad, (size_t)kParams * 4});
+  if (direct) {
     if (grad) touch_pages(grad, kParams * 4);
   } else {
     if ((st = ensure_data(m, n)) != KPZ_OK) return st;
@@ -680,7 +685,7 @@ kpz_status kpz_mlp_loss_grad(kpz_mlp* m, const float* x, const float* t, uint32_
   reduce_kernel<<<kReduceBlocks, 256, 0, m->stream>>>(m->gpart, parts, gout, &m->host->sq);
   count_launch();
   if (cudaGetLastError() != cudaSuccess ||
-      (grad && !m->direct_host &&
+      (grad && !direct &&
        cudaMemcpyAsync(grad, m->grad, kParams * 4, cudaMemcpyDeviceToHost, m->stream) != cudaSuccess))
     return KPZ_ECUDA;
   st = finish(m);

@@ -37,3 +37,47 @@ def test_heights(eng, L, offset):
         assert load().kpz_heights(lat.handle, _ptr(out), absolute) == 0
         assert np.array_equal(out.reshape(L, L), st.heights(absolute=bool(absolute)))
     lat.close()
+
+
+# The network: unaligned arrays give the bits aligned ones do, and an output may
+# overlap an input.
+@pytest.fixture(scope="module")
+def net(eng):
+    from paper_1204_5072_gb300 import surrogate
+    mlp = surrogate.MLP(surrogate.init_params(5))
+    n = 9000
+    x = np.random.default_rng(5).standard_normal((n, 4)).astype(np.float32)
+    t = x[:, 0].copy()
+    yield mlp, n, x, t, mlp.predict(x), mlp.loss_grad(x, t)
+    mlp.close()
+
+
+@pytest.mark.parametrize("ox,ot,oy", [(1, 0, 0), (0, 2, 0), (0, 0, 3), (2, 6, 1), (4, 8, 12)])
+def test_network_arrays(net, ox, ot, oy):
+    import ctypes
+    mlp, n, x, t, y, (loss, grad) = net
+    ux, ut = at_offset(4 * n, np.float32, ox), at_offset(n, np.float32, ot)
+    ux[:], ut[:] = x.ravel(), t
+    out = at_offset(n, np.float32, oy)
+    assert load().kpz_mlp_predict(mlp._m, _ptr(ux), n, _ptr(out)) == 0
+    assert np.array_equal(out, y)
+    g, l = at_offset(len(grad), np.float32, oy), ctypes.c_float()
+    assert load().kpz_mlp_loss_grad(mlp._m, _ptr(ux), _ptr(ut), n, ctypes.byref(l), _ptr(g)) == 0
+    assert l.value == loss and np.array_equal(g, grad)
+    assert np.array_equal(mlp.predict(ux.reshape(n, 4)), y)   # numpy hands an unaligned view on as it is
+    assert np.array_equal(mlp.loss_grad(ux.reshape(n, 4), ut)[1], grad)
+
+
+@pytest.mark.parametrize("shift", [0, 1, 4000])
+def test_network_output_over_its_input(net, shift):
+    import ctypes
+    mlp, n, x, t, y, (loss, grad) = net
+    xs = x.ravel().copy()
+    assert load().kpz_mlp_predict(mlp._m, _ptr(xs), n, _ptr(xs[shift:])) == 0
+    assert np.array_equal(xs[shift:shift + n], y)
+    xs = x.ravel().copy()
+    assert load().kpz_mlp_loss_grad(mlp._m, _ptr(xs), _ptr(t), n, ctypes.byref(ctypes.c_float()), _ptr(xs[shift // 2:])) == 0
+    assert np.array_equal(xs[shift // 2:][:len(grad)], grad)
+    ts = np.concatenate([t, np.zeros(len(grad), np.float32)])
+    assert load().kpz_mlp_loss_grad(mlp._m, _ptr(x), _ptr(ts), n, ctypes.byref(ctypes.c_float()), _ptr(ts[shift:])) == 0
+    assert np.array_equal(ts[shift:][:len(grad)], grad)
