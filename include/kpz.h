@@ -21,7 +21,9 @@
  *     kpz_free and the library never frees it.
  *   - Work is queued on the context's stream (kpz_opts.stream, or the legacy
  *     default stream when NULL). Functions that return data to the host
- *     synchronise that stream; kpz_run does not.
+ *     synchronise that stream; kpz_run does not. The stream must live as long
+ *     as the context, except that kpz_free does not use it when the memory is
+ *     the caller's (dev_buf, decompositions 0 to 3).
  *   - A context is not thread-safe; distinct contexts are independent.
  *   - After KPZ_ECUDA the context is poisoned: every later call returns
  *     KPZ_ESTATE until kpz_free.

@@ -95,6 +95,7 @@ struct kpz_ctx {
   unsigned long long* h00 = nullptr;   // absolute height of site (0,0)
   uint32_t* ticket = nullptr;          // roughness: blocks that have finished (zero between launches)
   long long* sums = nullptr;           // pinned host slot: results of the roughness kernel
+  bool sums_pending = false;           // a kernel that writes sums may still be running
   uint32_t* hcar = nullptr;            // import: height of (0, j0) modulo 4
   uint32_t* queue = nullptr;           // sweep work queue (zero between launches)
   GridSync* sync = nullptr;            // persistent kernels: grid barrier and error flag
@@ -441,9 +442,11 @@ kpz_status kpz_roughness(kpz_ctx* ctx, kpz_rough* out) {
   if (st) return st;
   if (!out) return fail(ctx, KPZ_EINVAL, "null output");
   // The kernel leaves its results in pinned host memory: no copy to queue.
+  ctx->sums_pending = true;
   KPZ_CUDA(launch_roughness(ctx->lat, ctx->g, ctx->col0, RoughOut{ctx->ticket, ctx->sums, ctx->h00, &ctx->sync->err},
                             ctx->stream));
   KPZ_CUDA(cudaStreamSynchronize(ctx->stream));
+  ctx->sums_pending = false;
   const volatile long long* res = ctx->sums;
   const unsigned long long host[4] = {(unsigned long long)res[0], (unsigned long long)res[1],
                                       (unsigned long long)res[2], (unsigned long long)res[3]};
@@ -724,10 +727,8 @@ void kpz_free(kpz_ctx* ctx) {
     cudaStreamSynchronize(ctx->stream);
     cudaFree(ctx->rsu_scratch);
   }
-  if (ctx->sums) {
-    cudaStreamSynchronize(ctx->stream);
-    host_slot_free(ctx->sums);
-  }
+  if (ctx->sums_pending) cudaStreamSynchronize(ctx->stream);   // a roughness call that failed on the way
+  host_slot_free(ctx->sums);
   delete ctx;
 }
 
