@@ -6,10 +6,8 @@
 #include <cstring>
 #include <algorithm>
 #include <atomic>
-#include <mutex>
 #include <new>
 #include <string>
-#include <vector>
 
 #include "kpz.h"
 #include "kpz_host.h"
@@ -23,55 +21,6 @@ using namespace kpz;
 namespace kpz {
 static std::atomic<uint64_t> g_launches{0};
 void count_launch(uint64_t n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
-
-// Pinned slots of all contexts and networks of the process: one allocation (20
-// us) for up to 64 of them instead of one each.
-namespace {
-struct Slab {
-  char* base;
-  uint64_t used;   // bit i: slot i
-};
-std::mutex g_slab_mu;
-std::vector<Slab> g_slabs;
-}  // namespace
-
-void* host_slot() {
-  std::lock_guard<std::mutex> lock(g_slab_mu);
-  Slab* s = nullptr;
-  for (Slab& x : g_slabs)
-    if (~x.used) { s = &x; break; }
-  if (!s) {
-    void* p = nullptr;
-    if (cudaHostAlloc(&p, 64 * kHostSlot, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
-      cudaGetLastError();
-      return nullptr;
-    }
-    try {
-      g_slabs.push_back(Slab{(char*)p, 0u});
-    } catch (...) {
-      cudaFreeHost(p);
-      return nullptr;
-    }
-    s = &g_slabs.back();
-  }
-  const int i = __builtin_ctzll(~s->used);
-  s->used |= 1ull << i;
-  memset(s->base + i * kHostSlot, 0, kHostSlot);
-  return s->base + i * kHostSlot;
-}
-
-void host_slot_free(void* p) {
-  if (!p) return;
-  std::lock_guard<std::mutex> lock(g_slab_mu);
-  bool any = false;
-  for (Slab& x : g_slabs) {
-    if ((char*)p >= x.base && (char*)p < x.base + 64 * kHostSlot) x.used &= ~(1ull << (((char*)p - x.base) / kHostSlot));
-    any = any || x.used;
-  }
-  if (any) return;
-  for (Slab& x : g_slabs) cudaFreeHost(x.base);
-  g_slabs.clear();
-}
 }  // namespace kpz
 
 struct kpz_ctx {
@@ -94,8 +43,13 @@ struct kpz_ctx {
   uint64_t* t_dev = nullptr;           // sweep counter
   unsigned long long* h00 = nullptr;   // absolute height of site (0,0)
   uint32_t* ticket = nullptr;          // roughness: blocks that have finished (zero between launches)
-  long long* sums = nullptr;           // pinned host slot: results of the roughness kernel
-  bool sums_pending = false;           // a kernel that writes sums may still be running
+  // Results of the roughness kernel. Where the GPU reaches pageable memory it
+  // writes them here itself, elsewhere to device memory they are copied from. A
+  // sample of W^2 takes as long as with pinned memory (16.0 us at L = 256, 16.4
+  // at 1024), which costs 300 us to have and to give back and waits for the GPU.
+  alignas(64) long long result[8] = {};
+  long long* sums = nullptr;           // where the kernel puts them: result, or device memory
+  bool sums_pending = false;           // a kernel that writes result may still be running
   uint32_t* hcar = nullptr;            // import: height of (0, j0) modulo 4
   uint32_t* queue = nullptr;           // sweep work queue (zero between launches)
   GridSync* sync = nullptr;            // persistent kernels: grid barrier and error flag
@@ -138,7 +92,7 @@ Layout layout(uint32_t L) {
   Layout y{};
   const size_t lat_bytes = (size_t)L * L / 8;   // 1 bit per site
   y.lat = 0;
-  y.small = align_up(lat_bytes);                 // t, h00, hcar, queue, ticket; at +128 GridSync
+  y.small = align_up(lat_bytes);                 // t, h00, hcar, queue, ticket; at +64 sums, at +128 GridSync
   y.col0 = y.small + kAlign;
   y.io = y.col0 + align_up((size_t)L * 4);
   const size_t io_bytes = std::min(kIoMax, (size_t)L * L / 4);
@@ -342,17 +296,10 @@ kpz_status kpz_init(kpz_ctx** out, uint32_t L, double p, double q, uint64_t seed
     ctx->own_buf = true;
     ctx->buf_bytes = y.total;
   }
-  ctx->sums = (long long*)host_slot();
-  if (!ctx->sums) {
-    if (ctx->own_buf) cudaFree(ctx->buf);
-    delete ctx;
-    return KPZ_ENOMEM;
-  }
   if (ctx->decomposition == 4u) {   // per-sweep attempt buckets of the exact random-sequential sweep
     cudaError_t e = cudaMalloc(&ctx->rsu_scratch, rsu_scratch_bytes(L));
     if (e != cudaSuccess) {
       cudaGetLastError();
-      host_slot_free(ctx->sums);
       if (ctx->own_buf) cudaFree(ctx->buf);
       delete ctx;
       return KPZ_ENOMEM;
@@ -366,6 +313,7 @@ kpz_status kpz_init(kpz_ctx** out, uint32_t L, double p, double q, uint64_t seed
   ctx->ticket = (uint32_t*)(base + y.small + 56);
   ctx->hcar = (uint32_t*)(base + y.small + 40);
   ctx->queue = (uint32_t*)(base + y.small + 48);
+  ctx->sums = ctx->direct_host ? ctx->result : (long long*)(base + y.small + 64);
   ctx->sync = (GridSync*)(base + y.small + 128);
   ctx->col0 = (int32_t*)(base + y.col0);
   ctx->io = base + y.io;
@@ -441,13 +389,14 @@ kpz_status kpz_roughness(kpz_ctx* ctx, kpz_rough* out) {
   kpz_status st = enter(ctx);
   if (st) return st;
   if (!out) return fail(ctx, KPZ_EINVAL, "null output");
-  // The kernel leaves its results in pinned host memory: no copy to queue.
-  ctx->sums_pending = true;
+  ctx->sums_pending = ctx->direct_host;
   KPZ_CUDA(launch_roughness(ctx->lat, ctx->g, ctx->col0, RoughOut{ctx->ticket, ctx->sums, ctx->h00, &ctx->sync->err},
                             ctx->stream));
+  if (!ctx->direct_host)
+    KPZ_CUDA(cudaMemcpyAsync(ctx->result, ctx->sums, 5 * sizeof(long long), cudaMemcpyDeviceToHost, ctx->stream));
   KPZ_CUDA(cudaStreamSynchronize(ctx->stream));
   ctx->sums_pending = false;
-  const volatile long long* res = ctx->sums;
+  const volatile long long* res = ctx->result;
   const unsigned long long host[4] = {(unsigned long long)res[0], (unsigned long long)res[1],
                                       (unsigned long long)res[2], (unsigned long long)res[3]};
   ctx->unchecked = false;
@@ -728,7 +677,6 @@ void kpz_free(kpz_ctx* ctx) {
     cudaFree(ctx->rsu_scratch);
   }
   if (ctx->sums_pending) cudaStreamSynchronize(ctx->stream);   // a roughness call that failed on the way
-  host_slot_free(ctx->sums);
   delete ctx;
 }
 

@@ -38,14 +38,6 @@ inline void touch_pages(void* p, size_t bytes) {
   if (bytes) *(volatile char*)(base + bytes - 1) = 0;
 }
 
-// A 64-byte slot of pinned host memory every device reaches, zeroed; null if
-// there is none to be had. Slots come from 4 KiB slabs (kpz_api.cu), which are
-// given back when the last slot in use is; callers synchronise the work that
-// writes a slot before they return it.
-constexpr size_t kHostSlot = 64;
-void* host_slot();
-void host_slot_free(void* p);
-
 // Whether the current device reads and writes pageable host memory itself.
 inline bool reaches_pageable(int device) {
   int v = 0;

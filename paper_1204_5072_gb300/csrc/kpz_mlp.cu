@@ -506,8 +506,11 @@ struct kpz_mlp {
   // per-call buffers: data (x, t, y) for `cap` samples, partials of `pcap` blocks, a gradient
   float *x = nullptr, *t = nullptr, *y = nullptr, *gpart = nullptr, *grad = nullptr;
   size_t cap = 0, pcap = 0;
-  struct Host { int err; float sq; };
-  Host* host = nullptr;         // pinned slot: set when a tensor-core wait timed out; sum of squared errors
+  // Set when a tensor-core wait timed out; sum of squared errors. The kernels
+  // write them here where the GPU reaches pageable memory, else to device memory.
+  struct Out { int err; float sq; };
+  alignas(64) Out result = {};
+  Out* out = nullptr;
 };
 
 namespace {
@@ -516,16 +519,20 @@ void mlp_release(kpz_mlp* m) {
   float* ptrs[] = {m->theta, m->m, m->v, m->grad, m->x, m->t, m->y, m->gpart};
   for (float* p : ptrs) if (p) cudaFree(p);
   if (m->P) cudaFree(m->P);
-  host_slot_free(m->host);
+  if (m->out && m->out != &m->result) cudaFree(m->out);
 }
 
 // Synchronises the stream; KPZ_ETIMEOUT when a kernel's tensor-core wait ran
 // out (the flag is then cleared).
 kpz_status finish(kpz_mlp* m) {
+  if (m->out != &m->result &&
+      cudaMemcpyAsync(&m->result, m->out, sizeof(m->result), cudaMemcpyDeviceToHost, m->stream) != cudaSuccess)
+    return KPZ_ECUDA;
   if (cudaStreamSynchronize(m->stream) != cudaSuccess) return KPZ_ECUDA;
-  volatile kpz_mlp::Host* h = m->host;
+  volatile kpz_mlp::Out* h = &m->result;
   if (h->err) {
     h->err = 0;
+    if (m->out != &m->result) cudaMemsetAsync(&m->out->err, 0, sizeof(int), m->stream);
     return KPZ_ETIMEOUT;
   }
   return KPZ_OK;
@@ -572,7 +579,7 @@ kpz_status ensure_parts(kpz_mlp* m, size_t n) {
 int queue_grad(kpz_mlp* m, const float* x, const float* t, int n) {
   const int blocks = grad_blocks(m, (size_t)n);
   net_kernel<true><<<blocks, tc::kThreads, tc::kSmemGrad, m->stream>>>(m->P, x, t, n, 1.f / (float)n, nullptr, m->gpart,
-                                                                      &m->host->err);
+                                                                      &m->out->err);
   count_launch();
   return blocks;
 }
@@ -594,10 +601,12 @@ kpz_status kpz_mlp_create(kpz_mlp** out, const float* params, void* stream) {
   cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, m->device);
   m->sms = std::max(m->sms, 1);
   m->direct_host = reaches_pageable(m->device);
+  if (m->direct_host) m->out = &m->result;
   m->stream = (cudaStream_t)stream;
   if (cudaMalloc(&m->theta, kParams * 4) != cudaSuccess || cudaMalloc(&m->m, kParams * 4) != cudaSuccess ||
       cudaMalloc(&m->v, kParams * 4) != cudaSuccess || cudaMalloc(&m->grad, kParams * 4) != cudaSuccess ||
-      cudaMalloc(&m->P, kParams * 2) != cudaSuccess || !(m->host = (kpz_mlp::Host*)host_slot())) {
+      cudaMalloc(&m->P, kParams * 2) != cudaSuccess ||
+      (!m->direct_host && cudaMalloc(&m->out, sizeof(*m->out)) != cudaSuccess)) {
     cudaGetLastError();
     mlp_release(m);
     delete m;
@@ -609,7 +618,8 @@ kpz_status kpz_mlp_create(kpz_mlp** out, const float* params, void* stream) {
           cudaSuccess ||
       cudaMemcpyAsync(m->theta, params, kParams * 4, cudaMemcpyHostToDevice, m->stream) != cudaSuccess ||
       cudaMemsetAsync(m->m, 0, kParams * 4, m->stream) != cudaSuccess ||
-      cudaMemsetAsync(m->v, 0, kParams * 4, m->stream) != cudaSuccess) {
+      cudaMemsetAsync(m->v, 0, kParams * 4, m->stream) != cudaSuccess ||
+      (!m->direct_host && cudaMemsetAsync(m->out, 0, sizeof(*m->out), m->stream) != cudaSuccess)) {
     mlp_release(m);
     delete m;
     return KPZ_ECUDA;
@@ -654,7 +664,7 @@ kpz_status kpz_mlp_predict(kpz_mlp* m, const float* x, uint32_t n, float* y) {
     yout = m->y;
   }
   net_kernel<false><<<std::min(tiles_of(n), 2 * m->sms), tc::kThreads, tc::kSmemPredict, m->stream>>>(
-      m->P, xin, nullptr, (int)n, 0.f, yout, nullptr, &m->host->err);
+      m->P, xin, nullptr, (int)n, 0.f, yout, nullptr, &m->out->err);
   count_launch();
   if (cudaGetLastError() != cudaSuccess ||
       (!direct && cudaMemcpyAsync(y, m->y, (size_t)n * 4, cudaMemcpyDeviceToHost, m->stream) != cudaSuccess))
@@ -682,14 +692,14 @@ kpz_status kpz_mlp_loss_grad(kpz_mlp* m, const float* x, const float* t, uint32_
     gout = grad ? m->grad : nullptr;
   }
   const int parts = queue_grad(m, xin, tin, (int)n);
-  reduce_kernel<<<kReduceBlocks, 256, 0, m->stream>>>(m->gpart, parts, gout, &m->host->sq);
+  reduce_kernel<<<kReduceBlocks, 256, 0, m->stream>>>(m->gpart, parts, gout, &m->out->sq);
   count_launch();
   if (cudaGetLastError() != cudaSuccess ||
       (grad && !direct &&
        cudaMemcpyAsync(grad, m->grad, kParams * 4, cudaMemcpyDeviceToHost, m->stream) != cudaSuccess))
     return KPZ_ECUDA;
   st = finish(m);
-  if (loss) *loss = *(volatile float*)&m->host->sq / (float)n;
+  if (loss) *loss = *(volatile float*)&m->result.sq / (float)n;
   return st;
 }
 
@@ -712,18 +722,19 @@ kpz_status kpz_mlp_train(kpz_mlp* m, const float* x, const float* t, uint32_t n,
       cudaMemcpyAsync(m->t, tg.data(), total * 4, cudaMemcpyHostToDevice, m->stream) != cudaSuccess)
     return KPZ_ECUDA;
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-  m->host->sq = 0.f;
+  m->result.sq = 0.f;   // the loss of no step at all
+  if (m->out != &m->result && cudaMemsetAsync(&m->out->sq, 0, sizeof(float), m->stream) != cudaSuccess) return KPZ_ECUDA;
   for (uint32_t s = 0; s < steps; ++s) {
     ++m->step;
     const float c1 = 1.f - std::pow(b1, (float)m->step), c2 = 1.f - std::pow(b2, (float)m->step);
     const int parts = queue_grad(m, m->x + (size_t)s * batch * kIn, m->t + (size_t)s * batch, (int)batch);
-    adam_kernel<<<kReduceBlocks, 256, 0, m->stream>>>(m->gpart, parts, m->theta, m->m, m->v, m->P, &m->host->sq, lr, b1, b2,
+    adam_kernel<<<kReduceBlocks, 256, 0, m->stream>>>(m->gpart, parts, m->theta, m->m, m->v, m->P, &m->out->sq, lr, b1, b2,
                                                       c1, c2, eps);
     count_launch();
   }
   if (cudaGetLastError() != cudaSuccess) return KPZ_ECUDA;
   st = finish(m);
-  if (last_loss) *last_loss = *(volatile float*)&m->host->sq / (float)batch;
+  if (last_loss) *last_loss = *(volatile float*)&m->result.sq / (float)batch;
   return st;
 }
 

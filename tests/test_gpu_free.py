@@ -58,3 +58,15 @@ def test_stream_destroyed_before_free(env):
     again = eng.Lattice(L, device_buffer=buf)
     assert again.run(2).roughness()["w2"] == w2
     again.close()
+
+
+def test_neither_waits_for_other_streams(env):
+    # No other context is alive.
+    eng, torch, a, b, buf = env
+    lat = eng.Lattice(L, stream=a.cuda_stream, device_buffer=buf)
+    lat.run(2).roughness()
+    busy(torch, b)
+    took = seconds(lat.close)
+    took += seconds(lambda: eng.Lattice(L, stream=a.cuda_stream, device_buffer=buf).close())
+    waited = seconds(torch.cuda.synchronize)
+    assert took < 0.1 < waited
