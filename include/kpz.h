@@ -294,7 +294,8 @@ void kpz_batch_free(kpz_batch* b);
  * a call with the same inputs gives the same result. The 128 x 128 layers run
  * on the tcgen05 tensor cores with waits bounded in time: predict, loss_grad
  * and train return KPZ_ETIMEOUT if one ran out (the results are then
- * invalid; the handle stays usable), KPZ_ECUDA on a CUDA error.            */
+ * invalid; the handle stays usable), KPZ_ECUDA on a CUDA error. More than
+ * 2^31 - 32 samples in a pass are refused with KPZ_ENOMEM.                  */
 typedef struct kpz_mlp kpz_mlp;
 /* Upload initial parameters (caller-chosen initialisation); stream may be NULL. */
 kpz_status kpz_mlp_create(kpz_mlp** out, const float* params, void* stream);

@@ -559,6 +559,10 @@ kpz_status ensure_data(kpz_mlp* m, size_t n) {
 int tiles_of(size_t n) { return (int)((n + tc::kS - 1) / tc::kS); }
 int grad_blocks(const kpz_mlp* m, size_t n) { return std::min(tiles_of(n), m->sms); }
 
+// The kernels count samples in 32 bits, a tile beyond the last one included; a
+// call for more is refused before any of its arrays is touched.
+constexpr uint32_t kMaxSamples = 0x7FFFFFFFu - (uint32_t)(tc::kS - 1);
+
 // Partials for gradients over n samples.
 kpz_status ensure_parts(kpz_mlp* m, size_t n) {
   const size_t b = (size_t)grad_blocks(m, n);
@@ -650,6 +654,7 @@ kpz_status kpz_mlp_params(kpz_mlp* m, float* params) {
 kpz_status kpz_mlp_predict(kpz_mlp* m, const float* x, uint32_t n, float* y) {
   if (!m || !x || !y) return KPZ_EINVAL;
   if (n == 0) return KPZ_OK;
+  if (n > kMaxSamples) return KPZ_ENOMEM;
   const float* xin = x;
   float* yout = y;
   const HostSpan in = {x, (size_t)n * kIn * 4};
@@ -674,6 +679,7 @@ kpz_status kpz_mlp_predict(kpz_mlp* m, const float* x, uint32_t n, float* y) {
 
 kpz_status kpz_mlp_loss_grad(kpz_mlp* m, const float* x, const float* t, uint32_t n, float* loss, float* grad) {
   if (!m || !x || !t || n == 0) return KPZ_EINVAL;
+  if (n > kMaxSamples) return KPZ_ENOMEM;
   kpz_status st = ensure_parts(m, n);
   if (st) return st;
   const float *xin = x, *tin = t;
@@ -706,6 +712,7 @@ kpz_status kpz_mlp_loss_grad(kpz_mlp* m, const float* x, const float* t, uint32_
 kpz_status kpz_mlp_train(kpz_mlp* m, const float* x, const float* t, uint32_t n, const uint32_t* order,
                          uint32_t steps, uint32_t batch, float lr, float* last_loss) {
   if (!m || !x || !t || !order || n == 0 || batch == 0 || !(lr > 0.f)) return KPZ_EINVAL;
+  if (batch > kMaxSamples) return KPZ_ENOMEM;
   // Upload the minibatches already gathered in the order the caller chose:
   // step s uses samples order[s*batch .. s*batch + batch - 1] (indices < n).
   const size_t total = (size_t)steps * batch;

@@ -81,3 +81,16 @@ def test_network_output_over_its_input(net, shift):
     ts = np.concatenate([t, np.zeros(len(grad), np.float32)])
     assert load().kpz_mlp_loss_grad(mlp._m, _ptr(x), _ptr(ts), n, ctypes.byref(ctypes.c_float()), _ptr(ts[shift:])) == 0
     assert np.array_equal(ts[shift:][:len(grad)], grad)
+
+
+@pytest.mark.parametrize("n", [2 ** 31 - 31, 2 ** 31, 2 ** 32 - 1])
+def test_network_refuses_more_samples_than_it_counts(net, n):
+    """Answered from the count alone: the arrays are far smaller and stay as they are."""
+    import ctypes
+    from paper_1204_5072_gb300._lib import KPZ_ENOMEM
+    m, lib, l = net[0]._m, load(), ctypes.c_float(-1.0)
+    x, t, order = np.full(64, 7, np.float32), np.full(16, 7, np.float32), np.zeros(16, np.uint32)
+    assert lib.kpz_mlp_predict(m, _ptr(x), n, _ptr(t)) == KPZ_ENOMEM
+    assert lib.kpz_mlp_loss_grad(m, _ptr(x), _ptr(t), n, ctypes.byref(l), None) == KPZ_ENOMEM
+    assert lib.kpz_mlp_train(m, _ptr(x), _ptr(t), 16, _ptr(order), 1, n, ctypes.c_float(1e-3), ctypes.byref(l)) == KPZ_ENOMEM
+    assert l.value == -1.0 and (x == 7).all() and (t == 7).all()
