@@ -108,7 +108,7 @@ K_ALG_ALU_GENERAL = 30 / 32 + 20 / 64 + 1 / 32 + C_CAND * 2 * (20 / 128 + 2 / 32
 
 # Files the sweep kernel is compiled from (their hash ties a profile to the source).
 SWEEP_SOURCES = ("kpz_sweep.cu", "kpz_run.cuh", "kpz_rounds.cuh", "kpz_tilemem.cuh", "kpz_common.cuh",
-                 "kpz_internal.h")
+                 "kpz_internal.h", "kpz_gridsync.cuh")
 
 
 def sweep_source_sha():
