@@ -71,8 +71,7 @@ __device__ __forceinline__ bool rows_done(uint32_t* done, uint32_t i, uint32_t n
   }
   const uint64_t t0 = gridsync::now_ns();
   for (uint32_t it = 1; !ready(); ++it) {
-    if ((it & 63u) == 0u &&
-        __any_sync(kFull, gridsync::now_ns() - t0 > gridsync::kWaitNs || *(volatile uint32_t*)&sync->err)) {
+    if ((it & 63u) == 0u && __any_sync(kFull, gridsync::gave_up(sync, t0))) {
       if (lane == 0u) atomicExch(&sync->err, 1u);
       return false;
     }
