@@ -42,3 +42,20 @@ def test_grid(eng, L, p, q, decomposition):
     (256, 1.0, 0.0, 1), (512, 0.95, 0.05, 1), (1024, 0.6, 0.3, 1), (1024, 1.0, 0.0, 1), (2048, 1.0, 0.0, 1)])
 def test_cluster(eng, L, p, q, decomposition):
     same_after(eng, L, p, q, decomposition, (4000, 1501))
+
+
+# The one shape in which tile sets run on seven tile warps a block that draw
+# their own numbers; from an odd start parity and a later sweep count.
+@pytest.mark.parametrize("p,q", [(1.0, 0.0), (0.95, 0.05), (0.5, 1.0)])
+def test_tile_sets_without_drawing_warps(eng, p, q):
+    L = 8192
+    lat = eng.Lattice(L, p, q, seed=21, sample=4, decomposition=1)
+    ref = eng.Lattice(L, p, q, seed=21, sample=4, decomposition=1, run=2, warps_per_cta=4)
+    start = ref.run(1).slopes()
+    for x in (lat, ref):
+        x.set_slopes(start, h00=-5, t=9)
+    for n in (1, 3, 40):
+        assert lat.run(n).roughness() == ref.run(n).roughness()
+        assert np.array_equal(lat.slopes(), ref.slopes())
+    lat.close()
+    ref.close()
