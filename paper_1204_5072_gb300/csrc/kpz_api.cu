@@ -421,10 +421,10 @@ kpz_status kpz_heights(kpz_ctx* ctx, int64_t* host_out, int absolute) {
   if (!host_out) return fail(ctx, KPZ_EINVAL, "null output");
   const uint32_t L = ctx->g.L;
   KPZ_CUDA(launch_col0(ctx->lat, ctx->g, ctx->col0, ctx->stream));
-  touch_pages(host_out, (size_t)L * L * 8);
   // The kernel stores to the caller's buffer itself, 16 bytes at a time; an
   // int64 array may start at any multiple of 8, and such a one is copied to.
   if (ctx->direct_host && ((uintptr_t)host_out & 15u) == 0) {
+    touch_pages(host_out, (size_t)L * L * 8);
     KPZ_CUDA(launch_heights(ctx->lat, ctx->g, ctx->col0, 0, L, absolute ? ctx->h00 : nullptr, host_out, ctx->stream));
     KPZ_CUDA(cudaStreamSynchronize(ctx->stream));
     return settle(ctx);
@@ -460,7 +460,6 @@ kpz_status kpz_slopes(kpz_ctx* ctx, uint32_t* host_out) {
   size_t half = 0;
   const uint32_t band = io_band_rows(ctx, row_bytes, &half);
   char* buf[2] = {(char*)ctx->io, (char*)ctx->io + half};
-  touch_pages(host_out, (size_t)L * row_bytes);
   KPZ_CUDA(io_prepare(ctx));
   uint32_t b = 0;
   for (uint32_t j0 = 0; j0 < L; j0 += band, ++b) {

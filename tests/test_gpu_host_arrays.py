@@ -94,3 +94,25 @@ def test_network_refuses_more_samples_than_it_counts(net, n):
     assert lib.kpz_mlp_loss_grad(m, _ptr(x), _ptr(t), n, ctypes.byref(l), None) == KPZ_ENOMEM
     assert lib.kpz_mlp_train(m, _ptr(x), _ptr(t), 16, _ptr(order), 1, n, ctypes.c_float(1e-3), ctypes.byref(l)) == KPZ_ENOMEM
     assert l.value == -1.0 and (x == 7).all() and (t == 7).all()
+
+
+def test_slopes_into_a_used_array_cost_a_copy(eng):
+    """An export into an array whose pages exist takes about as long as the copy
+    it is (1.3 times at this size; touching every page first made it 2.4)."""
+    import time
+    import torch
+    L = 16384
+    lat = eng.Lattice(L)
+    out = np.zeros(L * L // 16, np.uint32)
+    host, dev = torch.from_numpy(out.view(np.int32)), torch.zeros(L * L // 16, dtype=torch.int32, device="cuda")
+
+    def best(f):
+        times = []
+        for _ in range(30):
+            t = time.perf_counter()
+            f()
+            times.append(time.perf_counter() - t)
+        return min(times)
+
+    assert best(lambda: lat.slopes_into(out)) < 1.8 * best(lambda: host.copy_(dev))
+    lat.close()
