@@ -25,8 +25,9 @@
  *     as the context, except that kpz_free does not use it when the memory is
  *     the caller's (dev_buf, decompositions 0 to 3).
  *   - A context is not thread-safe; distinct contexts are independent.
- *   - After KPZ_ECUDA the context is poisoned: every later call returns
- *     KPZ_ESTATE until kpz_free.
+ *   - After KPZ_ECUDA or KPZ_ETIMEOUT the context is poisoned: every later
+ *     call returns KPZ_ESTATE until kpz_free. (A kpz_batch or kpz_mlp stays
+ *     usable after KPZ_ETIMEOUT.)
  *
  * Packed exchange format (kpz_slopes / kpz_set_slopes): row j (y) occupies
  * L/16 consecutive 32-bit words; site i (x) sits in word j*(L/16) + i/16 at bit
@@ -68,7 +69,8 @@ typedef struct {
                              trajectories; 128 x 256 needs L >= 256               */
     uint32_t run;         /* tiles per work item: the resident warps take runs of
                              `run` tiles of one tile row from a queue (power of two
-                             <= L/128; 0 = as many as leave 8192 runs, at least 1,
+                             <= L/128; 0 = as many as leave 4096 runs where sweeps
+                             are chained in a launch, 8192 elsewhere, at least 1,
                              at most L/4096); execution only, it does not change
                              the result                                            */
     uint32_t warps_per_cta; /* 1..8; 0 = 4 for 128-row tiles from L = 65536, else 8;

@@ -365,9 +365,11 @@ __global__ void __launch_bounds__(kBandThreads, kBandBlocks) roughness_kernel(co
   }
   __syncthreads();
   if (!last) return;
-  // Chain the bands: thread t takes bands [t per, (t + 1) per), at most 32; a
-  // band's sum of squares is below 2^57, so a thread's fits 64 bits, and the
-  // block adds the threads' 32-bit halves.
+  // Chain the bands: thread t takes bands [t per, (t + 1) per), at most 32. A
+  // height is at most the distance from (0,0) along the axes, both ways round,
+  // so at L = 2^18 a band's sum of squares is at most 7/3 2^57 (a tent in each
+  // direction, at the crest) and a thread's 32 bands stay below 2^64, unsigned;
+  // the block adds the threads' 32-bit halves.
   __threadfence();
   __shared__ long long scan[kBandThreads];
   const uint32_t per = (nb + kBandThreads - 1u) / kBandThreads, k0 = min(nb, threadIdx.x * per), k1 = min(nb, k0 + per);
