@@ -29,7 +29,7 @@
 // for memory four times). Counting, prefix sums, scattering and sorting
 // into buckets, rounds that looked up five buckets a site, and the host
 // polling every eight rounds took 466 us a sweep at L = 1024 and 6.3 ms at
-// L = 4096; this takes 154 us (320 with each thread doing its own four) and 2.5 ms.
+// L = 4096; this takes 154 us (320 with each thread doing its own four) and 2.4 ms.
 #include <algorithm>
 
 #include "kpz_rsu.h"
