@@ -9,8 +9,7 @@
 
 namespace kpz {
 
-// Writes to every page of a caller's buffer that a kernel is about to fill
-// (copies do not need it: kpz_slopes into a used array took 1.8 times as long).
+// Writes to every page of a caller's buffer that a kernel is about to fill.
 // Pages of a fresh allocation exist only once touched, and a GPU that is the
 // first to touch them waits some 55 us for every 64 KiB it stores (heights at L
 // = 2048 took 28 ms into a fresh array, 1.2 ms into a touched one). One write to
